@@ -74,17 +74,89 @@ __global__ void k_hop_grad(const double2 *__restrict__ chi, const double2 *__res
     GA[(size_t)k * g.V + site] = G;
 }
 
-// step 2: G_A = VJP of the projection (off-axis canonical fields, in place)
-__global__ void k_project_vjp(const M3<double2> *__restrict__ A, M3<double2> *GA, Geom g) {
-    const int site = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y;
-    if (site >= g.V) return;
-    const int k = canon_k(j);
-    if (off_class(k) < 2) return;
-    const M3<double2> a = A[(size_t)k * g.V + site];
-    const M3<double2> G = GA[(size_t)k * g.V + site];
+// traceless anti-hermitian part
+BRI_D M3<double2> ta_part(const M3<double2> &B) {
+    M3<double2> P;
+    const double tr = (B.e[0].y + B.e[4].y + B.e[8].y) * (1.0 / 3.0);
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        P.e[4 * i] = make_double2(0.0, B.e[4 * i].y - tr);
+#pragma unroll
+        for (int j = i + 1; j < 3; j++) {
+            const double2 q = cscale(csub(B.e[3 * i + j], cconj(B.e[3 * j + i])), 0.5);
+            P.e[3 * i + j] = q;
+            P.e[3 * j + i] = make_double2(-q.x, q.y);
+        }
+    }
+    return P;
+}
+
+// -Y L^{-1}(TA(G^dagger Y)) from the FP32 basis of the projection by
+// refinement: L is applied in FP64 (L(X) = TA(H X)) and inverted in FP32, an
+// error falls by the FP32 accuracy per step.  Two solves' worth of FP64 matrix
+// products where the closed form below takes eight after an FP64
+// eigendecomposition.  False: take the closed form.
+BRI_D bool project_vjp_fast(const M3<double2> &A, const M3<double2> &G, M3<double2> &out) {
+    M3<double2> Y, H;
+    ProjectionSeed sd;
+    if (!project_fast(A, Y, sd)) return false;
+    M3<double2> P = ta_part(m3_mul(m3_dag(G), Y));
+    {
+        const M3<double2> B = m3_mul(m3_dag(A), Y);
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+#pragma unroll
+            for (int j = 0; j < 3; j++) H.e[3 * i + j] = cscale(cadd(B.e[3 * i + j], cconj(B.e[3 * j + i])), 0.5);
+    }
+    // the right-hand side scaled to about 1 for FP32
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < 9; i++)
+        m = max(m, max((unsigned)__double2hiint(P.e[i].x) & 0x7fffffffu, (unsigned)__double2hiint(P.e[i].y) & 0x7fffffffu));
+    const int e = (int)(m >> 20) - 1023;
+    if (e > 900 || (m != 0 && e < -900)) return false;
+    const double up = __hiloint2double((1023 + e) << 20, 0), dn = __hiloint2double((1023 - e) << 20, 0);
+    M3<double2> Q = m3_zero<double2>();
+    if (m != 0) {
+#pragma unroll
+        for (int i = 0; i < 9; i++) P.e[i] = cscale(P.e[i], dn);
+        float last = 0.f, size = 0.f;
+        bool done = false;
+#pragma unroll 1
+        for (int it = 0; it < 6 && !done; it++) {
+            M3<float2> R;
+#pragma unroll
+            for (int i = 0; i < 9; i++) R.e[i] = to_f32(P.e[i]);
+            R = seed_solve(sd, R);
+            const M3<double2> D = su3_algebra_f64(R);
+            float w = 0.f;
+#pragma unroll
+            for (int i = 0; i < 9; i++) {
+                Q.e[i] = cadd(Q.e[i], D.e[i]);
+                w = fmaxf(w, fmaxf(fabsf(R.e[i].x), fabsf(R.e[i].y)));
+            }
+            if (it == 0) size = w;
+            // the next step would change Q by about w times this step's contraction
+            done = w == 0.f || (it > 0 && w * fmaxf(w / last, 1e-7f) < 1e-17f * size);
+            last = w;
+            if (done) break;
+            const M3<double2> L = ta_part(m3_mul(H, D));
+#pragma unroll
+            for (int i = 0; i < 9; i++) P.e[i] = csub(P.e[i], L.e[i]);
+        }
+        if (!done) return false;
+    }
+    out = m3_mul(Y, Q);
+#pragma unroll
+    for (int i = 0; i < 9; i++) out.e[i] = cscale(out.e[i], -up);
+    return true;
+}
+
+// the closed form, in FP64 throughout
+static __device__ __noinline__ void project_vjp_general(const M3<double2> &a, const M3<double2> &G, M3<double2> &out) {
     ProjectionParts pp;
-    M3<double2> Y = project_su3(a, &pp);
+    M3<double2> Y;
+    project_su3_general(a, Y, &pp);
     // P = TA(G^dagger Y) in the basis V: P' = V^dagger TA(G^dagger Y) V
     M3<double2> B = m3_mul(m3_dag(G), Y);
     M3<double2> Vm, Vd;
@@ -110,8 +182,21 @@ __global__ void k_project_vjp(const M3<double2> *__restrict__ A, M3<double2> *GA
     const double m = -sp / sh;
     for (int i = 0; i < 3; i++) Q.e[4 * i] = make_double2(0.0, (p[i] + m) / h[i]);
     M3<double2> Qv = m3_mul(Vm, m3_mul(Q, Vd));
-    M3<double2> out = m3_mul(Y, Qv);
+    out = m3_mul(Y, Qv);
     for (int i = 0; i < 9; i++) out.e[i] = cscale(out.e[i], -1.0);
+}
+
+// step 2: G_A = VJP of the projection (off-axis canonical fields, in place)
+__global__ void k_project_vjp(const M3<double2> *__restrict__ A, M3<double2> *GA, Geom g) {
+    const int site = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.y;
+    if (site >= g.V) return;
+    const int k = canon_k(j);
+    if (off_class(k) < 2) return;
+    const M3<double2> a = A[(size_t)k * g.V + site];
+    const M3<double2> G = GA[(size_t)k * g.V + site];
+    M3<double2> out;
+    if (!project_vjp_fast(a, G, out)) project_vjp_general(a, G, out);
     GA[(size_t)k * g.V + site] = out;
 }
 

@@ -88,3 +88,48 @@ def test_empty_projection_batch(gpu):
     op = Brillouin((3, 3, 3, 3), AP)
     A = torch.zeros((0, 3, 3), dtype=torch.complex128, device=gpu)
     assert op.project_su3(A).shape == (0, 3, 3)
+
+
+@pytest.mark.parametrize("what", ["smooth", "rough", "haar", "gauss", "tiny", "huge", "identity", "near singular", "det phase"])
+def test_projection_seeds(gpu, what):
+    """Matrices that the FP32-seeded projection takes and ones that it hands to
+    the general form (any scale, either branch, nearly singular), mixed in one
+    launch: special unitary, stationary (the traceless anti-hermitian part of
+    A^dagger Y vanishes) and no worse than the oracle's maximum.  Bounds: a few
+    roundings of 3x3 products, 16 2^-52, relative to |A| for the last two."""
+    rng = np.random.default_rng(77)
+    n = 400
+
+    def near(eps):
+        return synth.random_su3_links((n, 1, 1, 1), eps, int(rng.integers(1 << 30)))[:, 0]
+
+    A = sum(near(0.5) for _ in range(4)) / 4
+    if what == "rough":
+        A = sum(near(2.0) for _ in range(4)) / 4
+    elif what == "haar":
+        A = sum(synth.random_su3(n, s) for s in range(3))
+    elif what == "gauss":
+        A = rng.standard_normal((n, 3, 3)) + 1j * rng.standard_normal((n, 3, 3))
+    elif what == "tiny":
+        A = A * 1e-40
+    elif what == "huge":
+        A = A * 1e40
+    elif what == "identity":
+        A = A * 0 + np.eye(3)
+    elif what == "near singular":
+        A[:, 2] = A[:, 1] + 1e-7 * A[:, 2]
+    elif what == "det phase":
+        A = A * np.exp(1j * np.linspace(0, 2 * np.pi, n))[:, None, None]  # through branch A, its edge and branch B
+    op = Brillouin((3, 3, 3, 3), (1, 1, 1, 1))
+    Y = op.project_su3(torch.as_tensor(np.ascontiguousarray(A), device=gpu)).cpu().numpy()
+    eps = 16 * 2.0 ** -52
+    size = np.abs(A).max(axis=(1, 2))
+    assert np.abs(Y.conj().transpose(0, 2, 1) @ Y - np.eye(3)).max() <= eps
+    assert np.abs(np.linalg.det(Y) - 1).max() <= eps
+    B = A.conj().transpose(0, 2, 1) @ Y
+    T = 0.5 * (B - B.conj().transpose(0, 2, 1))
+    T -= np.eye(3) * (np.trace(T, axis1=1, axis2=2) / 3)[:, None, None]
+    assert (np.abs(T).max(axis=(1, 2)) <= eps * size).all()
+    for i in range(0, n, 40):
+        best = np.trace(A[i].conj().T @ oracle.project_su3(A[i])).real
+        assert np.trace(B[i]).real >= best - eps * size[i]
