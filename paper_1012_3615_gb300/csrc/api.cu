@@ -121,6 +121,9 @@ bri_status bri_destroy(bri_ctx *ctx) {
     cudaFree(ctx->tc_f);
     cudaFree(ctx->U);
     cudaFree(ctx->hops64);
+    cudaFree(ctx->hopsfx);
+    cudaFree(ctx->fxinfo);
+    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
     cudaFreeHost(ctx->werr_h);
     for (LinkStore *st : {&ctx->f32, &ctx->f16, &ctx->p32, &ctx->p16}) {
         cudaFree(st->a);

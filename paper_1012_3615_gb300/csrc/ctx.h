@@ -26,6 +26,10 @@ struct bri_ctx {
     double2 *U = nullptr;       // copy of the links, [V][4][9]
     double2 *hops64 = nullptr;  // FP64 hops, [40][9][V]
     bool have64 = false;
+    int4 *hopsfx = nullptr;      // fixed-point copy of hops64 (dslash_fx.cu), [40][9][V]; null without memory for it
+    unsigned *fxinfo = nullptr;  // its scale and validity (device)
+    bool have_fx = false, fx_tried = false;
+    cudaMemPool_t pool = nullptr;  // stream-ordered work space of the calls, released by bri_destroy
     LinkStore f32, f16;
     LinkStore p32, p16;  // site-pair interleaved copies (full / 2-row, even t extent)
     SolverWork *work = nullptr;
@@ -106,7 +110,12 @@ bri_status bri_dslash_tc(bri_ctx *ctx, void *out, const void *in, int nrhs, doub
 bri_status bri_tc_reserve(bri_ctx *ctx, int nrhs, int cap);
 // dslash with an explicit launch shape; skip[r] != 0 skips right-hand side r
 bri_status bri_dslash_raw(bri_ctx *ctx, void *out, const void *in, int nrhs, double m0, int mode, bri_prec prec,
-                          const int *skip, int threads, cudaStream_t s);
+                          const int *skip, int threads, cudaStream_t s, void *work = nullptr);
+// FP64 apply in fixed point (dslash_fx.cu)
+bri_status bri_fx_store_impl(bri_ctx *ctx, cudaStream_t s);
+size_t bri_fx_work_bytes(bri_ctx *ctx, int nrhs);
+bri_status bri_dslash_fx(bri_ctx *ctx, const bri::Geom &g, void *out, const void *in, int nrhs, double m0, int mode,
+                         const int *skip, void *work, int *ndone, cudaStream_t s);
 int bri_dslash_threads(bri_ctx *ctx, bri_prec prec, int nrhs);
 std::string bri_tune_key(bri_ctx *ctx, bri_prec prec, int nrhs);
 bri_status bri_export_hops_impl(bri_ctx *ctx, double2 *out, cudaStream_t s);

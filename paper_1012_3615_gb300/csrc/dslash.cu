@@ -57,11 +57,11 @@ int bri_dslash_threads(bri_ctx *ctx, bri_prec prec, int nrhs) {
 }
 
 static bri_status dslash_geom(bri_ctx *ctx, const Geom &g, void *out, const void *in, int nrhs, double m0, int mode,
-                              bri_prec prec, const int *skip, int threads, cudaStream_t s);
+                              bri_prec prec, const int *skip, int threads, cudaStream_t s, void *work = nullptr);
 
 bri_status bri_dslash_raw(bri_ctx *ctx, void *out, const void *in, int nrhs, double m0, int mode, bri_prec prec,
-                          const int *skip, int threads, cudaStream_t s) {
-    return dslash_geom(ctx, ctx->g, out, in, nrhs, m0, mode, prec, skip, threads, s);
+                          const int *skip, int threads, cudaStream_t s, void *work) {
+    return dslash_geom(ctx, ctx->g, out, in, nrhs, m0, mode, prec, skip, threads, s, work);
 }
 
 // only sites [s0, s1) of out are written (the plain kernels; the tiled and
@@ -77,7 +77,7 @@ bri_status bri_dslash_range(bri_ctx *ctx, void *out, const void *in, int nrhs, d
 }
 
 static bri_status dslash_geom(bri_ctx *ctx, const Geom &g, void *out, const void *in, int nrhs, double m0, int mode,
-                              bri_prec prec, const int *skip, int threads, cudaStream_t s) {
+                              bri_prec prec, const int *skip, int threads, cudaStream_t s, void *work) {
     if (ctx->werr_h && *(volatile int *)ctx->werr_h) {
         *(volatile int *)ctx->werr_h = 0;
         return bri_fail(ctx, BRI_ETIMEOUT, "a bounded wait of an earlier apply gave up; its output is invalid");
@@ -85,6 +85,16 @@ static bri_status dslash_geom(bri_ctx *ctx, const Geom &g, void *out, const void
     const double diag = m0 + g.lamd[0];
     if (prec == BRI_F64) {
         if (!ctx->have64) return bri_fail(ctx, BRI_ESTATE, "FP64 hopping fields not built");
+        if (ctx->have_fx) {
+            int done = 0;
+            BRI_RETURN_IF(bri_dslash_fx(ctx, g, out, in, nrhs, m0, mode, skip, work, &done, s));
+            if (done == nrhs) return BRI_OK;
+            const size_t field = (size_t)done * g.V * 12;
+            out = (double2 *)out + field;
+            in = (const double2 *)in + field;
+            nrhs -= done;
+            if (skip) skip += done;
+        }
         LinkF64 ll{ctx->hops64, g.V};
         dslash_launch(mode, ll, in, out, nrhs, g, diag, skip, threads, s);
     } else {

@@ -1,0 +1,625 @@
+// FP64 stencil apply on the integer pipe.
+//
+// GB300 runs 2 FP64 FMAs per clock and SM, but 32 integer multiply-adds
+// 32 x 32 + 64 -> 64 bits, so the colour products, 11,520 of the 17,016 FP64
+// operations of a site, are taken in fixed point and exact integer sums:
+//
+//   link entries  w  = fw 2^(we - 62),    fw = wh 2^32 + wl, |wh| <= 2^30
+//   spinors       p  = fp 2^(e(y) - 60),  fp = ph 2^32 + pl, |ph| <= 2^28,
+//                 e(y) the exponent of the largest component of site y
+//   products      w p = wh ph 2^(we + e - 58) + (wh pl + wl ph) 2^(we + e - 90)
+//
+// (three multiply-adds a product; wl pl is below 2^-60 of the largest product
+// and dropped).  One 64-bit accumulator holds the six high products of a colour
+// row exactly, another the twelve cross products: rows and columns of a link
+// have norm <= 2^we, so |sum wh pl| <= sqrt(6) 2^61, |sum wl ph| <= 6 2^59,
+// together 7.9 2^60 < 2^63.  The row is rounded to the unit 2^(we + X_n - 58)
+// of its hop class n, X_n = the largest e(y) of the class's neighbours + h_n,
+// and the rows are summed as 64-bit integers: once with the class weight
+// lambda and once through gamma_d (entries +-1, +-i: additions only).  A
+// class sum holds at most 8, 48, 96, 64 rows (hops x directions of gamma_d) of
+// sqrt(6) 2^58: h_n = 0, 2, 3, 3.  Per class, the sums are converted and
+// weighted in FP64.  Every row is thus known to 2^-55 of its class's largest
+// neighbour and the sums over hops are exact, in any order, where FP64 rounds
+// each of ~480 partial sums: against quad precision 7.6e-17 relative (FP64 loop:
+// 1.6e-16) for Gaussian spinors, 8e-17 (1.6e-16) for a field that falls by e^-2
+// a step in every direction.
+//
+// Measured: 16^3x32 0.887 ms (FP64 kernel 4.12), 8^4 62 us (629), 32^4 6.7 ms
+// (31.2).  Bound by the integer multiply-adds (4 clocks a warp) and by fixed
+// latencies at 12 warps per SM.
+//
+// A site that meets an infinity, a NaN or an exponent outside the range of
+// FP64 scales takes the FP64 loop (fx_slow), as every site does when the links
+// hold such an entry.
+#include <algorithm>
+#include <string>
+
+#include "dslash_kernel.cuh"
+
+using namespace bri;
+
+// canonical field list of the operator in class order (sums are kept per class)
+struct FxOrder {
+    unsigned char t[NCANON];    // index into Geom::hop
+    unsigned char cls[NCANON];  // its class n
+};
+
+namespace {
+
+constexpr int FX_BAD = 1 << 20;     // block exponent of a site with an infinity or a NaN
+constexpr int FX_ZERO = -(1 << 20);  // ... of a site that is zero
+constexpr int FX_WB = 62, FX_PB = 60;  // fraction bits of links and spinors
+constexpr int FX_AB = FX_WB + FX_PB - 64;  // of the row sums
+// head room h_n of the class sums
+BRI_D int fx_head(int n) { return n == 1 ? 0 : n == 2 ? 2 : 3; }
+
+// v 2^sh rounded to an integer (|v| 2^sh < 2^63), by shifts: conversions run on
+// the FP64 pipe
+BRI_D long long fx_int(double v, int sh) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)(bits >> 52) & 0x7ff;
+    const unsigned long long m = (bits & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+    const int s = max(e, 1) - 1075 + sh, r = min(-s, 63);
+    const long long f = (long long)(s >= 0 ? m << s : (m + ((1ull << r) >> 1)) >> r);
+    return (long long)bits < 0 ? -f : f;
+}
+BRI_D int4 fx_split(double re, double im, int sh) {
+    // the low word is never INT_MIN, so that limbs can be negated
+    const long long a = fx_int(re, sh), b = fx_int(im, sh);
+    int4 v;
+    v.y = (int)a;
+    v.x = (int)((a - v.y) >> 32);
+    v.w = (int)b;
+    v.z = (int)((b - v.w) >> 32);
+    if (v.y == (int)0x80000000) v.y++;
+    if (v.w == (int)0x80000000) v.w++;
+    return v;
+}
+BRI_D unsigned abs_hi(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+
+// largest |row|^2, |column|^2 of a field matrix, as the high word of a double
+// (NaN and infinities come out largest)
+BRI_D unsigned norm_hi(const double2 w[9]) {
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        m = max(m, abs_hi(cnorm2(w[3 * i]) + cnorm2(w[3 * i + 1]) + cnorm2(w[3 * i + 2])));
+        m = max(m, abs_hi(cnorm2(w[i]) + cnorm2(w[3 + i]) + cnorm2(w[6 + i])));
+    }
+    return m;
+}
+// info[0]: the largest of the one-hop fields, which are the links as given (the
+// other fields are unitary); info[1]: 1 if a field matrix does not fit
+__global__ void k_fx_max(const double2 *__restrict__ h, int V, unsigned *info) {
+    constexpr int jf[4] = {0, 2, 8, 26};  // canonical fields of +x, +y, +z, +t
+    const int site = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned m = 0;
+    if (site < V) {
+        double2 w[9];
+        const int j = blockIdx.y == 0 ? jf[0] : blockIdx.y == 1 ? jf[1] : blockIdx.y == 2 ? jf[2] : jf[3];
+#pragma unroll
+        for (int e = 0; e < 9; e++) w[e] = h[((size_t)j * 9 + e) * V + site];
+        m = norm_hi(w);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(info, m);
+}
+constexpr unsigned FX_ONE = 0x3ff00010u;  // 1 + 2^-16: a unitary matrix and its rounding
+// exponent we: norms are at most 2^we
+BRI_D int fx_we(unsigned hi) {
+    if (hi <= FX_ONE) return 0;
+    return ((int)(hi >> 20) - 1022 + 1) >> 1;  // |.|^2 < 2^(exponent field - 1022)
+}
+
+// limb copies are stored in blocks of 32 sites, [..][Vp/32][entries][32] with Vp
+// = V rounded up to 32: the entries of a site lie at fixed offsets from its first
+BRI_D size_t fx_at(int site, int entries) { return (size_t)(site >> 5) * (32 * entries) + (site & 31); }
+
+__global__ void k_fx_links(const double2 *__restrict__ h, int4 *__restrict__ o, int V, unsigned *info) {
+    const int site = blockIdx.x * blockDim.x + threadIdx.x;
+    if (site >= V) return;
+    const int we = fx_we(info[0]);
+    double2 w[9];
+#pragma unroll
+    for (int e = 0; e < 9; e++) w[e] = h[((size_t)blockIdx.y * 9 + e) * V + site];
+    if (we > 400 || norm_hi(w) > max(info[0], FX_ONE)) {  // infinities, NaN or huge entries
+        info[1] = 1;
+        return;
+    }
+#pragma unroll
+    for (int e = 0; e < 9; e++)
+        o[(size_t)blockIdx.y * 9 * ((V + 31) & ~31) + fx_at(site, 9) + 32 * e] = fx_split(w[e].x, w[e].y, FX_WB - we);
+}
+
+// spinors to limbs [nrhs][Vp/32][12][32] and block exponents [nrhs][V], for n
+// sites from s0 on (modulo V)
+__global__ void k_fx_spinor(const double2 *__restrict__ in, int4 *__restrict__ p, int *__restrict__ ex, int V, int s0,
+                            int n, const int *__restrict__ skip) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, rhs = blockIdx.y;
+    if (i >= n || (skip && skip[rhs])) return;
+    int site = s0 + i;
+    if (site >= V) site -= V;
+    double2 v[12];
+    load_spinor(in + ((size_t)rhs * V + site) * 12, v);
+    unsigned m = 0;
+    bool zero = true;
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+        m = max(m, max(abs_hi(v[k].x), abs_hi(v[k].y)));
+        zero = zero && v[k].x == 0.0 && v[k].y == 0.0;
+    }
+    const int f = (int)(m >> 20);
+    const bool bad = f == 2047;
+    const int e = bad ? FX_BAD : zero ? FX_ZERO : f - 1022;
+    ex[(size_t)rhs * V + site] = e;
+    p += (size_t)rhs * 12 * ((V + 31) & ~31) + fx_at(site, 12);
+#pragma unroll
+    for (int k = 0; k < 12; k++)
+        p[32 * k] = (bad || zero) ? make_int4(0, 0, 0, 0) : fx_split(v[k].x, v[k].y, FX_PB - e);
+}
+
+// one colour row of W p (SGN = 1, w = row c of W) or W^dagger p (SGN = -1,
+// w = column c of W) for the two spins in p, rounded to units of
+// 2^(we + e - 58 + sh)
+template <int SGN>
+BRI_D void fx_row(const int4 w[3], const int4 p[6], int sh, long long half, long long re[2], long long im[2]) {
+    // The cross products are kept 2^63 up, so that their high word is added
+    // without a sign word (2^31 less in the other accumulator); both start at
+    // half a unit, which rounds to nearest and leaves a zero row zero
+    constexpr unsigned long long up = (1ull << 63) + (1ull << 31);
+    const long long a0 = half - (1ll << 31);
+    long long ar[2] = {a0, a0}, ai[2] = {a0, a0};
+    unsigned long long br[2] = {up, up}, bi[2] = {up, up};
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const int wrh = w[k].x, wrl = w[k].y;
+        const int wih = SGN > 0 ? w[k].z : -w[k].z, wil = SGN > 0 ? w[k].w : -w[k].w;
+        const int nih = SGN > 0 ? -w[k].z : w[k].z, nil = SGN > 0 ? -w[k].w : w[k].w;
+#pragma unroll
+        for (int l = 0; l < 2; l++) {
+            const int4 q = p[3 * l + k];
+            ar[l] += (long long)wrh * q.x;
+            ai[l] += (long long)wrh * q.z;
+            br[l] += (long long)wrh * q.y;
+            bi[l] += (long long)wrh * q.w;
+            br[l] += (long long)wrl * q.x;
+            bi[l] += (long long)wrl * q.z;
+            ar[l] += (long long)nih * q.z;
+            ai[l] += (long long)wih * q.x;
+            br[l] += (long long)nih * q.w;
+            bi[l] += (long long)wih * q.y;
+            br[l] += (long long)nil * q.z;
+            bi[l] += (long long)wil * q.x;
+        }
+    }
+#pragma unroll
+    for (int l = 0; l < 2; l++) {
+        re[l] = (ar[l] + (long long)(br[l] >> 32)) >> sh;
+        im[l] = (ai[l] + (long long)(bi[l] >> 32)) >> sh;
+    }
+}
+
+BRI_D void fx_negate(int4 p[6]) {
+#pragma unroll
+    for (int k = 0; k < 6; k++) p[k] = make_int4(-p[k].x, -p[k].y, -p[k].z, -p[k].w);
+}
+
+// the FP64 loop for one site, whole spinor (the arithmetic of hop_pair with
+// run-time offsets)
+__device__ __noinline__ void fx_slow(int mode, const LinkF64 &ll, const double2 *__restrict__ in,
+                                     double2 *__restrict__ out, int site, const Geom &g, double diag) {
+    int x[4];
+    const SiteNb nb = site_nb(g, site, x);
+    AccD acc;
+    for (int i = 0; i < 12; i++) acc.a[i] = make_double2(0.0, 0.0);
+    const double rsign = mode == 1 ? -1.0 : 1.0;
+#pragma unroll 1
+    for (int t = 0; t < g.nhop; t++) {
+        const HopArg &h = g.hop[t];
+        int yf, yb;
+        float phf, phb;
+        hop_nb(h.dm, site, nb, yf, phf, yb, phb);
+        const int n = abs(h.dm[0]) + abs(h.dm[1]) + abs(h.dm[2]) + abs(h.dm[3]);
+        const double q = (double)(phf * phb), L = g.lamd[n] * (double)phf, R = g.rhod[n] * (double)phf * rsign;
+        double2 cf[12];
+        {
+            const M3<double2> W = ll.load(h.j, site);
+            double2 p[12];
+            load_spinor(in + (size_t)yf * 12, p);
+#pragma unroll
+            for (int sp = 0; sp < 4; sp++) mv64<1>(W, p, sp, cf + 3 * sp);
+        }
+        const M3<double2> W = ll.load(h.j, yb);
+        double2 p[12];
+        load_spinor(in + (size_t)yb * 12, p);
+#pragma unroll
+        for (int sp = 0; sp < 4; sp++) {
+            double2 cb[3];
+            mv64<-1>(W, p, sp, cb);
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                double2 &f = cf[3 * sp + c];
+                const double sx = fma(q, cb[c].x, f.x), sy = fma(q, cb[c].y, f.y);
+                f.x = fma(-q, cb[c].x, f.x);
+                f.y = fma(-q, cb[c].y, f.y);
+                acc.a[3 * sp + c].x = fma(L, sx, acc.a[3 * sp + c].x);
+                acc.a[3 * sp + c].y = fma(L, sy, acc.a[3 * sp + c].y);
+            }
+        }
+#pragma unroll
+        for (int mu = 0; mu < 4; mu++) {
+            if (h.dm[mu] == 0) continue;
+            const double rd = R * (double)h.dm[mu];
+#pragma unroll
+            for (int sp = 0; sp < 4; sp++) {
+                const int s = gcol(mu, sp);
+                const int gr = gre(mu, s), gi = gim(mu, s);
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    if (gr != 0) acc_re(acc.a[3 * s + c], rd * (double)gr, cf[3 * sp + c]);
+                    else acc_im(acc.a[3 * s + c], rd * (double)gi, cf[3 * sp + c]);
+                }
+            }
+        }
+    }
+    if (g.clov64) dslash_finish<double2, true>(mode, in, out, site, g, diag, acc);
+    else dslash_finish<double2, false>(mode, in, out, site, g, diag, acc);
+}
+
+// One thread per (site, chirality, split): a warp holds 32 sites, its spins
+// 2h, 2h + 1, and every S-th pair of the class-ordered hop list; the two warps
+// of a group (h = 0, 1) share the links of a pair, which they copy to shared
+// memory one pair ahead (h = 0 those of x, h = 1 those of x - d).  The splits
+// fill the chip on small lattices.  At the end of each class its sums go to
+// shared memory in FP64: lambda's to the spins' own rows, gamma_d's to the
+// rows of the other chirality (to which gamma_mu maps).
+constexpr int FX_REGS = 168;                               // registers: 12 warps per SM (128 spill, 4% slower)
+template <int S> constexpr int FX_T = S == 4 ? 256 : 128;  // threads per block
+constexpr int FX_STAGE = 2 * 9 * 32;                        // int4 of the links of a pair, 32 sites
+template <int S> constexpr int FX_SMEM = FX_T<S> * 12 * 8 + (FX_T<S> / 64) * 2 * FX_STAGE * 16;
+
+BRI_D void fx_copy(uint32_t dst, const int4 *src) {
+#pragma unroll
+    for (int e = 0; e < 9; e++) cp_async16(dst + 512 * e, src + 32 * e);
+}
+BRI_D int4 lds4i(uint32_t a) {
+    int4 v;
+    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+
+template <int S, bool CLOV>
+__global__ void __maxnreg__(FX_REGS) k_dslash_fx(int mode, const int4 *__restrict__ W, const unsigned *__restrict__ info,
+                                                 LinkF64 ll, const int4 *__restrict__ P, const int *__restrict__ ex,
+                                                 const double2 *__restrict__ in, double2 *__restrict__ out,
+                                                 const __grid_constant__ Geom g, const FxOrder ord, double diag,
+                                                 const int *__restrict__ skip) {
+    constexpr int T = FX_T<S>, SPB = T / (2 * S);  // threads, sites per block
+    extern __shared__ __align__(16) unsigned char fx_sm[];
+    double *sm = (double *)fx_sm;  // [12][T]: the result's class sums
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int h = warp & 1, grp = warp >> 1, split = grp % S, sgrp = grp / S;
+    const uint32_t stage =
+        (uint32_t)__cvta_generic_to_shared(fx_sm + T * 12 * 8) + (uint32_t)(grp * 2 * FX_STAGE + lane) * 16u;
+    const int nblk = (g.s1 - g.s0 + SPB - 1) / SPB;
+    const int nr = (int)gridDim.x / nblk;
+    const int rhs = (int)blockIdx.x % nr;
+    if (skip && skip[rhs]) return;
+    const int want = g.s0 + ((int)blockIdx.x / nr) * SPB + sgrp * 32 + lane;
+    const bool active = want < g.s1;
+    const int site = active ? want : g.s1 - 1;
+    const int V = g.V, nh = g.nhop;
+    const size_t Vp = (size_t)((V + 31) & ~31);
+    in += (size_t)rhs * V * 12;
+    out += (size_t)rhs * V * 12;
+    P += (size_t)rhs * 12 * Vp + 6 * 32 * h;
+    ex += (size_t)rhs * V;
+    int x[4];
+    const SiteNb nb = site_nb(g, site, x);
+    // largest block exponent of each class's neighbours: the site's 2 S threads
+    // take the pairs in turn
+    int X[4] = {FX_ZERO, FX_ZERO, FX_ZERO, FX_ZERO};
+#pragma unroll 4
+    for (int i = 2 * split + h; i < nh; i += 2 * S) {
+        int yf, yb;
+        float phf, phb;
+        hop_nb(g.hop[ord.t[i]].dm, site, nb, yf, phf, yb, phb);
+        const int m = max(ex[yf], ex[yb]), n = ord.cls[i];
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            if (n == k + 1) X[k] = max(X[k], m);
+    }
+    int *se = (int *)sm;
+#pragma unroll
+    for (int k = 0; k < 4; k++) se[k * T + tid] = X[k];
+    __syncthreads();
+    const int we = fx_we(info[0]);
+    bool slow = info[1] != 0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        for (int q = 0; q < 2 * S; q++) X[k] = max(X[k], se[k * T + (sgrp * 2 * S + q) * 32 + lane]);
+        X[k] = X[k] == FX_ZERO ? 0 : X[k] + fx_head(k + 1);
+        slow = slow || we + X[k] > 900 || we + X[k] < -900;
+    }
+    __syncthreads();
+    const int sg = h ? 1 : -1;  // gamma_1..3 change sign between the chiralities, gamma_4 does not
+
+    long long La[12], Ga[12];  // own rows [spin][colour][re, im]; rows of the other chirality
+#pragma unroll
+    for (int i = 0; i < 12; i++) {
+        La[i] = Ga[i] = 0;
+        sm[i * T + tid] = 0.0;
+    }
+    int cls = split < nh ? ord.cls[split] : 1;
+    int Xn = cls == 1 ? X[0] : cls == 2 ? X[1] : cls == 3 ? X[2] : X[3];
+    auto flush = [&](int n) {
+        const double scale = slow ? 0.0 : __hiloint2double((1023 + we + Xn - FX_AB) << 20, 0);
+        const double cl = g.lamd[n] * scale, cg = g.rhod[n] * (mode == 1 ? -scale : scale);
+#pragma unroll
+        for (int i = 0; i < 12; i++) sm[i * T + tid] = fma((double)La[i], cl, sm[i * T + tid]);
+        asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");
+#pragma unroll
+        for (int i = 0; i < 12; i++) {
+            sm[i * T + (tid ^ 32)] = fma((double)Ga[i], cg, sm[i * T + (tid ^ 32)]);
+            La[i] = Ga[i] = 0;
+        }
+    };
+    int yf = site, yb = site;
+    float phf = 1.f, phb = 1.f;
+    const size_t own = fx_at(site, 9);
+    auto ahead = [&](int i, int buf) {  // neighbours of pair i and the copies of its links
+        const HopArg &hp = g.hop[ord.t[i]];
+        hop_nb(hp.dm, site, nb, yf, phf, yb, phb);
+        fx_copy(stage + (uint32_t)(buf * FX_STAGE + h * 9 * 32) * 16u,
+                W + (size_t)hp.j * 9 * Vp + (h ? fx_at(yb, 9) : own));
+    };
+    if (split < nh) ahead(split, 0);
+    int buf = 0;
+#pragma unroll 1
+    for (int i = split; i < nh; i += S) {
+        // this pair's copies (both warps'), and the other buffer free again
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");
+        const int cyf = yf, cyb = yb;
+        const bool nf = phf < 0.f, ng = phb < 0.f;
+        if (i + S < nh) ahead(i + S, buf ^ 1);
+        const HopArg &hp = g.hop[ord.t[i]];
+        if (ord.cls[i] != cls) {
+            flush(cls);
+            cls = ord.cls[i];
+            Xn = cls == 1 ? X[0] : cls == 2 ? X[1] : cls == 3 ? X[2] : X[3];
+        }
+        const uint32_t wf = stage + (uint32_t)(buf * FX_STAGE) * 16u, wb = wf + 9u * 512u;
+        buf ^= 1;
+        long long f[12];
+        {
+            int4 p[6];
+            const int4 *pp = P + fx_at(cyf, 12);
+#pragma unroll
+            for (int k = 0; k < 6; k++) p[k] = pp[32 * k];
+            const int sh = min(Xn - ex[cyf], 63);
+            const long long half = (long long)((1ull << sh) >> 1);
+            if (nf) fx_negate(p);
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                int4 w[3];
+#pragma unroll
+                for (int k = 0; k < 3; k++) w[k] = lds4i(wf + 512u * (3 * c + k));
+                long long re[2], im[2];
+                fx_row<1>(w, p, sh, half, re, im);
+#pragma unroll
+                for (int l = 0; l < 2; l++) {
+                    f[6 * l + 2 * c] = re[l];
+                    f[6 * l + 2 * c + 1] = im[l];
+                    La[6 * l + 2 * c] += re[l];
+                    La[6 * l + 2 * c + 1] += im[l];
+                }
+            }
+        }
+        {
+            int4 p[6];
+            const int4 *pp = P + fx_at(cyb, 12);
+#pragma unroll
+            for (int k = 0; k < 6; k++) p[k] = pp[32 * k];
+            const int sh = min(Xn - ex[cyb], 63);
+            const long long half = (long long)((1ull << sh) >> 1);
+            if (ng) fx_negate(p);
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                int4 w[3];
+#pragma unroll
+                for (int k = 0; k < 3; k++) w[k] = lds4i(wb + 512u * (3 * k + c));
+                long long re[2], im[2];
+                fx_row<-1>(w, p, sh, half, re, im);
+#pragma unroll
+                for (int l = 0; l < 2; l++) {
+                    La[6 * l + 2 * c] += re[l];
+                    La[6 * l + 2 * c + 1] += im[l];
+                    f[6 * l + 2 * c] -= re[l];
+                    f[6 * l + 2 * c + 1] -= im[l];
+                }
+            }
+        }
+        // gamma_d of the difference: additions to the other chirality's rows (for
+        // h = 1 the rows gcol(mu, 2 + l) of gamma_mu; for h = 0 the same places)
+        auto gamma_add = [&](int mu, bool pos) {
+#pragma unroll
+            for (int l = 0; l < 2; l++) {
+                const int r = gcol(mu, 2 + l), gr = gre(mu, r), gi = gim(mu, r);
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    const long long a = f[6 * l + 2 * c], b = f[6 * l + 2 * c + 1];
+                    long long &gx = Ga[6 * r + 2 * c], &gy = Ga[6 * r + 2 * c + 1];
+                    const bool up = (gr + gi > 0) == pos;
+                    if (gr != 0) {
+                        gx = up ? gx + a : gx - a;
+                        gy = up ? gy + b : gy - b;
+                    } else {
+                        gx = up ? gx - b : gx + b;
+                        gy = up ? gy + a : gy - a;
+                    }
+                }
+            }
+        };
+#pragma unroll
+        for (int mu = 0; mu < 4; mu++) {
+            const int dm = mu < 3 ? sg * hp.dm[mu] : hp.dm[mu];  // uniform across the warp
+            if (dm > 0) gamma_add(mu, true);
+            else if (dm < 0) gamma_add(mu, false);
+        }
+    }
+    flush(cls);
+    __syncthreads();
+    if (split != 0 || !active) return;
+    if (slow) {
+        if (h == 0) fx_slow(mode, ll, in, out, site, g, diag);
+        return;
+    }
+    double2 o[6], p[6];
+#pragma unroll
+    for (int i = 0; i < 6; i++) p[i] = in[(size_t)site * 12 + 6 * h + i];
+#pragma unroll
+    for (int i = 0; i < 6; i++) {
+        double2 v = make_double2(0.0, 0.0);
+        for (int k = 0; k < S; k++) {
+            v.x += sm[(2 * i) * T + tid + 64 * k];
+            v.y += sm[(2 * i + 1) * T + tid + 64 * k];
+        }
+        o[i] = make_double2(fma(diag, p[i].x, v.x), fma(diag, p[i].y, v.y));
+    }
+    if constexpr (CLOV) {
+        double2 c[18];
+#pragma unroll
+        for (int e = 0; e < 18; e++) c[e] = g.clov64[(size_t)(18 * h + e) * V + site];
+        clover_block(c, p, o);
+    }
+    const double s5 = mode == 2 && h == 1 ? -1.0 : 1.0;
+#pragma unroll
+    for (int i = 0; i < 6; i++) out[(size_t)site * 12 + 6 * h + i] = make_double2(s5 * o[i].x, s5 * o[i].y);
+}
+
+FxOrder fx_order(const Geom &g) {
+    FxOrder o{};
+    int n = 0;
+    for (int c = 1; c <= 4; c++)
+        for (int t = 0; t < g.nhop; t++) {
+            const int *d = g.hop[t].dm;
+            if ((d[0] != 0) + (d[1] != 0) + (d[2] != 0) + (d[3] != 0) != c) continue;
+            o.t[n] = (unsigned char)t;
+            o.cls[n++] = (unsigned char)c;
+        }
+    return o;
+}
+
+size_t fx_vp(const Geom &g) { return (size_t)((g.V + 31) & ~31); }
+size_t fx_bytes(const Geom &g, int nrhs) { return (sizeof(int4) * 12 + sizeof(int)) * fx_vp(g) * nrhs; }
+
+template <int S, bool CLOV>
+void fx_launch(int mode, bri_ctx *ctx, const Geom &g, const int4 *P, const int *ex, const void *in, void *out, int nrhs,
+               double diag, const int *skip, cudaStream_t s) {
+    constexpr int T = FX_T<S>, SPB = T / (2 * S);
+    static bool attr = false;
+    if (!attr) {
+        cudaFuncSetAttribute(k_dslash_fx<S, CLOV>, cudaFuncAttributeMaxDynamicSharedMemorySize, FX_SMEM<S>);
+        attr = true;
+    }
+    const unsigned nb = (unsigned)((g.s1 - g.s0 + SPB - 1) / SPB) * (unsigned)nrhs;
+    k_dslash_fx<S, CLOV><<<nb, T, FX_SMEM<S>, s>>>(mode, ctx->hopsfx, ctx->fxinfo, LinkF64{ctx->hops64, g.V}, P, ex,
+                                                   (const double2 *)in, (double2 *)out, g, fx_order(g), diag, skip);
+}
+
+}  // namespace
+
+// fixed-point copy of the FP64 fields; without memory for it the FP64 kernel is used
+bri_status bri_fx_store_impl(bri_ctx *ctx, cudaStream_t s) {
+    const Geom &g = ctx->g;
+    const size_t bytes = sizeof(int4) * 9 * NCANON * fx_vp(g);
+    ctx->have_fx = false;
+    if (!ctx->hopsfx) {
+        if (ctx->fx_tried) return BRI_OK;
+        ctx->fx_tried = true;
+        cudaError_t e = cudaMalloc(&ctx->hopsfx, bytes);
+        if (e == cudaErrorMemoryAllocation) {
+            // path sums just released may still be held by the stream-ordered pool
+            cudaGetLastError();
+            BRI_TRY_CUDA(ctx, cudaStreamSynchronize(s));
+            e = cudaMalloc(&ctx->hopsfx, bytes);
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            ctx->hopsfx = nullptr;
+            return BRI_OK;
+        }
+    }
+    if (!ctx->fxinfo) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->fxinfo, 2 * sizeof(unsigned)));
+    if (!ctx->pool) {
+        cudaMemPoolProps pp{};
+        pp.allocType = cudaMemAllocationTypePinned;
+        pp.location.type = cudaMemLocationTypeDevice;
+        pp.location.id = ctx->device;
+        BRI_TRY_CUDA(ctx, cudaMemPoolCreate(&ctx->pool, &pp));
+        uint64_t keep = ~0ull;  // held until the context is destroyed: at most the largest concurrent use
+        BRI_TRY_CUDA(ctx, cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep));
+    }
+    const int T = 128;
+    const unsigned nb = (unsigned)((g.V + T - 1) / T);
+    BRI_TRY_CUDA(ctx, cudaMemsetAsync(ctx->fxinfo, 0, 2 * sizeof(unsigned), s));
+    k_fx_max<<<dim3(nb, 4), T, 0, s>>>(ctx->hops64, g.V, ctx->fxinfo);
+    BRI_LAUNCHED(ctx);
+    k_fx_links<<<dim3(nb, NCANON), T, 0, s>>>(ctx->hops64, ctx->hopsfx, g.V, ctx->fxinfo);
+    BRI_LAUNCHED(ctx);
+    ctx->have_fx = true;
+    return BRI_OK;
+}
+
+size_t bri_fx_work_bytes(bri_ctx *ctx, int nrhs) { return fx_bytes(ctx->g, nrhs); }
+
+// FP64 apply of sites [g.s0, g.s1) in fixed point; work: bri_fx_work_bytes, or
+// null to take it from the context's stream-ordered pool.  The right-hand
+// sides done so far are counted in *ndone; fewer than nrhs with BRI_OK: no
+// memory for the limb copies, the caller runs the FP64 kernel on the rest.
+bri_status bri_dslash_fx(bri_ctx *ctx, const Geom &g, void *out, const void *in, int nrhs, double m0, int mode,
+                         const int *skip, void *work, int *ndone, cudaStream_t s) {
+    const double diag = m0 + g.lamd[0];
+    const size_t field = (size_t)g.V * 12;
+    // right-hand sides per launch: up to 2 GB of limb copies
+    const int rmax = (int)std::max<size_t>(1, std::min<size_t>(32, ((size_t)2 << 30) / fx_bytes(g, 1)));
+    if (nrhs > rmax && !work) {
+        for (int r = 0; r < nrhs && *ndone == r; r += rmax)
+            BRI_RETURN_IF(bri_dslash_fx(ctx, g, (double2 *)out + r * field, (const double2 *)in + r * field,
+                                        nrhs - r < rmax ? nrhs - r : rmax, m0, mode, skip ? skip + r : nullptr, work,
+                                        ndone, s));
+        return BRI_OK;
+    }
+    void *own = nullptr;
+    if (!work) {
+        const cudaError_t e = cudaMallocFromPoolAsync(&own, fx_bytes(g, nrhs), ctx->pool, s);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            return BRI_OK;
+        }
+        BRI_TRY_CUDA(ctx, e);
+        work = own;
+    }
+    int4 *P = (int4 *)work;
+    int *ex = (int *)(P + 12 * fx_vp(g) * nrhs);
+    // a site range reads one time slice beyond each end
+    const int S3 = g.L[0] * g.L[1] * g.L[2];
+    const bool all = g.s0 == 0 && g.s1 == g.V;
+    const long long span = (long long)g.s1 - g.s0 + 2 * S3;
+    const int n = all || span >= g.V ? g.V : (int)span, first = n == g.V ? 0 : (g.s0 - S3 + g.V) % g.V;
+    k_fx_spinor<<<dim3((unsigned)((n + 127) / 128), (unsigned)nrhs), 128, 0, s>>>((const double2 *)in, P, ex, g.V,
+                                                                                  first, n, skip);
+    BRI_LAUNCHED(ctx);
+    // splits of the hop list, so that the 608 schedulers have two warps or more
+    const long long warps = 2ll * ((g.s1 - g.s0 + 31) / 32) * nrhs;
+    const int S = warps >= 2432 ? 1 : warps >= 1216 ? 2 : 4;
+    auto launch = g.clov64 ? (S == 1 ? fx_launch<1, true> : S == 2 ? fx_launch<2, true> : fx_launch<4, true>)
+                           : (S == 1 ? fx_launch<1, false> : S == 2 ? fx_launch<2, false> : fx_launch<4, false>);
+    launch(mode, ctx, g, P, ex, in, out, nrhs, diag, skip, s);
+    BRI_LAUNCHED(ctx);
+    if (own) BRI_TRY_CUDA(ctx, cudaFreeAsync(own, s));
+    *ndone += nrhs;
+    return BRI_OK;
+}

@@ -234,7 +234,7 @@ bri_status bri_hops_build_impl(bri_ctx *ctx, cudaStream_t s) {
     ctx->f16.valid = false;
     ctx->p32.valid = false;
     ctx->p16.valid = false;
-    return BRI_OK;
+    return bri_fx_store_impl(ctx, s);
 }
 
 bri_status bri_hops_store_impl(bri_ctx *ctx, bri_prec prec, bri_comp comp, cudaStream_t s) {

@@ -351,6 +351,7 @@ struct SolverWork {
     int nrhs = 0;
     VecSet v64, v32;
     double2 *r64 = nullptr;
+    void *fxw = nullptr;  // work space of the FP64 apply inside captured iterations (one right-hand side)
     BiState *st = nullptr;
     int *flag = nullptr;
     int *done = nullptr;
@@ -358,7 +359,11 @@ struct SolverWork {
     unsigned *tick = nullptr;
     double *nrm = nullptr;
     cudaStream_t own = nullptr;
-    std::map<std::string, cudaGraphExec_t> graphs;
+    struct Captured {
+        cudaGraphExec_t exec;
+        long launches;  // kernels of one replay
+    };
+    std::map<std::string, Captured> graphs;
 };
 
 static void free_vecs(VecSet &v) {
@@ -372,10 +377,11 @@ static void free_vecs(VecSet &v) {
 void bri_solver_free(bri_ctx *ctx) {
     SolverWork *w = ctx->work;
     if (!w) return;
-    for (auto &kv : w->graphs) cudaGraphExecDestroy(kv.second);
+    for (auto &kv : w->graphs) cudaGraphExecDestroy(kv.second.exec);
     free_vecs(w->v64);
     free_vecs(w->v32);
     cudaFree(w->r64);
+    cudaFree(w->fxw);
     cudaFree(w->st);
     cudaFree(w->flag);
     cudaFree(w->done);
@@ -406,7 +412,10 @@ static bri_status ensure_work(bri_ctx *ctx, int nrhs, bool need64, bool need32) 
     w->n = n;
     w->nrhs = nrhs > have_nrhs ? nrhs : have_nrhs;
     const size_t R = w->nrhs;
-    if (need64 || had64) BRI_RETURN_IF(alloc_vecs(ctx, w->v64, sizeof(double2) * n * R));
+    if (need64 || had64) {
+        BRI_RETURN_IF(alloc_vecs(ctx, w->v64, sizeof(double2) * n * R));
+        BRI_TRY_CUDA(ctx, cudaMalloc(&w->fxw, bri_fx_work_bytes(ctx, 1)));
+    }
     if (need32 || had32) {
         BRI_RETURN_IF(alloc_vecs(ctx, w->v32, sizeof(float2) * n * R));
         BRI_TRY_CUDA(ctx, cudaMalloc(&w->r64, sizeof(double2) * n * R));
@@ -437,12 +446,12 @@ bri_status enqueue_iters(bri_ctx *ctx, const VecSet &vs, int nrhs, double m0, br
     for (int it = 0; it < iters; it++) {
         k_bi_p<T><<<grid, RT, 0, s>>>(p, r, v, w->st, w->flag, n);
         BRI_LAUNCHED(ctx);
-        BRI_RETURN_IF(bri_dslash_raw(ctx, v, p, nrhs, m0, 0, prec, w->flag, thr, s));
+        BRI_RETURN_IF(bri_dslash_raw(ctx, v, p, nrhs, m0, 0, prec, w->flag, thr, s, w->fxw));
         k_bi_alpha<T><<<grid, RT, 0, s>>>(rh, v, w->st, w->flag, w->part, w->tick, n);
         BRI_LAUNCHED(ctx);
         k_bi_s<T><<<grid, RT, 0, s>>>(sv, r, v, w->st, w->flag, n);
         BRI_LAUNCHED(ctx);
-        BRI_RETURN_IF(bri_dslash_raw(ctx, t, sv, nrhs, m0, 0, prec, w->flag, thr, s));
+        BRI_RETURN_IF(bri_dslash_raw(ctx, t, sv, nrhs, m0, 0, prec, w->flag, thr, s, w->fxw));
         k_bi_omega<T><<<grid, RT, 0, s>>>(t, sv, w->st, w->flag, w->part, w->tick, n);
         BRI_LAUNCHED(ctx);
         k_bi_xr<T><<<grid, RT, 0, s>>>(x, r, p, sv, t, rh, w->st, w->flag, w->part, w->tick, n);
@@ -474,10 +483,10 @@ bri_status bicgstab(bri_ctx *ctx, const VecSet &vs, const T *b, bool have_x0, in
     char key[192];
     snprintf(key, sizeof key, "bi:%d:%d:%d:%.17g:%p:%p:%p:%d", (int)sizeof(T), (int)prec, nrhs, m0, vs.x, vs.s,
              vs.t, bri_dslash_threads(ctx, prec, nrhs));
-    cudaGraphExec_t exec = nullptr;
+    SolverWork::Captured run{};
     auto it = w->graphs.find(key);
     if (it != w->graphs.end()) {
-        exec = it->second;
+        run = it->second;
     } else {
         // the tensor-core apply and the site-pair kernel allocate on first use:
         // not inside the capture
@@ -487,15 +496,17 @@ bri_status bicgstab(bri_ctx *ctx, const VecSet &vs, const T *b, bool have_x0, in
             !ctx->g.clov64)
             BRI_RETURN_IF(bri_pair_store_impl(ctx, prec, s));
         cudaGraph_t graph;
+        const long before = ctx->launches;
         BRI_TRY_CUDA(ctx, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
         bri_status st = enqueue_iters<T>(ctx, vs, nrhs, m0, prec, K, s);
         cudaError_t e = cudaStreamEndCapture(s, &graph);
         if (st != BRI_OK) return st;
         if (e != cudaSuccess) return bri_fail(ctx, BRI_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-        BRI_TRY_CUDA(ctx, cudaGraphInstantiate(&exec, graph, 0));
+        BRI_TRY_CUDA(ctx, cudaGraphInstantiate(&run.exec, graph, 0));
         cudaGraphDestroy(graph);
-        w->graphs[key] = exec;
-        ctx->launches -= 7 * K;  // captured, not launched
+        run.launches = ctx->launches - before;
+        ctx->launches = before;  // captured, not launched
+        w->graphs[key] = run;
     }
     flags.assign(nrhs, 0);
     iters.assign(nrhs, 0);
@@ -506,8 +517,8 @@ bri_status bicgstab(bri_ctx *ctx, const VecSet &vs, const T *b, bool have_x0, in
         bool all = true;
         for (int r = 0; r < nrhs; r++) all = all && flags[r] != 0;
         if (all) break;
-        BRI_TRY_CUDA(ctx, cudaGraphLaunch(exec, s));
-        ctx->launches += 7 * K;
+        BRI_TRY_CUDA(ctx, cudaGraphLaunch(run.exec, s));
+        ctx->launches += run.launches;
     }
     BRI_TRY_CUDA(ctx, cudaMemcpyAsync(flags.data(), w->flag, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, s));
     BRI_TRY_CUDA(ctx, cudaMemcpyAsync(hs.data(), w->st, sizeof(BiState) * nrhs, cudaMemcpyDeviceToHost, s));

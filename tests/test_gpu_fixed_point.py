@@ -1,0 +1,107 @@
+"""The FP64 apply in fixed point (csrc/dslash_fx.cu): at the sizes where its
+split of the hop list changes, on site ranges, with fields that span many
+orders of magnitude, with links that are not unitary, and with infinities and
+NaN (where it runs the FP64 loop), against the oracle.
+
+Tolerance: every product is known to 2^-55 of its class's largest neighbour,
+the final FP64 operations round a few times: 1e-15 of the largest result, and
+4e-15 of each site's own largest component (weights 1/16 to 1/432 times up to
+32 hops a class)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1012_3615_gb300 import Brillouin, synth
+
+pytestmark = pytest.mark.gpu
+AP = (1, 1, 1, -1)
+
+
+def _op(L, U, gpu):
+    """the operator, and its 81 fields in the oracle's order (W_{-d}(x) = W_d(x - d)^dagger)"""
+    op = Brillouin(L, AP)
+    op.build_hops(torch.as_tensor(U, device=gpu))
+    h = op.hops().cpu().numpy()
+    x = synth.coordinates(L)
+    W = np.zeros((len(x), 81, 3, 3), complex)
+    W[:, 40] = np.eye(3)
+    for j in range(40):
+        d = [((j + 41) // 3 ** mu) % 3 - 1 for mu in range(4)]
+        back = ((x - d) % L) @ np.cumprod((1,) + tuple(L[:3]))
+        W[:, 41 + j] = h[:, j]
+        W[:, 39 - j] = h[back, j].conj().transpose(0, 2, 1)
+    return op, W
+
+
+# volumes on both sides of the lines between 4, 2 and 1 splits of the hop list
+# (2 ceil(V / 32) nrhs warps at 1216 and 2432), ragged last groups
+@pytest.mark.parametrize("L,nrhs", [((3, 3, 3, 3), 1), ((5, 3, 7, 3), 2), ((11, 12, 12, 12), 1), ((11, 11, 12, 13), 1),
+                                    ((13, 14, 14, 15), 1), ((14, 14, 14, 15), 1), ((4, 5, 3, 4), 40)])
+def test_splits_against_oracle(gpu, L, nrhs):
+    U = synth.random_su3_links(L, 0.4, 5)
+    psi = synth.gaussian_spinor(L, nrhs, 6)
+    op, W = _op(L, U, gpu)
+    x = torch.as_tensor(psi, device=gpu)
+    for r in (0, nrhs - 1):
+        for dag in (False, True):
+            out = op.apply(x, m0=0.1, dagger=dag)[r].cpu().numpy()
+            ref = oracle.apply(L, AP, W, 0.1, psi[r], dagger=dag)
+            assert np.abs(out - ref).max() <= 1e-15 * np.abs(ref).max() * 4  # the oracle rounds ~480 sums in FP64
+
+
+def test_orders_of_magnitude(gpu):
+    """a field falling by e^-2 per step in every direction, a point source and a
+    tiny and a huge field: each site to rounding of its own size"""
+    L = (5, 4, 6, 4)
+    U = synth.random_su3_links(L, 0.3, 7)
+    op, W = _op(L, U, gpu)
+    psi = np.repeat(synth.gaussian_spinor(L, 1, 8), 4, axis=0)
+    psi[0] *= np.exp(-2.0 * synth.coordinates(L).sum(1))[:, None, None]
+    psi[1] = 0
+    psi[1, 17, 2, 1] = 1.0
+    psi[2] *= 1e-290
+    psi[3] *= 1e290
+    out = op.apply(torch.as_tensor(psi, device=gpu), m0=0.1).cpu().numpy()
+    for r in range(4):
+        ref = oracle.apply(L, AP, W, 0.1, psi[r])
+        size = np.abs(ref).max(axis=(1, 2), keepdims=True)
+        assert (np.abs(out[r] - ref) <= 4e-15 * size).all(), r
+        assert ((out[r] == 0) == (ref == 0)).all()
+
+
+@pytest.mark.parametrize("scale", [1.0, 3.7, 1e-3, 1e60])
+def test_links_that_are_not_unitary(gpu, scale):
+    """one-hop fields are the links as given (at 1e60 the path sums overflow in the
+    projection and nothing is finite)"""
+    L = (4, 3, 5, 4)
+    U = synth.random_su3_links(L, 0.3, 9)
+    rng = np.random.default_rng(10)
+    U = scale * (U + 0.2 * (rng.standard_normal(U.shape) + 1j * rng.standard_normal(U.shape)))
+    op, W = _op(L, U, gpu)
+    psi = synth.gaussian_spinor(L, 1, 11)
+    out = op.apply(torch.as_tensor(psi, device=gpu), m0=0.1).cpu().numpy()[0]
+    ref = oracle.apply(L, AP, W, 0.1, psi[0])
+    fine = np.isfinite(ref)
+    assert np.array_equal(np.isfinite(out), fine) and (fine.all() or scale == 1e60)
+    assert (np.abs(out - ref)[fine] <= 4e-15 * np.abs(ref[fine]).max(initial=0.0)).all()
+
+
+def test_infinities_and_nan_stay_local(gpu):
+    """sites that see an infinity or a NaN are as the FP64 loop gives them (not
+    finite where the oracle is not), the others are untouched"""
+    L = (6, 7, 6, 8)
+    U = synth.random_su3_links(L, 0.3, 12)
+    op, _ = _op(L, U, gpu)
+    psi = synth.gaussian_spinor(L, 1, 13)
+    clean = op.apply(torch.as_tensor(psi, device=gpu)).cpu().numpy()[0]
+    psi[0, 100, 1, 2] = np.inf
+    psi[0, 900, 3, 0] = np.nan
+    out = op.apply(torch.as_tensor(psi, device=gpu)).cpu().numpy()[0]
+    x = synth.coordinates(L)
+    far = np.ones(len(x), bool)
+    for s in (100, 900):
+        d = np.abs(x - x[s])
+        far &= (np.minimum(d, np.array(L) - d) > 1).any(1)
+    assert np.array_equal(out[far], clean[far])
+    assert not np.isfinite(out[~far]).all(axis=(1, 2)).any()
