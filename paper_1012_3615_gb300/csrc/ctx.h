@@ -112,7 +112,7 @@ bri_status bri_tc_reserve(bri_ctx *ctx, int nrhs, int cap);
 bri_status bri_dslash_raw(bri_ctx *ctx, void *out, const void *in, int nrhs, double m0, int mode, bri_prec prec,
                           const int *skip, int threads, cudaStream_t s, void *work = nullptr);
 // FP64 apply in fixed point (dslash_fx.cu)
-bri_status bri_fx_store_impl(bri_ctx *ctx, cudaStream_t s);
+bri_status bri_fx_reserve(bri_ctx *ctx);
 size_t bri_fx_work_bytes(bri_ctx *ctx, int nrhs);
 bri_status bri_dslash_fx(bri_ctx *ctx, const bri::Geom &g, void *out, const void *in, int nrhs, double m0, int mode,
                          const int *skip, void *work, int *ndone, cudaStream_t s);
@@ -122,7 +122,8 @@ bri_status bri_export_hops_impl(bri_ctx *ctx, double2 *out, cudaStream_t s);
 void bri_solver_free(bri_ctx *ctx);
 bri_status bri_cdot_impl(bri_ctx *ctx, double *res, const void *a, const void *b, size_t n, bri_prec prec,
                          cudaStream_t user);
-bri_status bri_dp_levels(bri_ctx *ctx, void *A, const int *klist, const int start[6], cudaStream_t s);
+// path sums of the 40 stored fields from ctx->U into A ([40][9][V])
+bri_status bri_path_sums(bri_ctx *ctx, double2 *A, cudaStream_t s);
 bri_status bri_force_impl(bri_ctx *ctx, double2 *dU, const double2 *chi, const double2 *psi, cudaStream_t s);
 void bri_overlap_free(bri_ctx *ctx);
 void bri_host_apply_free(bri_ctx *ctx);

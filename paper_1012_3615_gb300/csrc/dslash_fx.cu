@@ -36,6 +36,7 @@
 #include <string>
 
 #include "dslash_kernel.cuh"
+#include "fx.cuh"
 
 using namespace bri;
 
@@ -47,90 +48,8 @@ struct FxOrder {
 
 namespace {
 
-constexpr int FX_BAD = 1 << 20;     // block exponent of a site with an infinity or a NaN
-constexpr int FX_ZERO = -(1 << 20);  // ... of a site that is zero
-constexpr int FX_WB = 62, FX_PB = 60;  // fraction bits of links and spinors
-constexpr int FX_AB = FX_WB + FX_PB - 64;  // of the row sums
 // head room h_n of the class sums
 BRI_D int fx_head(int n) { return n == 1 ? 0 : n == 2 ? 2 : 3; }
-
-// v 2^sh rounded to an integer (|v| 2^sh < 2^63), by shifts: conversions run on
-// the FP64 pipe
-BRI_D long long fx_int(double v, int sh) {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
-    const int e = (int)(bits >> 52) & 0x7ff;
-    const unsigned long long m = (bits & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
-    const int s = max(e, 1) - 1075 + sh, r = min(-s, 63);
-    const long long f = (long long)(s >= 0 ? m << s : (m + ((1ull << r) >> 1)) >> r);
-    return (long long)bits < 0 ? -f : f;
-}
-BRI_D int4 fx_split(double re, double im, int sh) {
-    // the low word is never INT_MIN, so that limbs can be negated
-    const long long a = fx_int(re, sh), b = fx_int(im, sh);
-    int4 v;
-    v.y = (int)a;
-    v.x = (int)((a - v.y) >> 32);
-    v.w = (int)b;
-    v.z = (int)((b - v.w) >> 32);
-    if (v.y == (int)0x80000000) v.y++;
-    if (v.w == (int)0x80000000) v.w++;
-    return v;
-}
-BRI_D unsigned abs_hi(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
-
-// largest |row|^2, |column|^2 of a field matrix, as the high word of a double
-// (NaN and infinities come out largest)
-BRI_D unsigned norm_hi(const double2 w[9]) {
-    unsigned m = 0;
-#pragma unroll
-    for (int i = 0; i < 3; i++) {
-        m = max(m, abs_hi(cnorm2(w[3 * i]) + cnorm2(w[3 * i + 1]) + cnorm2(w[3 * i + 2])));
-        m = max(m, abs_hi(cnorm2(w[i]) + cnorm2(w[3 + i]) + cnorm2(w[6 + i])));
-    }
-    return m;
-}
-// info[0]: the largest of the one-hop fields, which are the links as given (the
-// other fields are unitary); info[1]: 1 if a field matrix does not fit
-__global__ void k_fx_max(const double2 *__restrict__ h, int V, unsigned *info) {
-    constexpr int jf[4] = {0, 2, 8, 26};  // canonical fields of +x, +y, +z, +t
-    const int site = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned m = 0;
-    if (site < V) {
-        double2 w[9];
-        const int j = blockIdx.y == 0 ? jf[0] : blockIdx.y == 1 ? jf[1] : blockIdx.y == 2 ? jf[2] : jf[3];
-#pragma unroll
-        for (int e = 0; e < 9; e++) w[e] = h[((size_t)j * 9 + e) * V + site];
-        m = norm_hi(w);
-    }
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(info, m);
-}
-constexpr unsigned FX_ONE = 0x3ff00010u;  // 1 + 2^-16: a unitary matrix and its rounding
-// exponent we: norms are at most 2^we
-BRI_D int fx_we(unsigned hi) {
-    if (hi <= FX_ONE) return 0;
-    return ((int)(hi >> 20) - 1022 + 1) >> 1;  // |.|^2 < 2^(exponent field - 1022)
-}
-
-// limb copies are stored in blocks of 32 sites, [..][Vp/32][entries][32] with Vp
-// = V rounded up to 32: the entries of a site lie at fixed offsets from its first
-BRI_D size_t fx_at(int site, int entries) { return (size_t)(site >> 5) * (32 * entries) + (site & 31); }
-
-__global__ void k_fx_links(const double2 *__restrict__ h, int4 *__restrict__ o, int V, unsigned *info) {
-    const int site = blockIdx.x * blockDim.x + threadIdx.x;
-    if (site >= V) return;
-    const int we = fx_we(info[0]);
-    double2 w[9];
-#pragma unroll
-    for (int e = 0; e < 9; e++) w[e] = h[((size_t)blockIdx.y * 9 + e) * V + site];
-    if (we > 400 || norm_hi(w) > max(info[0], FX_ONE)) {  // infinities, NaN or huge entries
-        info[1] = 1;
-        return;
-    }
-#pragma unroll
-    for (int e = 0; e < 9; e++)
-        o[(size_t)blockIdx.y * 9 * ((V + 31) & ~31) + fx_at(site, 9) + 32 * e] = fx_split(w[e].x, w[e].y, FX_WB - we);
-}
 
 // spinors to limbs [nrhs][Vp/32][12][32] and block exponents [nrhs][V], for n
 // sites from s0 on (modulo V)
@@ -531,25 +450,16 @@ void fx_launch(int mode, bri_ctx *ctx, const Geom &g, const int4 *P, const int *
 
 }  // namespace
 
-// fixed-point copy of the FP64 fields; without memory for it the FP64 kernel is used
-bri_status bri_fx_store_impl(bri_ctx *ctx, cudaStream_t s) {
+// memory for the fixed-point copy of the FP64 fields and the work space pool;
+// without memory for the copy (ctx->hopsfx null) the FP64 kernel is used
+bri_status bri_fx_reserve(bri_ctx *ctx) {
     const Geom &g = ctx->g;
-    const size_t bytes = sizeof(int4) * 9 * NCANON * fx_vp(g);
     ctx->have_fx = false;
-    if (!ctx->hopsfx) {
-        if (ctx->fx_tried) return BRI_OK;
+    if (!ctx->hopsfx && !ctx->fx_tried) {
         ctx->fx_tried = true;
-        cudaError_t e = cudaMalloc(&ctx->hopsfx, bytes);
-        if (e == cudaErrorMemoryAllocation) {
-            // path sums just released may still be held by the stream-ordered pool
-            cudaGetLastError();
-            BRI_TRY_CUDA(ctx, cudaStreamSynchronize(s));
-            e = cudaMalloc(&ctx->hopsfx, bytes);
-        }
-        if (e != cudaSuccess) {
+        if (cudaMalloc(&ctx->hopsfx, sizeof(int4) * 9 * NCANON * fx_vp(g)) != cudaSuccess) {
             cudaGetLastError();
             ctx->hopsfx = nullptr;
-            return BRI_OK;
         }
     }
     if (!ctx->fxinfo) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->fxinfo, 2 * sizeof(unsigned)));
@@ -559,17 +469,9 @@ bri_status bri_fx_store_impl(bri_ctx *ctx, cudaStream_t s) {
         pp.location.type = cudaMemLocationTypeDevice;
         pp.location.id = ctx->device;
         BRI_TRY_CUDA(ctx, cudaMemPoolCreate(&ctx->pool, &pp));
-        uint64_t keep = ~0ull;  // held until the context is destroyed: at most the largest concurrent use
+        uint64_t keep = 4ull << 30;  // bytes held between calls; released with the context
         BRI_TRY_CUDA(ctx, cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep));
     }
-    const int T = 128;
-    const unsigned nb = (unsigned)((g.V + T - 1) / T);
-    BRI_TRY_CUDA(ctx, cudaMemsetAsync(ctx->fxinfo, 0, 2 * sizeof(unsigned), s));
-    k_fx_max<<<dim3(nb, 4), T, 0, s>>>(ctx->hops64, g.V, ctx->fxinfo);
-    BRI_LAUNCHED(ctx);
-    k_fx_links<<<dim3(nb, NCANON), T, 0, s>>>(ctx->hops64, ctx->hopsfx, g.V, ctx->fxinfo);
-    BRI_LAUNCHED(ctx);
-    ctx->have_fx = true;
     return BRI_OK;
 }
 

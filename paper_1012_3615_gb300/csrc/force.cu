@@ -21,15 +21,57 @@
 //    run backwards level by level (gather form, no atomics), and every
 //    occurrence of a link collects its share.
 #include "ctx.h"
+#include "paths.cuh"
 #include "project.cuh"
 
 using namespace bri;
 
 namespace {
 
-// step 1 (thread per site, canonical field j = blockIdx.y)
-__global__ void k_hop_grad(const double2 *__restrict__ chi, const double2 *__restrict__ psi, M3<double2> *GA,
-                           Geom g) {
+// Z += conj(chi) (x) m for one colour of m: row cp of the 3x3 matrix
+// (Z_cp,c += sum_a conj(chi_a,c) m_a), or its conjugate transpose's column
+template <bool DAG> BRI_D void outer_add(M3<double2> &G, int cp, const double2 chi[12], const double2 m[4]) {
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        double2 &z = G.e[DAG ? 3 * c + cp : 3 * cp + c];
+#pragma unroll
+        for (int a = 0; a < 4; a++) {
+            const double2 u = chi[3 * a + c], v = m[a];
+            z.x = fma(u.x, v.x, fma(u.y, v.y, z.x));
+            const double im = DAG ? -1.0 : 1.0;  // the conjugate's imaginary part
+            z.y = fma(u.x, im * v.y, fma(-u.y, im * v.x, z.y));
+        }
+    }
+}
+// m = (lam + sg rho sum_mu d_mu gamma_mu) p for the four spins of one colour
+BRI_D void gamma_mix(const double2 p[4], const int d[4], double lam, double rho, double2 m[4]) {
+#pragma unroll
+    for (int a = 0; a < 4; a++) m[a] = cscale(p[a], lam);
+#pragma unroll
+    for (int mu = 0; mu < 4; mu++) {
+        if (d[mu] == 0) continue;  // uniform across the block
+        const double r = d[mu] > 0 ? rho : -rho;
+#pragma unroll
+        for (int a = 0; a < 4; a++) {
+            const double2 v = p[gcol(mu, a)];
+            const int gr = gre(mu, a), gi = gim(mu, a);
+            if (gr != 0) {
+                m[a].x = fma(gr > 0 ? r : -r, v.x, m[a].x);
+                m[a].y = fma(gr > 0 ? r : -r, v.y, m[a].y);
+            } else {
+                m[a].x = fma(gi > 0 ? -r : r, v.y, m[a].x);
+                m[a].y = fma(gi > 0 ? r : -r, v.x, m[a].y);
+            }
+        }
+    }
+}
+
+// step 1 (thread per site, canonical field j = blockIdx.y).  FP64 operations
+// bound it: the spin mix of a colour is taken once for its three outer
+// products, 470 operations a field where one mix per matrix entry took 1,900:
+// 12^4 3.13 -> 0.73 ms
+__global__ void k_hop_grad(const double2 *__restrict__ chi, const double2 *__restrict__ psi, double2 *__restrict__ GA,
+                           const __grid_constant__ Geom g) {
     const int site = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y;
     if (site >= g.V) return;
@@ -37,10 +79,11 @@ __global__ void k_hop_grad(const double2 *__restrict__ chi, const double2 *__res
     const int n = off_class(k);
     const double lam = g.lamd[n], rho = g.rhod[n];
     int x[4];
-    SiteNb nb = site_nb(g, site, x);
+    const SiteNb nb = site_nb(g, site, x);
     int d[4];
     float ph = 1.f;
     int y = site;
+#pragma unroll
     for (int mu = 0; mu < 4; mu++) {
         d[mu] = off_comp(k, mu);
         if (d[mu] > 0) { y += nb.fw[mu]; ph *= nb.sfw[mu]; }
@@ -49,29 +92,25 @@ __global__ void k_hop_grad(const double2 *__restrict__ chi, const double2 *__res
     // forward hop (x, d):   zf[cp][c] = sum_a chi(x)[a][c]^* (M_d psi(y))[a][cp]
     // reversed hop (y, -d): zb[cp][c] = sum_a chi(y)[a][c]^* (M_{-d} psi(x))[a][cp]
     // (the boundary phase of y -> x equals that of x -> y);  G = ph (zf^dagger + zb)
-    M3<double2> Zf, Zb;  // [cp][c]
-    for (int cp = 0; cp < 3; cp++)
-        for (int c = 0; c < 3; c++) {
-            double2 zf = make_double2(0, 0), zb = make_double2(0, 0);
-            for (int a = 0; a < 4; a++) {
-                double2 mf = cscale(psi[(size_t)y * 12 + 3 * a + cp], lam);
-                double2 mb = cscale(psi[(size_t)site * 12 + 3 * a + cp], lam);
-                for (int mu = 0; mu < 4; mu++) {
-                    if (!d[mu]) continue;
-                    const int col = gcol(mu, a);
-                    const double2 e = make_double2(gre(mu, a), gim(mu, a));
-                    mf = cadd(mf, cscale(cmul(e, psi[(size_t)y * 12 + 3 * col + cp]), rho * d[mu]));
-                    mb = cadd(mb, cscale(cmul(e, psi[(size_t)site * 12 + 3 * col + cp]), -rho * d[mu]));
-                }
-                zf = cadd(zf, cmulc(chi[(size_t)site * 12 + 3 * a + c], mf));
-                zb = cadd(zb, cmulc(chi[(size_t)y * 12 + 3 * a + c], mb));
-            }
-            Zf.e[3 * cp + c] = zf;
-            Zb.e[3 * cp + c] = zb;
+    M3<double2> G = m3_zero<double2>();
+#pragma unroll 1
+    for (int dir = 0; dir < 2; dir++) {
+        const double2 *cs = chi + (size_t)(dir ? y : site) * 12, *ps = psi + (size_t)(dir ? site : y) * 12;
+        double2 c12[12];
+#pragma unroll
+        for (int i = 0; i < 12; i++) c12[i] = cs[i];
+#pragma unroll
+        for (int cp = 0; cp < 3; cp++) {
+            double2 p[4], m[4];
+#pragma unroll
+            for (int a = 0; a < 4; a++) p[a] = ps[3 * a + cp];
+            gamma_mix(p, d, lam, dir ? -rho : rho, m);
+            if (dir) outer_add<false>(G, cp, c12, m);
+            else outer_add<true>(G, cp, c12, m);
         }
-    M3<double2> G = m3_add(m3_dag(Zf), Zb);
-    for (int i = 0; i < 9; i++) G.e[i] = cscale(G.e[i], (double)ph);
-    GA[(size_t)k * g.V + site] = G;
+    }
+#pragma unroll
+    for (int e = 0; e < 9; e++) GA[((size_t)j * 9 + e) * g.V + site] = cscale(G.e[e], (double)ph);
 }
 
 // traceless anti-hermitian part
@@ -187,120 +226,139 @@ static __device__ __noinline__ void project_vjp_general(const M3<double2> &a, co
 }
 
 // step 2: G_A = VJP of the projection (off-axis canonical fields, in place)
-__global__ void k_project_vjp(const M3<double2> *__restrict__ A, M3<double2> *GA, Geom g) {
+__global__ void k_project_vjp(const double2 *__restrict__ A, double2 *__restrict__ GA, int V) {
     const int site = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y;
-    if (site >= g.V) return;
-    const int k = canon_k(j);
-    if (off_class(k) < 2) return;
-    const M3<double2> a = A[(size_t)k * g.V + site];
-    const M3<double2> G = GA[(size_t)k * g.V + site];
+    if (site >= V || off_class(canon_k(j)) < 2) return;
+    const M3<double2> a = field_load<false>(A, j, V, site), G = field_load<false>(GA, j, V, site);
     M3<double2> out;
-    if (!project_vjp_fast(a, G, out)) project_vjp_general(a, G, out);
-    GA[(size_t)k * g.V + site] = out;
+    if (!project_vjp_fast(a, G, out)) {
+        const M3<double2> ac = a, Gc = G;  // in memory for the call only
+        M3<double2> o;
+        project_vjp_general(ac, Gc, o);
+        out = o;
+    }
+#pragma unroll
+    for (int e = 0; e < 9; e++) GA[((size_t)j * 9 + e) * V + site] = out.e[e];
 }
 
-// step 3a: G_{A_{d'}}(y) += sum_{mu notin supp d', s} (1/n) F_{mu,s}(y - s mu)^dagger G_{A_{d'+s mu}}(y - s mu)
-__global__ void k_dp_back(int nlow, const int *__restrict__ klist, int nk, const double2 *__restrict__ U,
-                          M3<double2> *GA, Geom g) {
+// step 3a, fields e of class n - 1 (list f), from the fields d of class n whose
+// path sums read them: for each mu outside e and both signs s, d = e + s mu,
+//   A_d(x) has F_{mu,s}(x) A_e(x + s mu) / n:  G_e(y) += F_{mu,s}(x)^dagger G_d(x) / n, x = y - s mu;
+// where d is not stored, -d = -e + mu is (s = -1) and has U_mu(x) A_e(y)^dagger / n,
+//   x = y + e - mu:                            G_e(y) += G_{-d}(x)^dagger U_mu(x) / n
+__global__ void k_path_back(int n, FieldList f, const double2 *__restrict__ A, double2 *__restrict__ GA,
+                            const __grid_constant__ Geom g) {
     const int site = blockIdx.x * blockDim.x + threadIdx.x;
-    if (site >= g.V || blockIdx.y >= (unsigned)nk) return;
-    const int kp = klist[blockIdx.y];
+    if (site >= g.V) return;
+    const int j = f.j[blockIdx.y], k = canon_k(j), V = g.V;
     int x[4];
-    SiteNb nb = site_nb(g, site, x);
-    M3<double2> acc = GA[(size_t)kp * g.V + site];
-    const double inv = 1.0 / (nlow + 1);
-    int p3 = 1;
-    for (int mu = 0; mu < 4; mu++, p3 *= 3) {
-        if (off_comp(kp, mu) != 0) continue;
+    const SiteNb nb = site_nb(g, site, x);
+    M3<double2> acc = m3_zero<double2>();
+#pragma unroll 1
+    for (int mu = 0; mu < 4; mu++) {
+        if (off_at(k, mu) != 0) continue;
+#pragma unroll 1
         for (int sg = -1; sg <= 1; sg += 2) {
-            const int k = kp + sg * p3;                  // d = d' + s mu
-            const int z = site + (sg > 0 ? nb.bw[mu] : nb.fw[mu]);  // z = y - s mu
-            // F_{mu,+}(z) = U_mu(z); F_{mu,-}(z) = U_mu(z - mu)^dagger = U_mu(y)^dagger
-            M3<double2> Fd;  // F^dagger
-            const double2 *u = U + ((size_t)(sg > 0 ? z : site) * 4 + mu) * 9;
-            M3<double2> Um;
-            for (int i = 0; i < 9; i++) Um.e[i] = u[i];
-            Fd = sg > 0 ? m3_dag(Um) : Um;
-            M3<double2> t = m3_mul(Fd, GA[(size_t)k * g.V + z]);
-            for (int i = 0; i < 9; i++) acc.e[i] = cadd(acc.e[i], cscale(t.e[i], inv));
+            const int kd = k + sg * p3_at(mu);
+            if (kd > 40) {
+                const int z = site + (sg > 0 ? nb.bw[mu] : nb.fw[mu]);
+                const M3<double2> Fd = sg > 0 ? field_load<true>(A, link_field(mu), V, z)
+                                              : field_load<false>(A, link_field(mu), V, site);
+                acc = m3_mad(acc, Fd, field_load<false>(GA, kd - 41, V, z));
+            } else {
+                const int z = site_at(kd, site, nb);  // y + e - mu
+                acc = m3_mad(acc, field_load<true>(GA, 39 - kd, V, z), field_load<false>(A, link_field(mu), V, z));
+            }
         }
     }
-    GA[(size_t)kp * g.V + site] = acc;
+    const double inv = 1.0 / n;
+#pragma unroll
+    for (int e = 0; e < 9; e++) {
+        double2 &o = GA[((size_t)j * 9 + e) * V + site];
+        o = make_double2(fma(acc.e[e].x, inv, o.x), fma(acc.e[e].y, inv, o.y));
+    }
 }
 
-// step 3b: link gradients (thread per site, mu = blockIdx.y), accumulated into dU [V][4][9]
-__global__ void k_link_grad(const M3<double2> *__restrict__ A, const M3<double2> *__restrict__ GA,
-                            double2 *__restrict__ dU, Geom g) {
+// step 3b: link gradients (thread per site, mu = blockIdx.y), accumulated into
+// dU [V][4][9]: every stored field with d_mu != 0 has the link as the first step
+// of one product
+__global__ void k_link_grad(const double2 *__restrict__ A, const double2 *__restrict__ GA, double2 *__restrict__ dU,
+                            const __grid_constant__ Geom g) {
     const int site = blockIdx.x * blockDim.x + threadIdx.x;
-    const int mu = blockIdx.y;
-    if (site >= g.V) return;
+    const int mu = blockIdx.y, V = g.V;
+    if (site >= V) return;
     int x[4];
-    SiteNb nb = site_nb(g, site, x);
-    const int xp = site + nb.fw[mu];
-    const int p3 = pow3(mu);
-    M3<double2> acc = m3_zero<double2>();
-    for (int k = 0; k < NOFF; k++) {
-        const int c = off_comp(k, mu);
-        if (c == 0) continue;
-        const int n = off_class(k);
-        if (c > 0) {
-            // A_d(x) with d_mu = +1: first step U_mu(x)
-            const M3<double2> G = GA[(size_t)k * g.V + site];
-            if (n == 1) acc = m3_add(acc, G);
-            else {
-                M3<double2> t = m3_mul(G, m3_dag(A[(size_t)(k - p3) * g.V + xp]));
-                for (int i = 0; i < 9; i++) acc.e[i] = cadd(acc.e[i], cscale(t.e[i], 1.0 / n));
+    const SiteNb nb = site_nb(g, site, x);
+    int xp = site;
+#pragma unroll
+    for (int m = 0; m < 4; m++)
+        if (m == mu) xp += nb.fw[m];
+    M3<double2> sum = field_load<false>(GA, link_field(mu), V, site);
+    auto terms = [&](int n, M3<double2> &acc) {
+#pragma unroll 1
+        for (int j = 0; j < NCANON; j++) {
+            const int k = canon_k(j), c = off_at(k, mu);
+            if (c == 0 || off_class(k) != n) continue;
+            if (c > 0) {
+                // A_d(x) has U_mu(x) R: G_d(x) R^dagger
+                const PathRest r = path_rest(k, mu, 1, site, nb);
+                const M3<double2> Rd = r.dag ? field_load<false>(A, r.j, V, r.site) : field_load<true>(A, r.j, V, r.site);
+                acc = m3_mad(acc, field_load<false>(GA, j, V, site), Rd);
+            } else {
+                // A_d(x + mu) has U_mu(x)^dagger A_{d + mu}(x): A_{d + mu}(x) G_d(x + mu)^dagger
+                const int jr = k + p3_at(mu) - 41;  // stored: d's last component stays
+                acc = m3_mad(acc, field_load<false>(A, jr, V, site), field_load<true>(GA, j, V, xp));
             }
-        } else {
-            // A_d(x+mu) with d_mu = -1: first step U_mu(x)^dagger
-            const M3<double2> G = GA[(size_t)k * g.V + xp];
-            if (n == 1) acc = m3_add(acc, m3_dag(G));
-            else {
-                M3<double2> t = m3_mul(A[(size_t)(k + p3) * g.V + site], m3_dag(G));
-                for (int i = 0; i < 9; i++) acc.e[i] = cadd(acc.e[i], cscale(t.e[i], 1.0 / n));
-            }
+        }
+    };
+#pragma unroll 1
+    for (int n = 2; n <= 4; n++) {
+        M3<double2> acc = m3_zero<double2>();
+        terms(n, acc);
+        const double inv = 1.0 / n;
+#pragma unroll
+        for (int e = 0; e < 9; e++) {
+            sum.e[e].x = fma(acc.e[e].x, inv, sum.e[e].x);
+            sum.e[e].y = fma(acc.e[e].y, inv, sum.e[e].y);
         }
     }
     double2 *o = dU + ((size_t)site * 4 + mu) * 9;
-    for (int i = 0; i < 9; i++) o[i] = cadd(o[i], acc.e[i]);
+#pragma unroll
+    for (int e = 0; e < 9; e++) o[e] = cadd(o[e], sum.e[e]);
 }
 
 }  // namespace
 
+// work space: path sums and gradients of the 40 stored fields (11,520 bytes per
+// site), stream-ordered from the context's pool.  12^4 (FP64 operations bound
+// every step): path sums 0.46 ms (0.93 over all 80 offsets), hop gradients 0.73
+// (3.13), projection 1.51 (8.37), path sums backwards 0.48 (0.98), links 0.56
+// (1.16)
 bri_status bri_force_impl(bri_ctx *ctx, double2 *dU, const double2 *chi, const double2 *psi, cudaStream_t s) {
-    const Geom g = ctx->g;
-    const size_t V = g.V;
-    M3<double2> *A = nullptr, *GA = nullptr;
-    int *klist = nullptr;
-    BRI_TRY_CUDA(ctx, cudaMallocAsync((void **)&A, sizeof(M3<double2>) * NOFF * V, s));
-    BRI_TRY_CUDA(ctx, cudaMallocAsync((void **)&GA, sizeof(M3<double2>) * NOFF * V, s));
-    BRI_TRY_CUDA(ctx, cudaMallocAsync((void **)&klist, sizeof(int) * NOFF, s));
-    BRI_TRY_CUDA(ctx, cudaMemsetAsync(GA, 0, sizeof(M3<double2>) * NOFF * V, s));
-    int hk[NOFF], start[6] = {0}, cnt = 0;
-    for (int n = 1; n <= 4; n++) {
-        start[n] = cnt;
-        for (int k = 0; k < NOFF; k++)
-            if (off_class(k) == n) hk[cnt++] = k;
-    }
-    start[5] = cnt;
-    BRI_TRY_CUDA(ctx, cudaMemcpyAsync(klist, hk, sizeof(int) * cnt, cudaMemcpyHostToDevice, s));
-    BRI_RETURN_IF(bri_dp_levels(ctx, A, klist, start, s));
-    const int T = 128;
-    const unsigned nb = (unsigned)((V + T - 1) / T);
-    k_hop_grad<<<dim3(nb, NCANON), T, 0, s>>>(chi, psi, GA, g);
-    BRI_LAUNCHED(ctx);
-    k_project_vjp<<<dim3(nb, NCANON), T, 0, s>>>(A, GA, g);
-    BRI_LAUNCHED(ctx);
-    for (int nlow = 3; nlow >= 1; nlow--) {
-        k_dp_back<<<dim3(nb, start[nlow + 1] - start[nlow]), T, 0, s>>>(nlow, klist + start[nlow],
-                                                                        start[nlow + 1] - start[nlow], ctx->U, GA, g);
+    const Geom &g = ctx->g;
+    const size_t fields = (size_t)9 * NCANON * g.V;
+    double2 *A = nullptr;
+    BRI_TRY_CUDA(ctx, cudaMallocFromPoolAsync((void **)&A, sizeof(double2) * 2 * fields, ctx->pool, s));
+    double2 *GA = A + fields;
+    auto run = [&]() -> bri_status {
+        BRI_RETURN_IF(bri_path_sums(ctx, A, s));
+        const int T = 128;
+        const unsigned nb = (unsigned)((g.V + T - 1) / T);
+        k_hop_grad<<<dim3(nb, NCANON), T, 0, s>>>(chi, psi, GA, g);
         BRI_LAUNCHED(ctx);
-    }
-    k_link_grad<<<dim3(nb, 4), T, 0, s>>>(A, GA, dU, g);
-    BRI_LAUNCHED(ctx);
+        k_project_vjp<<<dim3(nb, NCANON), T, 0, s>>>(A, GA, g.V);
+        BRI_LAUNCHED(ctx);
+        for (int n = 4; n >= 2; n--) {
+            const FieldList f = fields_of_class(n - 1);
+            k_path_back<<<dim3(nb, f.n), T, 0, s>>>(n, f, A, GA, g);
+            BRI_LAUNCHED(ctx);
+        }
+        k_link_grad<<<dim3(nb, 4), T, 0, s>>>(A, GA, dU, g);
+        BRI_LAUNCHED(ctx);
+        return BRI_OK;
+    };
+    const bri_status st = run();
     BRI_TRY_CUDA(ctx, cudaFreeAsync(A, s));
-    BRI_TRY_CUDA(ctx, cudaFreeAsync(GA, s));
-    BRI_TRY_CUDA(ctx, cudaFreeAsync(klist, s));
-    return BRI_OK;
+    return st;
 }

@@ -1,0 +1,71 @@
+// Fixed-point copies of the FP64 hopping fields and spinors (see dslash_fx.cu
+// for the format and its bounds).
+#pragma once
+#include "common.cuh"
+
+namespace bri {
+
+constexpr int FX_BAD = 1 << 20;     // block exponent of a site with an infinity or a NaN
+constexpr int FX_ZERO = -(1 << 20);  // ... of a site that is zero
+constexpr int FX_WB = 62, FX_PB = 60;  // fraction bits of links and spinors
+constexpr int FX_AB = FX_WB + FX_PB - 64;  // of the row sums
+// v 2^sh rounded to an integer (|v| 2^sh < 2^63), by shifts: conversions run on
+// the FP64 pipe
+BRI_D long long fx_int(double v, int sh) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)(bits >> 52) & 0x7ff;
+    const unsigned long long m = (bits & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+    const int s = max(e, 1) - 1075 + sh, r = min(-s, 63);
+    const long long f = (long long)(s >= 0 ? m << s : (m + ((1ull << r) >> 1)) >> r);
+    return (long long)bits < 0 ? -f : f;
+}
+BRI_D int4 fx_split(double re, double im, int sh) {
+    // the low word is never INT_MIN, so that limbs can be negated
+    const long long a = fx_int(re, sh), b = fx_int(im, sh);
+    int4 v;
+    v.y = (int)a;
+    v.x = (int)((a - v.y) >> 32);
+    v.w = (int)b;
+    v.z = (int)((b - v.w) >> 32);
+    if (v.y == (int)0x80000000) v.y++;
+    if (v.w == (int)0x80000000) v.w++;
+    return v;
+}
+BRI_D unsigned abs_hi(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+
+// largest |row|^2, |column|^2 of a field matrix, as the high word of a double
+// (NaN and infinities come out largest)
+BRI_D unsigned norm_hi(const double2 w[9]) {
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        m = max(m, abs_hi(cnorm2(w[3 * i]) + cnorm2(w[3 * i + 1]) + cnorm2(w[3 * i + 2])));
+        m = max(m, abs_hi(cnorm2(w[i]) + cnorm2(w[3 + i]) + cnorm2(w[6 + i])));
+    }
+    return m;
+}
+constexpr unsigned FX_ONE = 0x3ff00010u;  // 1 + 2^-16: a unitary matrix and its rounding
+// exponent we: norms are at most 2^we
+BRI_D int fx_we(unsigned hi) {
+    if (hi <= FX_ONE) return 0;
+    return ((int)(hi >> 20) - 1022 + 1) >> 1;  // |.|^2 < 2^(exponent field - 1022)
+}
+
+// limb copies are stored in blocks of 32 sites, [..][Vp/32][entries][32] with Vp
+// = V rounded up to 32: the entries of a site lie at fixed offsets from its first
+BRI_D size_t fx_at(int site, int entries) { return (size_t)(site >> 5) * (32 * entries) + (site & 31); }
+
+// the limbs of one field matrix of site s (o: the field's start); info[1] = 1 if
+// it does not fit
+BRI_D void fx_store(const double2 w[9], int4 *o, int site, unsigned *info) {
+    const int we = fx_we(info[0]);
+    if (we > 400 || norm_hi(w) > max(info[0], FX_ONE)) {  // infinities, NaN or huge entries
+        info[1] = 1;
+        return;
+    }
+    o += fx_at(site, 9);
+#pragma unroll
+    for (int e = 0; e < 9; e++) o[32 * e] = fx_split(w[e].x, w[e].y, FX_WB - we);
+}
+
+}  // namespace bri

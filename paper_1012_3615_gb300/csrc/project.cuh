@@ -566,7 +566,12 @@ BRI_D bool project_fast(const M3<double2> &A, M3<double2> &Y, ProjectionSeed &sd
 BRI_D M3<double2> project_su3(const M3<double2> &A) {
     M3<double2> Y;
     ProjectionSeed sd;
-    if (!project_fast(A, Y, sd)) project_su3_general(A, Y, nullptr);
+    if (!project_fast(A, Y, sd)) {
+        const M3<double2> a = A;  // in memory for the call only
+        M3<double2> y;
+        project_su3_general(a, y, nullptr);
+        Y = y;
+    }
     return Y;
 }
 
