@@ -514,8 +514,10 @@ bri_status bri_dslash_fx(bri_ctx *ctx, const Geom &g, void *out, const void *in,
     k_fx_spinor<<<dim3((unsigned)((n + 127) / 128), (unsigned)nrhs), 128, 0, s>>>((const double2 *)in, P, ex, g.V,
                                                                                   first, n, skip);
     BRI_LAUNCHED(ctx);
-    // splits of the hop list, so that the 608 schedulers have two warps or more
-    const long long warps = 2ll * ((g.s1 - g.s0 + 31) / 32) * nrhs;
+    // splits of the hop list, so that the 608 schedulers have two warps or more;
+    // by the lattice alone, so that a right-hand side gives the same bits alone, in
+    // a batch and on a range of sites
+    const int warps = 2 * ((g.V + 31) / 32);
     const int S = warps >= 2432 ? 1 : warps >= 1216 ? 2 : 4;
     auto launch = g.clov64 ? (S == 1 ? fx_launch<1, true> : S == 2 ? fx_launch<2, true> : fx_launch<4, true>)
                            : (S == 1 ? fx_launch<1, false> : S == 2 ? fx_launch<2, false> : fx_launch<4, false>);

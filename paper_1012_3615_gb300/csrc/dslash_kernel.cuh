@@ -313,14 +313,15 @@ BRI_D void pair_body_s(const float2 cf[12], const M3<float2> &W, const float2 p[
 
 // FP32 stencil over the 40 (d, -d) pairs as a compact loop.  PF = true also
 // prefetches the two links of the next pair into L2 (the links stream from DRAM;
-// the neighbour spinors mostly hit L1/L2).
-template <bool PF, int BODY, class LL>
+// the neighbour spinors mostly hit L1/L2).  RANGE: the pairs [t0, t1) only.
+template <bool PF, int BODY, bool RANGE = false, class LL>
 BRI_D void f32_hops(const LL &ll, const float2 *__restrict__ in, int site, const SiteNb &nb, float rsign,
-                    const Geom &g, AccF &acc) {
+                    const Geom &g, AccF &acc, int t0 = 0, int t1 = 0) {
+    static_assert(!RANGE || BODY == 2 || BODY == 3, "ranges of pairs: the pair-combined forms");
     if constexpr (BODY == 2 || BODY == 3) {
         // pair-combined body (pair_body), links of the next pair prefetched into L2
 #pragma unroll 1
-        for (int t = 0; t < g.nhop; t++) {
+        for (int t = RANGE ? t0 : 0; t < (RANGE ? t1 : g.nhop); t++) {
             if (PF && t + 1 < g.nhop) {
                 const HopArg hp = g.hop[t + 1];
                 int pyf, pyb;
@@ -429,17 +430,17 @@ BRI_D void f32_hops(const LL &ll, const float2 *__restrict__ in, int site, const
 // per-site part of every link address is computed once, each field adds
 // j VP NQ, and the neighbours of the next pair (found for its L2 prefetch)
 // are carried into the next iteration instead of being recomputed.
-template <class LL>
+template <bool RANGE = false, class LL>
 BRI_D void f32_hops_lean(const LL &ll, const float2 *__restrict__ in, int site, const SiteNb &nb, float rsign,
-                         const Geom &g, AccF &acc) {
-    if (g.nhop == 0) return;
+                         const Geom &g, AccF &acc, int t0 = 0, int t1 = 0) {
+    if (RANGE ? t0 >= t1 : g.nhop == 0) return;
     const long long sc = ll.cidx(site);
     int yf, yb;
     float phf, phb;
-    hop_nb(g.hop[0].dm, site, nb, yf, phf, yb, phb);
+    hop_nb(g.hop[RANGE ? t0 : 0].dm, site, nb, yf, phf, yb, phb);
     long long bc = ll.cidx(yb);
 #pragma unroll 1
-    for (int t = 0; t < g.nhop; t++) {
+    for (int t = RANGE ? t0 : 0; t < (RANGE ? t1 : g.nhop); t++) {
         const int cyf = yf, cyb = yb;
         const float cphf = phf, cphb = phb;
         const long long cbc = bc;
@@ -838,6 +839,100 @@ __global__ void __maxnreg__(128) k_dslash_r128(int mode, LL ll, const typename L
                                                const int *__restrict__ skip) {
     dslash_body<LL, 5, false>(mode, ll, in, out, g, diag, skip);
 }
+
+// The pair loops of variants 5 and 9 with the hop list of a site split over S
+// warps (4 warps per block, 4 / S groups of 32 sites): a lattice of few sites
+// otherwise leaves most of the 608 schedulers with one warp or none.  The
+// site's sum is that of SPLIT_PARTS partial sums over quarters of the list,
+// added in order, for every S, so that a right-hand side gives the same bits
+// alone, in a batch and on a range of sites; a warp takes SPLIT_PARTS / S of
+// them one after the other.
+constexpr int SPLIT_PARTS = 4;
+template <class LL, int VAR, bool CLOV, int S>
+BRI_D void dslash_split_body(int mode, const LL &ll, const float2 *__restrict__ in, float2 *__restrict__ out,
+                             const Geom &g, double diag, const int *__restrict__ skip) {
+    constexpr int SPB = 128 / S, PER = SPLIT_PARTS / S;
+    __shared__ float2 sm[(1 + (S - 1) * PER) * 12 * SPB];  // the first warp's sum, then the others' parts
+    const int nblk = (g.s1 - g.s0 + SPB - 1) / SPB;
+    const int nr = (int)gridDim.x / nblk;
+    const int rhs = (int)blockIdx.x % nr;
+    if (skip && skip[rhs]) return;
+    const int warp = (int)threadIdx.x >> 5, split = warp % S, at = (warp / S) * 32 + ((int)threadIdx.x & 31);
+    const int want = g.s0 + ((int)blockIdx.x / nr) * SPB + at;
+    const bool active = want < g.s1;
+    const int site = active ? want : g.s1 - 1;
+    const size_t off = (size_t)rhs * g.V * 12;
+    in += off;
+    out += off;
+    // site_nb with divisions in FP32, exact for these few sites: its integer
+    // divisions would be 4% of a quarter of the list
+    SiteNb nb;
+    {
+        int s = site, stride = 1;
+#pragma unroll
+        for (int mu = 0; mu < 4; mu++) {
+            const int L = g.L[mu], q = (int)(((float)s + 0.5f) * __frcp_rn((float)L)), x = s - q * L;
+            const bool top = x == L - 1, bot = x == 0;
+            s = q;
+            nb.fw[mu] = top ? -(L - 1) * stride : stride;
+            nb.bw[mu] = bot ? (L - 1) * stride : -stride;
+            nb.sfw[mu] = top ? (float)g.bc[mu] : 1.f;
+            nb.sbw[mu] = bot ? (float)g.bc[mu] : 1.f;
+            stride *= L;
+        }
+    }
+    const float rsign = mode == 1 ? -1.f : 1.f;
+#pragma unroll 1
+    for (int p = 0; p < PER; p++) {
+        const int part = split * PER + p, t0 = part * g.nhop / SPLIT_PARTS, t1 = (part + 1) * g.nhop / SPLIT_PARTS;
+        AccF acc;
+#pragma unroll
+        for (int i = 0; i < 12; i++) acc.a[i] = acc.ai[i] = make_float2(0.f, 0.f);
+        if constexpr (VAR == 9) f32_hops_lean<true>(ll, in, site, nb, rsign, g, acc, t0, t1);
+        else f32_hops<true, 2, true>(ll, in, site, nb, rsign, g, acc, t0, t1);
+        const int slot = split == 0 ? 0 : 1 + part - PER;
+#pragma unroll
+        for (int i = 0; i < 12; i++) {
+            float2 &z = sm[(slot * 12 + i) * SPB + at];
+            const float2 v = make_float2(acc.a[i].x - acc.ai[i].y, acc.a[i].y + acc.ai[i].x);
+            z = split == 0 && p > 0 ? cadd(z, v) : v;
+        }
+    }
+    __syncthreads();
+    if (split || !active) return;
+    AccF acc;
+#pragma unroll
+    for (int i = 0; i < 12; i++) {
+        acc.a[i] = sm[i * SPB + at];
+        acc.ai[i] = make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int w = 1; w <= (S - 1) * PER; w++)
+#pragma unroll
+        for (int i = 0; i < 12; i++) acc.a[i] = cadd(acc.a[i], sm[(w * 12 + i) * SPB + at]);
+    dslash_finish<float2, CLOV>(mode, in, out, site, g, diag, acc);
+}
+template <class LL, int VAR, bool CLOV, int S>
+__global__ void __launch_bounds__(128) k_dslash_split(int mode, LL ll, const float2 *__restrict__ in,
+                                                      float2 *__restrict__ out, Geom g, double diag,
+                                                      const int *__restrict__ skip) {
+    dslash_split_body<LL, VAR, CLOV, S>(mode, ll, in, out, g, diag, skip);
+}
+template <class LL, int S>
+__global__ void __maxnreg__(128) k_dslash_split_r128(int mode, LL ll, const float2 *__restrict__ in,
+                                                     float2 *__restrict__ out, Geom g, double diag,
+                                                     const int *__restrict__ skip) {
+    dslash_split_body<LL, 5, false, S>(mode, ll, in, out, g, diag, skip);
+}
+// Lattices that are summed in parts, and the warps per group for a launch of so
+// many groups.  Measured (us; FP32 full, FP32 2-row, FP16 2-row): 8^4, one
+// right-hand side: one thread a site 31, 35, 34, four warps 12.9; three: 31, 35,
+// 35 -> 18.7; twelve: 55, 56, 58 -> 56, 56, 57.  Above 128 groups the parts cost
+// twelve right-hand sides 3-11% (12^4: 224 -> 249) for a quarter of one's time,
+// so the line lies there; up to 1,600 groups of a launch four warps a site are
+// the faster form of the two, above it one (8^4, 24: 109 against 100 in one part).
+inline bool dslash_in_parts(int V) { return V <= 128 * 32; }
+inline int dslash_splits(long long groups) { return groups <= 1600 ? 4 : 1; }
 
 // launch variant 10: the bulk-copy link pipeline.  Needs s0 a multiple of 32
 // (every warp covers one 32-site block); lanes past s1 compute on the range's
@@ -1393,6 +1488,31 @@ void dslash_launch(int mode, const LL &ll, const void *in, void *out, int nrhs, 
                 dslash_launch(mode, ll, (const char *)in + r0 * field, (char *)out + r0 * field, nr, g, diag,
                               skip ? skip + r0 : nullptr, threads, s);
             }
+            return;
+        }
+    }
+    if constexpr (sizeof(T) == 8) {
+        // pair loops on small lattices: the split form
+        const int v = threads >> 11;
+        if (dslash_in_parts(g.V) && (g.clov64 || v == 5 || v == 6 || v == 9)) {
+            constexpr int VF = LL::COMP == BRI_LINK_8PARAM || LL::FULL32 ? 5 : 9;
+            auto launch = [&](auto S, auto C) {
+                constexpr int spb = 128 / decltype(S)::value;
+                const dim3 grid((unsigned)((g.s1 - g.s0 + spb - 1) / spb) * (unsigned)nrhs);
+                if constexpr (LL::COMP == BRI_LINK_8PARAM && !decltype(C)::value)
+                    k_dslash_split_r128<LL, decltype(S)::value><<<grid, 128, 0, s>>>(mode, ll, (const T *)in, (T *)out,
+                                                                                    g, diag, skip);
+                else
+                    k_dslash_split<LL, VF, decltype(C)::value, decltype(S)::value>
+                        <<<grid, 128, 0, s>>>(mode, ll, (const T *)in, (T *)out, g, diag, skip);
+            };
+            const int S = dslash_splits((long long)((g.s1 - g.s0 + 31) / 32) * nrhs);
+            auto with = [&](auto C) {
+                if (S == 4) launch(std::integral_constant<int, 4>{}, C);
+                else launch(std::integral_constant<int, 1>{}, C);
+            };
+            if (g.clov64) with(std::true_type{});
+            else with(std::false_type{});
             return;
         }
     }

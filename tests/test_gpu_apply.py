@@ -417,3 +417,29 @@ def test_tuner_choice_is_correct_and_cached(gpu, tmp_path, monkeypatch):
     op3 = Brillouin(L, bc)
     op3.build_hops(torch.as_tensor(U, device=gpu), prec="f32", comp="2row")
     assert op3.threads("f32", 3) == 11 * 2048 + 64
+
+
+@pytest.mark.parametrize("prec,comp", [("f32", "full"), ("f32", "2row"), ("f32", "8param"), ("f16", "full"),
+                                       ("f16", "2row"), ("f16", "8param")])
+@pytest.mark.parametrize("L,nrhs", [((3, 3, 3, 3), 1), ((8, 8, 8, 8), 2), ((8, 8, 8, 8), 13), ((7, 4, 12, 12), 1), ((3, 11, 5, 25), 1)])
+def test_parts_of_the_hop_list(gpu, prec, comp, L, nrhs):
+    """Lattices of up to 128 groups of 32 sites sum a site in four parts, on four
+    warps or (from 1,600 groups of a launch on) one: D, D^dagger, the overlap
+    kernel and the clover operator against the one-part launch shape (variant
+    4), with equal bits for a right-hand side alone and in the batch."""
+    U = torch.as_tensor(synth.random_su3_links(L, 0.4, 61), device=gpu)
+    x = synth.gaussian_spinor_torch(L, nrhs, 62, device=gpu).to(torch.complex64)
+    op = Brillouin(L, AP)
+    op.build_hops(U, prec=prec, comp=comp)
+    calls = [lambda: op.apply(x, 0.1, prec=prec), lambda: op.apply(x, 0.1, dagger=True, prec=prec),
+             lambda: op.overlap_kernel(x, 1.0, prec=prec)]
+    got = [c() for c in calls]
+    assert torch.equal(got[0][-1:], op.apply(x[-1:].contiguous(), 0.1, prec=prec))
+    op.set_threads(prec, nrhs, 4 * 2048 + 128)
+    for g, c in zip(got, calls):
+        ref = c()
+        assert torch.abs(g - ref).max() <= 1e-6 * torch.abs(ref).max()
+    op.set_clover(1.0)
+    clov = op.apply(x, 0.1, prec=prec)
+    C64 = op.apply(x.to(torch.complex128), 0.1) - (op.set_clover(0.0) or op.apply(x.to(torch.complex128), 0.1))
+    assert torch.abs(clov - got[0] - C64).max() <= 1e-6 * torch.abs(clov).max()
