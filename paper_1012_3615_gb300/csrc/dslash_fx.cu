@@ -462,7 +462,7 @@ bri_status bri_fx_reserve(bri_ctx *ctx) {
             ctx->hopsfx = nullptr;
         }
     }
-    if (!ctx->fxinfo) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->fxinfo, 2 * sizeof(unsigned)));
+    if (!ctx->fxinfo) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->fxinfo, 3 * sizeof(unsigned)));
     if (!ctx->pool) {
         cudaMemPoolProps pp{};
         pp.allocType = cudaMemAllocationTypePinned;

@@ -332,7 +332,7 @@ __global__ void k_link_grad(const double2 *__restrict__ A, const double2 *__rest
 
 // work space: path sums and gradients of the 40 stored fields (11,520 bytes per
 // site), stream-ordered from the context's pool.  12^4 (FP64 operations bound
-// every step): path sums 0.46 ms (0.93 over all 80 offsets), hop gradients 0.73
+// every step but the first): path sums 0.2 ms (0.93 over all 80 offsets in FP64), hop gradients 0.73
 // (3.13), projection 1.51 (8.37), path sums backwards 0.48 (0.98), links 0.56
 // (1.16)
 bri_status bri_force_impl(bri_ctx *ctx, double2 *dU, const double2 *chi, const double2 *psi, cudaStream_t s) {

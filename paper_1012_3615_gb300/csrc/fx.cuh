@@ -33,6 +33,27 @@ BRI_D int4 fx_split(double re, double im, int sh) {
 }
 BRI_D unsigned abs_hi(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 
+// f 2^sh, rounded to nearest even, by integer operations
+BRI_D double fx_double(long long f, int sh) {
+    const unsigned long long u = f < 0 ? 0ull - (unsigned long long)f : (unsigned long long)f;
+    if (u == 0) return 0.0;
+    const int lz = __clzll((long long)u);
+    const unsigned long long m = u << lz;  // leading one at bit 63
+    const unsigned long long r = (m + 0x3ffull + ((m >> 11) & 1ull)) >> 11;  // 53 bits; 2^53 when it rounds up
+    const bool up = r < (1ull << 52);  // m + ... ran over 2^64
+    const unsigned long long q = up ? 1ull << 52 : r;
+    const unsigned long long e = (unsigned long long)(1023 + 63 - lz + sh + (up ? 1 : 0) - 1);
+    return __longlong_as_double((long long)((e << 52) + q + (f < 0 ? 1ull << 63 : 0ull)));
+}
+// two signed limbs of an integer (the low one never INT_MIN: limbs can be negated)
+BRI_D int2 fx_limbs(long long f) {
+    int lo = (int)f;
+    const int hi = (int)((f - lo) >> 32);
+    if (lo == (int)0x80000000) lo++;
+    return make_int2(hi, lo);
+}
+BRI_D long long fx_join(int hi, int lo) { return (long long)hi * (1ll << 32) + lo; }
+
 // largest |row|^2, |column|^2 of a field matrix, as the high word of a double
 // (NaN and infinities come out largest)
 BRI_D unsigned norm_hi(const double2 w[9]) {

@@ -12,8 +12,8 @@
 // instead of 208.  Level n reads level n-1 at neighbouring sites, so each level
 // is one launch over (site, field), in the fields' own array: the projection
 // then replaces each path sum by its field in place, so the build holds no
-// second copy (5,760 bytes per site instead of 17,424).  16^3x32: path sums 5.6
-// -> 2.7 ms, whole build 10.4 -> 7.7 ms; both steps are bound by FP64 operations.
+// second copy (5,760 bytes per site instead of 17,424).  16^3x32: 80 offsets in
+// FP64 5.6 ms, 40 in FP64 2.7, 40 in fixed point (below) 0.9.
 #include <cuda_fp16.h>
 
 #include "ctx.h"
@@ -26,67 +26,207 @@ using namespace bri;
 
 namespace {
 
+// ---- path sums in fixed point ---------------------------------------------------
+// The matrix products run on the integer pipe (see dslash_fx.cu: three
+// 32 x 32 -> 64-bit multiply-adds for a product, against 64 FP32 instruction
+// slots for one FP64 operation): entries as two limbs of v 2^61, rows and
+// columns of norm at most 1, so that with hi 2^32 + lo the sums of an entry's
+// cross products stay below 2 sqrt(6) 2^60 < 2^63 and those of its high
+// products, over the n terms of a level, below n sqrt(6) 2^58.  A level's sum
+// is scaled by 2^-1, 2^-2, 2^-2 (n = 2, 3, 4) instead of 1/n.  Known to 2^-57.
+// 16^3x32: 0.90 ms (FP64 products: 2.7), the whole build 5.1 ms (7.7), of which
+// the projection takes 3.7.
+// Links whose rows and columns are not of norm 1 to 2^-16 (only their user
+// knows what they are) take the FP64 form: info[0] and info[2] hold the largest
+// and the smallest norm, and every kernel takes the same branch.
+constexpr int PS_B = 61;
+BRI_D bool paths_fixed(const unsigned *info) { return info[0] <= FX_ONE && ~info[2] >= 0x3fefffe0u; }
+
+// smallest |row|^2, |column|^2 of a matrix, as the high word of a double
+BRI_D unsigned norm_lo(const double2 w[9]) {
+    unsigned m = 0xffffffffu;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        m = min(m, abs_hi(cnorm2(w[3 * i]) + cnorm2(w[3 * i + 1]) + cnorm2(w[3 * i + 2])));
+        m = min(m, abs_hi(cnorm2(w[i]) + cnorm2(w[3 + i]) + cnorm2(w[6 + i])));
+    }
+    return m;
+}
+// info[0]: largest norm of the links (the other fields are unitary), info[1]: 1
+// if a field matrix does not fit its limbs, info[2]: complement of the smallest
+__global__ void k_link_norms(const double2 *__restrict__ U, int n, unsigned *info) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned m = 0, l = 0;
+    if (i < n) {
+        double2 w[9];
+#pragma unroll
+        for (int e = 0; e < 9; e++) w[e] = U[(size_t)i * 9 + e];
+        m = norm_hi(w);
+        l = ~norm_lo(w);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    l = __reduce_max_sync(0xffffffffu, l);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(info, m);
+        atomicMax(info + 2, l);
+    }
+}
+
+template <bool DAG> BRI_D M3<int4> field_load_fx(const double2 *__restrict__ A, int j, int V, int site) {
+    const int4 *p = reinterpret_cast<const int4 *>(A);
+    M3<int4> m;
+#pragma unroll
+    for (int r = 0; r < 3; r++)
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            const int4 v = p[((size_t)j * 9 + (DAG ? 3 * c + r : 3 * r + c)) * V + site];
+            m.e[3 * r + c] = DAG ? make_int4(v.x, v.y, -v.z, -v.w) : v;
+        }
+    return m;
+}
+// sum += F M, entry (i, j) at sum[2 (3 i + j)], in units of 2^-58
+BRI_D void fx_mad(const M3<int4> &F, const M3<int4> &M, long long sum[18]) {
+    constexpr unsigned long long up = (1ull << 63) + (1ull << 31);  // as in dslash_fx.cu: no sign word, rounded
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            long long re = sum[2 * (3 * i + j)] - (1ll << 31), im = sum[2 * (3 * i + j) + 1] - (1ll << 31);
+            unsigned long long br = up, bi = up;
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const int4 w = F.e[3 * i + k], q = M.e[3 * k + j];
+                re += (long long)w.x * q.x;
+                im += (long long)w.x * q.z;
+                br += (long long)w.x * q.y;
+                bi += (long long)w.x * q.w;
+                br += (long long)w.y * q.x;
+                bi += (long long)w.y * q.z;
+                re += (long long)-w.z * q.z;
+                im += (long long)w.z * q.x;
+                br += (long long)-w.z * q.w;
+                bi += (long long)w.z * q.y;
+                br += (long long)-w.w * q.z;
+                bi += (long long)w.w * q.x;
+            }
+            sum[2 * (3 * i + j)] = re + (long long)(br >> 32);
+            sum[2 * (3 * i + j) + 1] = im + (long long)(bi >> 32);
+        }
+}
+// the path sum of an off-axis field as an FP64 matrix: from limbs, or as it stands
+BRI_D M3<double2> path_load(const double2 *__restrict__ A, int j, int V, int site, bool fixed) {
+    if (!fixed) return field_load<false>(A, j, V, site);
+    const int4 *p = reinterpret_cast<const int4 *>(A);
+    M3<double2> m;
+#pragma unroll
+    for (int e = 0; e < 9; e++) {
+        const int4 v = p[((size_t)j * 9 + e) * V + site];
+        m.e[e] = make_double2(fx_double(fx_join(v.x, v.y), -PS_B), fx_double(fx_join(v.z, v.w), -PS_B));
+    }
+    return m;
+}
+
 // level n >= 2 of the path sums, field f.j[blockIdx.y]
-__global__ void k_path_level(int n, FieldList f, double2 *__restrict__ A, const __grid_constant__ Geom g) {
+__global__ void k_path_level(int n, FieldList f, double2 *__restrict__ A, const unsigned *__restrict__ info,
+                             const __grid_constant__ Geom g) {
     const int site = blockIdx.x * blockDim.x + threadIdx.x;
     if (site >= g.V) return;
-    const int j = f.j[blockIdx.y], k = canon_k(j);
+    const int j = f.j[blockIdx.y], k = canon_k(j), V = g.V;
     int x[4];
     const SiteNb nb = site_nb(g, site, x);
+    if (paths_fixed(info)) {
+        long long sum[18];
+#pragma unroll
+        for (int i = 0; i < 18; i++) sum[i] = 0;
+#pragma unroll 1
+        for (int mu = 0; mu < 4; mu++) {
+            const int c = off_at(k, mu);
+            if (c == 0) continue;
+            const PathRest r = path_rest(k, mu, c, site, nb);
+            const M3<int4> F = c > 0 ? field_load_fx<false>(A, link_field(mu), V, site)
+                                     : field_load_fx<true>(A, link_field(mu), V, site + nb.bw[mu]);
+            const M3<int4> M = r.dag ? field_load_fx<true>(A, r.j, V, r.site) : field_load_fx<false>(A, r.j, V, r.site);
+            fx_mad(F, M, sum);
+        }
+        int4 *o = reinterpret_cast<int4 *>(A);
+        const int sh = PS_B - 58 - (n == 2 ? 1 : 2);
+#pragma unroll
+        for (int e = 0; e < 9; e++) {
+            const int2 re = fx_limbs(sum[2 * e] << sh), im = fx_limbs(sum[2 * e + 1] << sh);
+            o[((size_t)j * 9 + e) * V + site] = make_int4(re.x, re.y, im.x, im.y);
+        }
+        return;
+    }
     M3<double2> acc = m3_zero<double2>();
 #pragma unroll 1
     for (int mu = 0; mu < 4; mu++) {
         const int c = off_at(k, mu);
         if (c == 0) continue;
         const PathRest r = path_rest(k, mu, c, site, nb);
-        const M3<double2> F = c > 0 ? field_load<false>(A, link_field(mu), g.V, site)
-                                    : field_load<true>(A, link_field(mu), g.V, site + nb.bw[mu]);
-        const M3<double2> M = r.dag ? field_load<true>(A, r.j, g.V, r.site) : field_load<false>(A, r.j, g.V, r.site);
+        const M3<double2> F = c > 0 ? field_load<false>(A, link_field(mu), V, site)
+                                    : field_load<true>(A, link_field(mu), V, site + nb.bw[mu]);
+        const M3<double2> M = r.dag ? field_load<true>(A, r.j, V, r.site) : field_load<false>(A, r.j, V, r.site);
         acc = m3_mad(acc, F, M);
     }
     const double inv = 1.0 / n;
 #pragma unroll
-    for (int e = 0; e < 9; e++) A[((size_t)j * 9 + e) * g.V + site] = cscale(acc.e[e], inv);
+    for (int e = 0; e < 9; e++) A[((size_t)j * 9 + e) * V + site] = cscale(acc.e[e], inv);
 }
 
-// level 1: the links, site-fastest
-__global__ void k_path_links(const double2 *__restrict__ U, double2 *__restrict__ A, int V) {
+// level 1: the links, site-fastest, as limbs or as they are
+__global__ void k_path_links(const double2 *__restrict__ U, double2 *__restrict__ A, int V,
+                             const unsigned *__restrict__ info) {
     const int site = blockIdx.x * blockDim.x + threadIdx.x, mu = blockIdx.y;
     if (site >= V) return;
+    const bool fixed = paths_fixed(info);
+    int4 *o = reinterpret_cast<int4 *>(A);
 #pragma unroll
-    for (int e = 0; e < 9; e++) A[((size_t)link_field(mu) * 9 + e) * V + site] = U[((size_t)site * 4 + mu) * 9 + e];
+    for (int e = 0; e < 9; e++) {
+        const double2 u = U[((size_t)site * 4 + mu) * 9 + e];
+        const size_t i = ((size_t)link_field(mu) * 9 + e) * V + site;
+        if (fixed) o[i] = fx_split(u.x, u.y, PS_B);
+        else A[i] = u;
+    }
 }
 
-// fields from path sums, in place: W_j(x) = A (1-hop) or P_SU(3)(A) (2..4
+// limbs to FP64 in place, averages over paths (the force's form of the sums)
+__global__ void k_path_f64(const double2 *__restrict__ U, double2 *__restrict__ A, int V,
+                           const unsigned *__restrict__ info) {
+    const int site = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+    if (site >= V || !paths_fixed(info)) return;
+    const int n = off_class(canon_k(j));
+    if (n == 1) {
+        const int mu = j == 0 ? 0 : j == 2 ? 1 : j == 8 ? 2 : 3;
+#pragma unroll
+        for (int e = 0; e < 9; e++) A[((size_t)j * 9 + e) * V + site] = U[((size_t)site * 4 + mu) * 9 + e];
+        return;
+    }
+    const M3<double2> m = path_load(A, j, V, site, true);
+    const double s = n == 2 ? 1.0 : 4.0 / 3.0;  // 2^-1 = 1/2; 2^-2 = (3/4) 1/3; 2^-2 = 1/4 of the level below
+#pragma unroll
+    for (int e = 0; e < 9; e++) A[((size_t)j * 9 + e) * V + site] = n == 2 ? m.e[e] : cscale(m.e[e], s);
+}
+
+// fields from path sums, in place: W_j(x) = U (1-hop) or P_SU(3)(A) (2..4
 // hops), and their limbs where there is a fixed-point copy
-__global__ void k_project_hops(double2 *__restrict__ hops64, int4 *__restrict__ fx, unsigned *info, int V) {
+__global__ void k_project_hops(const double2 *__restrict__ U, double2 *__restrict__ hops64, int4 *__restrict__ fx,
+                               unsigned *info, int V) {
     const int site = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y;
     if (site >= V) return;
-    M3<double2> w = field_load<false>(hops64, j, V, site);
-    if (off_class(canon_k(j)) != 1) {
-        w = project_su3(w);
+    M3<double2> w;
+    if (off_class(canon_k(j)) == 1) {
+        const int mu = j == 0 ? 0 : j == 2 ? 1 : j == 8 ? 2 : 3;
 #pragma unroll
-        for (int e = 0; e < 9; e++) hops64[((size_t)j * 9 + e) * V + site] = w.e[e];
+        for (int e = 0; e < 9; e++) w.e[e] = U[((size_t)site * 4 + mu) * 9 + e];
+    } else {
+        w = project_su3(path_load(hops64, j, V, site, paths_fixed(info)));
     }
+#pragma unroll
+    for (int e = 0; e < 9; e++) hops64[((size_t)j * 9 + e) * V + site] = w.e[e];
     if (fx) fx_store(w.e, fx + (size_t)j * 9 * ((V + 31) & ~31), site, info);
 }
 
-// info[0]: the largest of the one-hop fields, which are the links as given (the
-// other fields are unitary); info[1]: 1 if a field matrix does not fit
-__global__ void k_fx_max(const double2 *__restrict__ h, int V, unsigned *info) {
-    const int site = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned m = 0;
-    if (site < V) {
-        double2 w[9];
-        const int j = link_field(blockIdx.y);
-#pragma unroll
-        for (int e = 0; e < 9; e++) w[e] = h[((size_t)j * 9 + e) * V + site];
-        m = norm_hi(w);
-    }
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(info, m);
-}
 __global__ void k_project_batch(const M3<double2> *__restrict__ A, M3<double2> *__restrict__ Y, long n) {
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -188,13 +328,21 @@ template <int E> __global__ void k_store_pair_f16(const double2 *__restrict__ h,
     }
 }
 
-// [40][9][V] -> [V][40][9]
-__global__ void k_export_hops(const double2 *__restrict__ h, double2 *__restrict__ out, Geom g) {
-    const int site = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y;
-    if (site >= g.V) return;
-#pragma unroll
-    for (int e = 0; e < 9; e++) out[((size_t)site * NCANON + j) * 9 + e] = h[((size_t)j * 9 + e) * g.V + site];
+// [40][9][V] -> [V][40][9], 32 sites x 40 entries at a time through shared
+// memory: both sides in runs of 512 and 640 bytes (16^3x32 0.67 ms with one
+// 16-byte store per entry and thread)
+__global__ void __launch_bounds__(256) k_export_hops(const double2 *__restrict__ h, double2 *__restrict__ out, int V) {
+    __shared__ double2 sm[40 * 33];
+    const int s0 = blockIdx.x * 32, e0 = blockIdx.y * 40;
+    for (int i = threadIdx.x; i < 40 * 32; i += 256) {
+        const int e = i >> 5, s = i & 31;
+        if (s0 + s < V) sm[e * 33 + s] = h[(size_t)(e0 + e) * V + s0 + s];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 40 * 32; i += 256) {
+        const int s = i / 40, e = i - 40 * s;
+        if (s0 + s < V) out[(size_t)(s0 + s) * (9 * NCANON) + e0 + e] = sm[e * 33 + s];
+    }
 }
 
 size_t store_bytes_a(bri_prec p, bri_comp c) {
@@ -208,17 +356,25 @@ size_t store_bytes_b(bri_prec p, bri_comp c) {
 
 }  // namespace
 
-bri_status bri_path_sums(bri_ctx *ctx, double2 *A, cudaStream_t s) {
+// levels 1 to 4 into A, in the form that ctx->fxinfo calls for
+static bri_status path_levels(bri_ctx *ctx, double2 *A, cudaStream_t s) {
     const Geom &g = ctx->g;
     const int T = 128;
     const unsigned nb = (unsigned)((g.V + T - 1) / T);
-    k_path_links<<<dim3(nb, 4), T, 0, s>>>(ctx->U, A, g.V);
+    k_path_links<<<dim3(nb, 4), T, 0, s>>>(ctx->U, A, g.V, ctx->fxinfo);
     BRI_LAUNCHED(ctx);
     for (int n = 2; n <= 4; n++) {
         const FieldList f = fields_of_class(n);
-        k_path_level<<<dim3(nb, f.n), T, 0, s>>>(n, f, A, g);
+        k_path_level<<<dim3(nb, f.n), T, 0, s>>>(n, f, A, ctx->fxinfo, g);
         BRI_LAUNCHED(ctx);
     }
+    return BRI_OK;
+}
+
+bri_status bri_path_sums(bri_ctx *ctx, double2 *A, cudaStream_t s) {
+    BRI_RETURN_IF(path_levels(ctx, A, s));
+    k_path_f64<<<dim3((unsigned)((ctx->g.V + 127) / 128), NCANON), 128, 0, s>>>(ctx->U, A, ctx->g.V, ctx->fxinfo);
+    BRI_LAUNCHED(ctx);
     return BRI_OK;
 }
 
@@ -227,13 +383,13 @@ bri_status bri_hops_build_impl(bri_ctx *ctx, cudaStream_t s) {
     if (!ctx->hops64) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->hops64, sizeof(double2) * 9 * NCANON * (size_t)g.V));
     BRI_RETURN_IF(bri_fx_reserve(ctx));
     ctx->have64 = false;
-    BRI_RETURN_IF(bri_path_sums(ctx, ctx->hops64, s));
-    const int T = 128;
-    const unsigned nb = (unsigned)((g.V + T - 1) / T);
-    BRI_TRY_CUDA(ctx, cudaMemsetAsync(ctx->fxinfo, 0, 2 * sizeof(unsigned), s));
-    k_fx_max<<<dim3(nb, 4), T, 0, s>>>(ctx->hops64, g.V, ctx->fxinfo);
+    BRI_TRY_CUDA(ctx, cudaMemsetAsync(ctx->fxinfo, 0, 3 * sizeof(unsigned), s));
+    k_link_norms<<<(unsigned)(((size_t)g.V * 4 + 127) / 128), 128, 0, s>>>(ctx->U, 4 * g.V, ctx->fxinfo);
     BRI_LAUNCHED(ctx);
-    k_project_hops<<<dim3(nb, NCANON), T, 0, s>>>(ctx->hops64, ctx->hopsfx, ctx->fxinfo, g.V);
+    BRI_RETURN_IF(path_levels(ctx, ctx->hops64, s));
+    const int T = 128;
+    k_project_hops<<<dim3((unsigned)((g.V + T - 1) / T), NCANON), T, 0, s>>>(ctx->U, ctx->hops64, ctx->hopsfx,
+                                                                             ctx->fxinfo, g.V);
     BRI_LAUNCHED(ctx);
     ctx->have64 = true;
     ctx->have_fx = ctx->hopsfx != nullptr;
@@ -319,9 +475,7 @@ bri_status bri_project_impl(bri_ctx *ctx, double2 *Y, const double2 *A, long n, 
 }
 
 bri_status bri_export_hops_impl(bri_ctx *ctx, double2 *out, cudaStream_t s) {
-    const int T = 128;
-    dim3 grid((unsigned)((ctx->g.V + T - 1) / T), NCANON);
-    k_export_hops<<<grid, T, 0, s>>>(ctx->hops64, out, ctx->g);
+    k_export_hops<<<dim3((unsigned)((ctx->g.V + 31) / 32), 9), 256, 0, s>>>(ctx->hops64, out, ctx->g.V);
     BRI_LAUNCHED(ctx);
     return BRI_OK;
 }

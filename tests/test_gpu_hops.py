@@ -133,3 +133,28 @@ def test_projection_seeds(gpu, what):
     for i in range(0, n, 40):
         best = np.trace(A[i].conj().T @ oracle.project_su3(A[i])).real
         assert np.trace(B[i]).real >= best - eps * size[i]
+
+
+@pytest.mark.parametrize("what", ["unitary", "rough", "norm 1 + 1e-4", "scaled", "one bad link"])
+def test_path_sums_fixed_point_and_fp64(gpu, what):
+    """Unit-norm links take the fixed-point path sums, any others the FP64 ones
+    (also when a single link is the reason): fields and force against the
+    oracle, to the bounds of the other tests."""
+    L = (3, 4, 5, 3)
+    U = synth.random_su3_links(L, 2.0 if what == "rough" else 0.3, 91)
+    if what == "norm 1 + 1e-4":
+        U = U * (1 + 1e-4)
+    elif what == "scaled":
+        U = U * 1e-3
+    elif what == "one bad link":
+        U[17, 2] *= 1.5
+    op = Brillouin(L, AP)
+    op.build_hops(torch.as_tensor(U, device=gpu))
+    W = oracle.build_hops(L, U)
+    Wg = op.hops().cpu().numpy()
+    for j in range(40):
+        assert np.abs(Wg[:, j] - W[:, j + 41]).max() < 1e-12, j
+    chi, psi = synth.gaussian_spinor(L, 2, 92)
+    ref = oracle.force(L, AP, U, 0.0, chi, psi)
+    dU = op.force(torch.as_tensor(chi, device=gpu), torch.as_tensor(psi, device=gpu)).cpu().numpy()
+    assert np.abs(dU - ref).max() <= 1e-10 * np.abs(ref).max()
