@@ -1,33 +1,37 @@
-// FP64 stencil apply on the integer pipe.
+// FP64 stencil apply on the integer and FP32 pipes.
 //
 // GB300 runs 2 FP64 FMAs per clock and SM, but 32 integer multiply-adds
-// 32 x 32 + 64 -> 64 bits, so the colour products, 11,520 of the 17,016 FP64
-// operations of a site, are taken in fixed point and exact integer sums:
+// 32 x 32 + 64 -> 64 bits and 128 FP32 FMAs, so the colour products, 11,520 of
+// the 17,016 FP64 operations of a site, are taken on two-limb fixed-point
+// numbers with exact integer sums:
 //
-//   link entries  w  = fw 2^(we - 62),    fw = wh 2^32 + wl, |wh| <= 2^30
-//   spinors       p  = fp 2^(e(y) - 60),  fp = ph 2^32 + pl, |ph| <= 2^28,
+//   link entries  w  = fw 2^(we - 62),    fw = (wh + wl) 2^32, |wh| <= 2^30
+//   spinors       p  = fp 2^(e(y) - 60),  fp = (ph + pl) 2^32, |ph| <= 2^28,
 //                 e(y) the exponent of the largest component of site y
-//   products      w p = wh ph 2^(we + e - 58) + (wh pl + wl ph) 2^(we + e - 90)
+//   products      w p = (wh ph + wh pl + wl ph) 2^(we + e - 58)
 //
-// (three multiply-adds a product; wl pl is below 2^-60 of the largest product
-// and dropped).  One 64-bit accumulator holds the six high products of a colour
-// row exactly, another the twelve cross products: rows and columns of a link
-// have norm <= 2^we, so |sum wh pl| <= sqrt(6) 2^61, |sum wl ph| <= 6 2^59,
-// together 7.9 2^60 < 2^63.  The row is rounded to the unit 2^(we + X_n - 58)
-// of its hop class n, X_n = the largest e(y) of the class's neighbours + h_n,
-// and the rows are summed as 64-bit integers: once with the class weight
-// lambda and once through gamma_d (entries +-1, +-i: additions only).  A
-// class sum holds at most 8, 48, 96, 64 rows (hops x directions of gamma_d) of
-// sqrt(6) 2^58: h_n = 0, 2, 3, 3.  Per class, the sums are converted and
-// weighted in FP64.  Every row is thus known to 2^-55 of its class's largest
-// neighbour and the sums over hops are exact, in any order, where FP64 rounds
-// each of ~480 partial sums: against quad precision 7.6e-17 relative (FP64 loop:
-// 1.6e-16) for Gaussian spinors, 8e-17 (1.6e-16) for a field that falls by e^-2
-// a step in every direction.
+// with integers wh, ph and |wl|, |pl| <= 1/2 kept as FP32 numbers; wl pl is
+// below 2^-60 of the largest product and dropped.  A 64-bit accumulator holds
+// the six high products of a colour row exactly; the twelve cross products, at
+// most 2^-30 of the largest product, are summed in packed FP32 FMAs (rounded to
+// 2^-24 of themselves) and added as an integer: rows and columns of a link
+// have norm <= 2^we, so |sum wh pl + wl ph| <= 7.9 2^28 < 2^31.  The row is
+// rounded to the unit 2^(we + X_n - 58) of its hop class n, X_n = the largest
+// e(y) of the class's neighbours + h_n, and the rows are summed as 64-bit
+// integers: once with the class weight lambda and once through gamma_d (entries
+// +-1, +-i: additions only).  A class sum holds at most 8, 48, 96, 64 rows
+// (hops x directions of gamma_d) of sqrt(6) 2^58: h_n = 0, 2, 3, 3.  Per
+// class, the sums are converted and weighted in FP64.  Every row is thus known
+// to about 2^-54 of its class's largest neighbour and the sums over hops are exact,
+// in any order, where FP64 rounds each of ~480 partial sums: against quad
+// precision 1.04e-16 relative (FP64 loop: 1.6e-16) for Gaussian spinors,
+// 1.02e-16 (1.6e-16) for a field that falls by e^-2 a step in every direction.
 //
-// Measured: 16^3x32 0.887 ms (FP64 kernel 4.12), 8^4 62 us (629), 32^4 6.7 ms
-// (31.2).  Bound by the integer multiply-adds (4 clocks a warp) and by fixed
-// latencies at 12 warps per SM.
+// Measured: 16^3x32 0.736 ms (FP64 kernel 4.12; cross products as integers 0.887),
+// 8^4 47 us (629; 62), 32^4 5.5 ms (31.2; 6.7).  Per pair and warp 144 wide
+// multiply-adds (4 clocks each), 144 packed FMAs (2) and 770 other
+// instructions; latency at 12 warps per SM bounds it (issue 42%, long
+// scoreboard and fixed-latency waits the top stalls).
 //
 // A site that meets an infinity, a NaN or an exponent outside the range of
 // FP64 scales takes the FP64 loop (fx_slow), as every site does when the links
@@ -75,53 +79,48 @@ __global__ void k_fx_spinor(const double2 *__restrict__ in, int4 *__restrict__ p
     p += (size_t)rhs * 12 * ((V + 31) & ~31) + fx_at(site, 12);
 #pragma unroll
     for (int k = 0; k < 12; k++)
-        p[32 * k] = (bad || zero) ? make_int4(0, 0, 0, 0) : fx_split(v[k].x, v[k].y, FX_PB - e);
+        p[32 * k] = (bad || zero) ? make_int4(0, 0, 0, 0) : fx_split_f(v[k].x, v[k].y, FX_PB - e);
 }
 
 // one colour row of W p (SGN = 1, w = row c of W) or W^dagger p (SGN = -1,
 // w = column c of W) for the two spins in p, rounded to units of
-// 2^(we + e - 58 + sh)
+// 2^(we + e - 58 + sh).  pf: the spinor's high limbs as FP32 numbers
 template <int SGN>
-BRI_D void fx_row(const int4 w[3], const int4 p[6], int sh, long long half, long long re[2], long long im[2]) {
-    // The cross products are kept 2^63 up, so that their high word is added
-    // without a sign word (2^31 less in the other accumulator); both start at
-    // half a unit, which rounds to nearest and leaves a zero row zero
-    constexpr unsigned long long up = (1ull << 63) + (1ull << 31);
-    const long long a0 = half - (1ll << 31);
-    long long ar[2] = {a0, a0}, ai[2] = {a0, a0};
-    unsigned long long br[2] = {up, up}, bi[2] = {up, up};
+BRI_D void fx_row(const int4 w[3], const int4 p[6], const float2 pf[6], int sh, long long half, long long re[2],
+                  long long im[2]) {
+    // the high products' sums start at half a unit (a zero row stays zero)
+    long long ar[2] = {half, half}, ai[2] = {half, half};
+    float2 x[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-        const int wrh = w[k].x, wrl = w[k].y;
-        const int wih = SGN > 0 ? w[k].z : -w[k].z, wil = SGN > 0 ? w[k].w : -w[k].w;
-        const int nih = SGN > 0 ? -w[k].z : w[k].z, nil = SGN > 0 ? -w[k].w : w[k].w;
+        const int wr = w[k].x, wi = SGN > 0 ? w[k].z : -w[k].z, ni = SGN > 0 ? -w[k].z : w[k].z;
+        const float fr = (float)wr, fi = (float)wi;
+        const float lr = __int_as_float(w[k].y), li = SGN > 0 ? __int_as_float(w[k].w) : -__int_as_float(w[k].w);
+        const float2 F = make_float2(fr, fi), Fi = make_float2(-fi, fr), G = make_float2(lr, li),
+                     Gi = make_float2(-li, lr);
 #pragma unroll
         for (int l = 0; l < 2; l++) {
             const int4 q = p[3 * l + k];
-            ar[l] += (long long)wrh * q.x;
-            ai[l] += (long long)wrh * q.z;
-            br[l] += (long long)wrh * q.y;
-            bi[l] += (long long)wrh * q.w;
-            br[l] += (long long)wrl * q.x;
-            bi[l] += (long long)wrl * q.z;
-            ar[l] += (long long)nih * q.z;
-            ai[l] += (long long)wih * q.x;
-            br[l] += (long long)nih * q.w;
-            bi[l] += (long long)wih * q.y;
-            br[l] += (long long)nil * q.z;
-            bi[l] += (long long)wil * q.x;
+            ar[l] += (long long)wr * q.x;
+            ai[l] += (long long)wr * q.z;
+            ar[l] += (long long)ni * q.z;
+            ai[l] += (long long)wi * q.x;
+            x[l] = __ffma2_rn(F, f2(__int_as_float(q.y)), x[l]);
+            x[l] = __ffma2_rn(Fi, f2(__int_as_float(q.w)), x[l]);
+            x[l] = __ffma2_rn(G, f2(pf[3 * l + k].x), x[l]);
+            x[l] = __ffma2_rn(Gi, f2(pf[3 * l + k].y), x[l]);
         }
     }
 #pragma unroll
     for (int l = 0; l < 2; l++) {
-        re[l] = (ar[l] + (long long)(br[l] >> 32)) >> sh;
-        im[l] = (ai[l] + (long long)(bi[l] >> 32)) >> sh;
+        re[l] = (ar[l] + __float2int_rn(x[l].x)) >> sh;
+        im[l] = (ai[l] + __float2int_rn(x[l].y)) >> sh;
     }
 }
-
 BRI_D void fx_negate(int4 p[6]) {
 #pragma unroll
-    for (int k = 0; k < 6; k++) p[k] = make_int4(-p[k].x, -p[k].y, -p[k].z, -p[k].w);
+    for (int k = 0; k < 6; k++)
+        p[k] = make_int4(-p[k].x, p[k].y ^ (int)0x80000000, -p[k].z, p[k].w ^ (int)0x80000000);
 }
 
 // the FP64 loop for one site, whole spinor (the arithmetic of hop_pair with
@@ -187,25 +186,65 @@ __device__ __noinline__ void fx_slow(int mode, const LinkF64 &ll, const double2 
 }
 
 // One thread per (site, chirality, split): a warp holds 32 sites, its spins
-// 2h, 2h + 1, and every S-th pair of the class-ordered hop list; the two warps
+// 2h, 2h + 1, and an S-th of the class-ordered hop list; the two warps
 // of a group (h = 0, 1) share the links of a pair, which they copy to shared
-// memory one pair ahead (h = 0 those of x, h = 1 those of x - d).  The splits
+// memory one pair ahead (h = 0 those of x, h = 1 those of x - d), and each lane
+// copies its neighbours' spinors there as soon as it has taken the last ones.  The splits
 // fill the chip on small lattices.  At the end of each class its sums go to
 // shared memory in FP64: lambda's to the spins' own rows, gamma_d's to the
 // rows of the other chirality (to which gamma_mu maps).
-constexpr int FX_REGS = 168;                               // registers: 12 warps per SM (128 spill, 4% slower)
+constexpr int FX_REGS = 160;  // 12 warps per SM, as the shared memory allows (168: 3% slower, 128: 10%, spills)
 template <int S> constexpr int FX_T = S == 4 ? 256 : 128;  // threads per block
 constexpr int FX_STAGE = 2 * 9 * 32;                        // int4 of the links of a pair, 32 sites
-template <int S> constexpr int FX_SMEM = FX_T<S> * 12 * 8 + (FX_T<S> / 64) * 2 * FX_STAGE * 16;
+template <int S> constexpr int FX_SMEM = FX_T<S> * (12 * 8 + 4 * 4 + 12 * 16) + (FX_T<S> / 64) * 2 * FX_STAGE * 16;
 
-BRI_D void fx_copy(uint32_t dst, const int4 *src) {
+template <int N> BRI_D void fx_copy(uint32_t dst, const int4 *src) {
 #pragma unroll
-    for (int e = 0; e < 9; e++) cp_async16(dst + 512 * e, src + 32 * e);
+    for (int e = 0; e < N; e++) cp_async16(dst + 512 * e, src + 32 * e);
 }
 BRI_D int4 lds4i(uint32_t a) {
     int4 v;
     asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
     return v;
+}
+
+// neighbours x + d and x - d of a pair (d uniform across the warp) and whether
+// the fermion phase on the way is -1, from 8 bits of the site's position: bit mu
+// is set at the top of direction mu, bit 4 + mu at the bottom (SiteNb holds
+// the same in 16 registers)
+BRI_D unsigned fx_edges(const Geom &g, int site) {
+    unsigned m = 0;
+#pragma unroll
+    for (int mu = 0; mu < 4; mu++) {
+        const int x = site % g.L[mu];
+        site /= g.L[mu];
+        m |= (x == g.L[mu] - 1 ? 1u << mu : 0u) | (x == 0 ? 16u << mu : 0u);
+    }
+    return m;
+}
+BRI_D void fx_nb(const int dm[4], const Geom &g, int site, unsigned edges, int &yf, int &yb, bool &nf, bool &nb) {
+    unsigned wf = 0, wb = 0;  // wraps, by direction
+    int stride = 1, f = site, b = site;
+#pragma unroll
+    for (int mu = 0; mu < 4; mu++) {
+        const int L = g.L[mu], c = dm[mu];
+        if (c != 0) {
+            const unsigned up = edges >> mu & 1u, dn = edges >> (4 + mu) & 1u;
+            const unsigned ff = c > 0 ? up : dn, bb = c > 0 ? dn : up;
+            const int step = c > 0 ? stride : -stride, back = L * step;
+            f += step - (ff ? back : 0);
+            b -= step - (bb ? back : 0);
+            if (g.bc[mu] < 0) {
+                wf ^= ff;
+                wb ^= bb;
+            }
+        }
+        stride *= L;
+    }
+    yf = f;
+    yb = b;
+    nf = wf != 0;
+    nb = wb != 0;
 }
 
 template <int S, bool CLOV>
@@ -234,16 +273,15 @@ __global__ void __maxnreg__(FX_REGS) k_dslash_fx(int mode, const int4 *__restric
     out += (size_t)rhs * V * 12;
     P += (size_t)rhs * 12 * Vp + 6 * 32 * h;
     ex += (size_t)rhs * V;
-    int x[4];
-    const SiteNb nb = site_nb(g, site, x);
+    const unsigned edges = fx_edges(g, site);
     // largest block exponent of each class's neighbours: the site's 2 S threads
     // take the pairs in turn
     int X[4] = {FX_ZERO, FX_ZERO, FX_ZERO, FX_ZERO};
 #pragma unroll 4
     for (int i = 2 * split + h; i < nh; i += 2 * S) {
         int yf, yb;
-        float phf, phb;
-        hop_nb(g.hop[ord.t[i]].dm, site, nb, yf, phf, yb, phb);
+        bool nf, nb;
+        fx_nb(g.hop[ord.t[i]].dm, g, site, edges, yf, yb, nf, nb);
         const int m = max(ex[yf], ex[yb]), n = ord.cls[i];
 #pragma unroll
         for (int k = 0; k < 4; k++)
@@ -262,6 +300,12 @@ __global__ void __maxnreg__(FX_REGS) k_dslash_fx(int mode, const int4 *__restric
         slow = slow || we + X[k] > 900 || we + X[k] < -900;
     }
     __syncthreads();
+    int *sx = (int *)(fx_sm + T * 12 * 8 + (T / 64) * 2 * FX_STAGE * 16) + tid;  // the four exponents
+#pragma unroll
+    for (int k = 0; k < 4; k++) sx[k * T] = X[k];
+    // this lane's slots of the warp's spinor stage: 6 entries of x + d, 6 of x - d
+    const uint32_t pst = (uint32_t)__cvta_generic_to_shared(fx_sm + T * (12 * 8 + 4 * 4) + (T / 64) * 2 * FX_STAGE * 16) +
+                         (uint32_t)(warp * 12 * 32 + lane) * 16u;
     const int sg = h ? 1 : -1;  // gamma_1..3 change sign between the chiralities, gamma_4 does not
 
     long long La[12], Ga[12];  // own rows [spin][colour][re, im]; rows of the other chirality
@@ -270,63 +314,75 @@ __global__ void __maxnreg__(FX_REGS) k_dslash_fx(int mode, const int4 *__restric
         La[i] = Ga[i] = 0;
         sm[i * T + tid] = 0.0;
     }
-    int cls = split < nh ? ord.cls[split] : 1;
-    int Xn = cls == 1 ? X[0] : cls == 2 ? X[1] : cls == 3 ? X[2] : X[3];
+    const int i0 = split * nh / S, i1 = (split + 1) * nh / S;
+    int cls = i0 < i1 ? ord.cls[i0] : 1;
+    int Xn = sx[(cls - 1) * T];
     auto flush = [&](int n) {
         const double scale = slow ? 0.0 : __hiloint2double((1023 + we + Xn - FX_AB) << 20, 0);
         const double cl = g.lamd[n] * scale, cg = g.rhod[n] * (mode == 1 ? -scale : scale);
 #pragma unroll
-        for (int i = 0; i < 12; i++) sm[i * T + tid] = fma((double)La[i], cl, sm[i * T + tid]);
+        for (int i = 0; i < 12; i++) sm[i * T + tid] = fma(fx_double(La[i], 0), cl, sm[i * T + tid]);
         asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");
 #pragma unroll
         for (int i = 0; i < 12; i++) {
-            sm[i * T + (tid ^ 32)] = fma((double)Ga[i], cg, sm[i * T + (tid ^ 32)]);
+            sm[i * T + (tid ^ 32)] = fma(fx_double(Ga[i], 0), cg, sm[i * T + (tid ^ 32)]);
             La[i] = Ga[i] = 0;
         }
     };
     int yf = site, yb = site;
-    float phf = 1.f, phb = 1.f;
+    bool nextf = false, nextb = false;
+    int exf = 0, exb = 0;
     const size_t own = fx_at(site, 9);
     auto ahead = [&](int i, int buf) {  // neighbours of pair i and the copies of its links
         const HopArg &hp = g.hop[ord.t[i]];
-        hop_nb(hp.dm, site, nb, yf, phf, yb, phb);
-        fx_copy(stage + (uint32_t)(buf * FX_STAGE + h * 9 * 32) * 16u,
-                W + (size_t)hp.j * 9 * Vp + (h ? fx_at(yb, 9) : own));
+        fx_nb(hp.dm, g, site, edges, yf, yb, nextf, nextb);
+        exf = ex[yf];
+        exb = ex[yb];
+        fx_copy<9>(stage + (uint32_t)(buf * FX_STAGE + h * 9 * 32) * 16u,
+                   W + (size_t)hp.j * 9 * Vp + (h ? fx_at(yb, 9) : own));
     };
-    if (split < nh) ahead(split, 0);
+    // a spinor's copy into the slots that this lane has read into registers
+    auto spinor = [&](int y, int slot) { fx_copy<6>(pst + 512u * slot, P + fx_at(y, 12)); };
+    if (i0 < i1) {
+        ahead(i0, 0);
+        spinor(yf, 0);
+        spinor(yb, 6);
+    }
     int buf = 0;
 #pragma unroll 1
-    for (int i = split; i < nh; i += S) {
+    for (int i = i0; i < i1; i++) {
         // this pair's copies (both warps'), and the other buffer free again
         asm volatile("cp.async.wait_all;" ::: "memory");
         asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");
-        const int cyf = yf, cyb = yb;
-        const bool nf = phf < 0.f, ng = phb < 0.f;
-        if (i + S < nh) ahead(i + S, buf ^ 1);
+        const int cef = exf, ceb = exb;
+        const bool nf = nextf, ng = nextb;
+        if (i + 1 < i1) ahead(i + 1, buf ^ 1);
         const HopArg &hp = g.hop[ord.t[i]];
         if (ord.cls[i] != cls) {
             flush(cls);
             cls = ord.cls[i];
-            Xn = cls == 1 ? X[0] : cls == 2 ? X[1] : cls == 3 ? X[2] : X[3];
+            Xn = sx[(cls - 1) * T];
         }
         const uint32_t wf = stage + (uint32_t)(buf * FX_STAGE) * 16u, wb = wf + 9u * 512u;
         buf ^= 1;
         long long f[12];
         {
             int4 p[6];
-            const int4 *pp = P + fx_at(cyf, 12);
 #pragma unroll
-            for (int k = 0; k < 6; k++) p[k] = pp[32 * k];
-            const int sh = min(Xn - ex[cyf], 63);
+            for (int k = 0; k < 6; k++) p[k] = lds4i(pst + 512u * k);
+            const int sh = min(Xn - cef, 63);
             const long long half = (long long)((1ull << sh) >> 1);
             if (nf) fx_negate(p);
+            float2 pf[6];
+#pragma unroll
+            for (int k = 0; k < 6; k++) pf[k] = make_float2((float)p[k].x, (float)p[k].z);
 #pragma unroll
             for (int c = 0; c < 3; c++) {
                 int4 w[3];
 #pragma unroll
                 for (int k = 0; k < 3; k++) w[k] = lds4i(wf + 512u * (3 * c + k));
                 long long re[2], im[2];
-                fx_row<1>(w, p, sh, half, re, im);
+                fx_row<1>(w, p, pf, sh, half, re, im);
 #pragma unroll
                 for (int l = 0; l < 2; l++) {
                     f[6 * l + 2 * c] = re[l];
@@ -336,21 +392,24 @@ __global__ void __maxnreg__(FX_REGS) k_dslash_fx(int mode, const int4 *__restric
                 }
             }
         }
+        if (i + 1 < i1) spinor(yf, 0);
         {
             int4 p[6];
-            const int4 *pp = P + fx_at(cyb, 12);
 #pragma unroll
-            for (int k = 0; k < 6; k++) p[k] = pp[32 * k];
-            const int sh = min(Xn - ex[cyb], 63);
+            for (int k = 0; k < 6; k++) p[k] = lds4i(pst + 512u * (6 + k));
+            const int sh = min(Xn - ceb, 63);
             const long long half = (long long)((1ull << sh) >> 1);
             if (ng) fx_negate(p);
+            float2 pf[6];
+#pragma unroll
+            for (int k = 0; k < 6; k++) pf[k] = make_float2((float)p[k].x, (float)p[k].z);
 #pragma unroll
             for (int c = 0; c < 3; c++) {
                 int4 w[3];
 #pragma unroll
                 for (int k = 0; k < 3; k++) w[k] = lds4i(wb + 512u * (3 * k + c));
                 long long re[2], im[2];
-                fx_row<-1>(w, p, sh, half, re, im);
+                fx_row<-1>(w, p, pf, sh, half, re, im);
 #pragma unroll
                 for (int l = 0; l < 2; l++) {
                     La[6 * l + 2 * c] += re[l];
@@ -360,6 +419,7 @@ __global__ void __maxnreg__(FX_REGS) k_dslash_fx(int mode, const int4 *__restric
                 }
             }
         }
+        if (i + 1 < i1) spinor(yb, 6);
         // gamma_d of the difference: additions to the other chirality's rows (for
         // h = 1 the rows gcol(mu, 2 + l) of gamma_mu; for h = 0 the same places)
         auto gamma_add = [&](int mu, bool pos) {

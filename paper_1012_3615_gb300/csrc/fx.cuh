@@ -31,6 +31,13 @@ BRI_D int4 fx_split(double re, double im, int sh) {
     if (v.w == (int)0x80000000) v.w++;
     return v;
 }
+// the same with the low limb as an FP32 number in units of the high one
+BRI_D int4 fx_split_f(double re, double im, int sh) {
+    const long long a = fx_int(re, sh), b = fx_int(im, sh);
+    const int al = (int)a, bl = (int)b;
+    return make_int4((int)((a - al) >> 32), __float_as_int((float)al * 0x1p-32f), (int)((b - bl) >> 32),
+                     __float_as_int((float)bl * 0x1p-32f));
+}
 BRI_D unsigned abs_hi(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 
 // f 2^sh, rounded to nearest even, by integer operations
@@ -86,7 +93,7 @@ BRI_D void fx_store(const double2 w[9], int4 *o, int site, unsigned *info) {
     }
     o += fx_at(site, 9);
 #pragma unroll
-    for (int e = 0; e < 9; e++) o[32 * e] = fx_split(w[e].x, w[e].y, FX_WB - we);
+    for (int e = 0; e < 9; e++) o[32 * e] = fx_split_f(w[e].x, w[e].y, FX_WB - we);
 }
 
 }  // namespace bri

@@ -3,7 +3,7 @@ split of the hop list changes, on site ranges, with fields that span many
 orders of magnitude, with links that are not unitary, and with infinities and
 NaN (where it runs the FP64 loop), against the oracle.
 
-Tolerance: every product is known to 2^-55 of its class's largest neighbour,
+Tolerance: every row is known to about 2^-54 of its class's largest neighbour,
 the final FP64 operations round a few times: 1e-15 of the largest result, and
 4e-15 of each site's own largest component (weights 1/16 to 1/432 times up to
 32 hops a class)."""
