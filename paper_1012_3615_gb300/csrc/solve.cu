@@ -27,11 +27,12 @@ using namespace bri;
 namespace {
 
 constexpr int RT = 256;     // threads of the vector / reduction kernels
-constexpr int RBLK = 304;   // blocks per right-hand side of the reduction kernels (2 x 152 SMs)
+constexpr int RBLK = 608;   // most blocks per right-hand side of the vector kernels (4 x 152 SMs)
 constexpr int NPART = 4;    // doubles per partial sum
 
 struct BiState {
-    double2 rho, rho_old, alpha, omega;
+    double2 rho, alpha, omega;
+    double2 beta;  // (rho / rho_old)(alpha / omega) of the next p update
     double rr, tol2, bb;
     int iters, maxit;
 };
@@ -46,20 +47,21 @@ BRI_D double warp_sum(double v) {
     return v;
 }
 
-// block-wide sum of NV doubles; the result is valid in thread 0
+// block-wide sum of NV doubles; the result is valid in thread 0.  One warp adds
+// the 256 values (8 per lane, then a tree), 13 FP64 additions per value of a
+// block: a tree in every warp takes 45, and an FP64 addition holds a scheduler's
+// pipe for 64 clocks
 template <int NV> BRI_D void block_sum(double v[NV]) {
-    __shared__ double sm[NV][RT / 32];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    __shared__ double sm[NV][RT];
 #pragma unroll
-    for (int k = 0; k < NV; k++) {
-        v[k] = warp_sum(v[k]);
-        if (l == 0) sm[k][w] = v[k];
-    }
+    for (int k = 0; k < NV; k++) sm[k][threadIdx.x] = v[k];
     __syncthreads();
-    if (w == 0) {
+    if (threadIdx.x < 32) {
 #pragma unroll
         for (int k = 0; k < NV; k++) {
-            double t = l < RT / 32 ? sm[k][l] : 0.0;
+            double t = sm[k][threadIdx.x];
+#pragma unroll
+            for (int j = 1; j < RT / 32; j++) t += sm[k][threadIdx.x + 32 * j];
             v[k] = warp_sum(t);
         }
     }
@@ -106,32 +108,84 @@ BRI_D bool finite2(double2 a) { return isfinite(a.x) && isfinite(a.y); }
 
 template <typename T> BRI_D T tc(double2 z) { return mk<T>(z.x, z.y); }
 
-// ---- BiCGstab step kernels (grid: RBLK x nrhs) ------------------------------
-template <typename T>
-__global__ void k_bi_p(T *p, const T *r, const T *v, const BiState *st, const int *flag, size_t n) {
-    const int rh = blockIdx.y;
-    if (flag[rh]) return;
-    const BiState s = st[rh];
-    const double2 beta = cmul(dcdiv(s.rho, s.rho_old), dcdiv(s.alpha, s.omega));
-    const T b = tc<T>(beta), om = tc<T>(s.omega);
-    p += rh * n; r += rh * n; v += rh * n;
-    for (size_t i = (size_t)blockIdx.x * RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT)
-        p[i] = cadd(r[i], cmul(b, csub(p[i], cmul(om, v[i]))));
+// ---- BiCGstab step kernels (grid: vec_grid(n, nrhs)) ---------------------------
+// Bound by memory: by HBM for many right-hand sides (16^3x32, FP32, 12: x/r update
+// 157 us, 6.7 TB/s), by L2 and latency for one: p, alpha, s, omega, x/r 9.5, 12.2,
+// 7.1, 12.4, 19.4 us (one element a load, a tree in every warp and beta's FP64
+// divisions in every thread: 19.3, 17.1, 12.7, 17.6, 34.3).  Vectors move in
+// 16-byte packs, two packs of each in flight per thread before either is used.
+template <typename T> constexpr int PK = 16 / sizeof(T);  // elements per pack
+template <typename T> struct alignas(16) Pack {
+    T e[PK<T>];
+};
+// f(pack index, second) over the packs of one right-hand side, two at a time:
+// load both, then compute both
+template <typename T, typename L, typename F> BRI_D void for_packs(size_t n, L &&load, F &&use) {
+    const size_t m = n / PK<T>, step = (size_t)gridDim.x * RT;
+    for (size_t i = (size_t)blockIdx.x * RT + threadIdx.x; i < m; i += 2 * step) {
+        const bool two = i + step < m;
+        const auto a = load(i);
+        const auto b = load(two ? i + step : i);
+        use(i, a);
+        if (two) use(i + step, b);
+    }
+}
+template <typename T> BRI_D Pack<T> pk(const T *p, size_t i) { return reinterpret_cast<const Pack<T> *>(p)[i]; }
+template <typename T> BRI_D void put(T *p, size_t i, const Pack<T> &v) { reinterpret_cast<Pack<T> *>(p)[i] = v; }
+// z + a b, z - a b
+template <typename T> BRI_D T cfma(T a, T b, T z) {
+    T r;
+    r.x = fma(a.x, b.x, fma(-a.y, b.y, z.x));
+    r.y = fma(a.x, b.y, fma(a.y, b.x, z.y));
+    return r;
+}
+template <typename T> BRI_D T cfms(T a, T b, T z) {
+    T r;
+    r.x = fma(-a.x, b.x, fma(a.y, b.y, z.x));
+    r.y = fma(-a.x, b.y, fma(-a.y, b.x, z.y));
+    return r;
+}
+// (re, im) += conj(a) b;  s += |a|^2
+template <typename T, typename A> BRI_D void dot_add(T a, T b, A &re, A &im) {
+    re = fma((A)a.x, (A)b.x, fma((A)a.y, (A)b.y, re));
+    im = fma((A)a.x, (A)b.y, fma(-(A)a.y, (A)b.x, im));
+}
+template <typename T, typename A> BRI_D void norm_add(T a, A &s) {
+    s = fma((A)a.x, (A)a.x, fma((A)a.y, (A)a.y, s));
 }
 
 template <typename T>
-__global__ void k_bi_alpha(const T *rhat, const T *v, BiState *st, int *flag, double *part, unsigned *tick,
-                           size_t n) {
+__global__ void __launch_bounds__(RT) k_bi_p(T *p, const T *__restrict__ r, const T *__restrict__ v, const BiState *st,
+                                             const int *flag, size_t n) {
+    const int rh = blockIdx.y;
+    if (flag[rh]) return;
+    const T b = tc<T>(st[rh].beta), om = tc<T>(st[rh].omega);
+    p += rh * n; r += rh * n; v += rh * n;
+    struct In { Pack<T> p, r, v; };
+    for_packs<T>(
+        n, [&](size_t i) { return In{pk(p, i), pk(r, i), pk(v, i)}; },
+        [&](size_t i, In z) {
+#pragma unroll
+            for (int k = 0; k < PK<T>; k++) z.p.e[k] = cfma(b, cfms(om, z.v.e[k], z.p.e[k]), z.r.e[k]);
+            put(p, i, z.p);
+        });
+}
+
+template <typename T>
+__global__ void __launch_bounds__(RT) k_bi_alpha(const T *__restrict__ rhat, const T *__restrict__ v, BiState *st,
+                                                 int *flag, double *part, unsigned *tick, size_t n) {
     const int rh = blockIdx.y;
     if (flag[rh]) return;
     rhat += rh * n; v += rh * n;
     using A = typename AccT<T>::A;
     A ac[2] = {0, 0};
-    for (size_t i = (size_t)blockIdx.x * RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT) {
-        T a = rhat[i], b = v[i];
-        ac[0] += (A)a.x * b.x + (A)a.y * b.y;
-        ac[1] += (A)a.x * b.y - (A)a.y * b.x;
-    }
+    struct In { Pack<T> h, v; };
+    for_packs<T>(
+        n, [&](size_t i) { return In{pk(rhat, i), pk(v, i)}; },
+        [&](size_t, const In &z) {
+#pragma unroll
+            for (int k = 0; k < PK<T>; k++) dot_add(z.h.e[k], z.v.e[k], ac[0], ac[1]);
+        });
     double acc[2] = {ac[0], ac[1]};
     if (partial_and_ticket<2>(acc, part + (size_t)rh * RBLK * NPART, tick + rh)) {
         double s[2];
@@ -146,28 +200,40 @@ __global__ void k_bi_alpha(const T *rhat, const T *v, BiState *st, int *flag, do
 }
 
 template <typename T>
-__global__ void k_bi_s(T *s, const T *r, const T *v, const BiState *st, const int *flag, size_t n) {
+__global__ void __launch_bounds__(RT) k_bi_s(T *__restrict__ s, const T *__restrict__ r, const T *__restrict__ v,
+                                             const BiState *st, const int *flag, size_t n) {
     const int rh = blockIdx.y;
     if (flag[rh]) return;
     const T a = tc<T>(st[rh].alpha);
     s += rh * n; r += rh * n; v += rh * n;
-    for (size_t i = (size_t)blockIdx.x * RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT)
-        s[i] = csub(r[i], cmul(a, v[i]));
+    struct In { Pack<T> r, v; };
+    for_packs<T>(
+        n, [&](size_t i) { return In{pk(r, i), pk(v, i)}; },
+        [&](size_t i, In z) {
+#pragma unroll
+            for (int k = 0; k < PK<T>; k++) z.r.e[k] = cfms(a, z.v.e[k], z.r.e[k]);
+            put(s, i, z.r);
+        });
 }
 
 template <typename T>
-__global__ void k_bi_omega(const T *t, const T *s, BiState *st, int *flag, double *part, unsigned *tick, size_t n) {
+__global__ void __launch_bounds__(RT) k_bi_omega(const T *__restrict__ t, const T *__restrict__ s, BiState *st,
+                                                 int *flag, double *part, unsigned *tick, size_t n) {
     const int rh = blockIdx.y;
     if (flag[rh]) return;
     t += rh * n; s += rh * n;
     using A = typename AccT<T>::A;
     A ac[3] = {0, 0, 0};
-    for (size_t i = (size_t)blockIdx.x * RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT) {
-        T a = t[i], b = s[i];
-        ac[0] += (A)a.x * b.x + (A)a.y * b.y;
-        ac[1] += (A)a.x * b.y - (A)a.y * b.x;
-        ac[2] += (A)a.x * a.x + (A)a.y * a.y;
-    }
+    struct In { Pack<T> t, s; };
+    for_packs<T>(
+        n, [&](size_t i) { return In{pk(t, i), pk(s, i)}; },
+        [&](size_t, const In &z) {
+#pragma unroll
+            for (int k = 0; k < PK<T>; k++) {
+                dot_add(z.t.e[k], z.s.e[k], ac[0], ac[1]);
+                norm_add(z.t.e[k], ac[2]);
+            }
+        });
     double acc[3] = {ac[0], ac[1], ac[2]};
     if (partial_and_ticket<3>(acc, part + (size_t)rh * RBLK * NPART, tick + rh)) {
         double q[3];
@@ -181,24 +247,31 @@ __global__ void k_bi_omega(const T *t, const T *s, BiState *st, int *flag, doubl
 }
 
 template <typename T>
-__global__ void k_bi_xr(T *x, T *r, const T *p, const T *s, const T *t, const T *rhat, BiState *st, int *flag,
-                        double *part, unsigned *tick, size_t n) {
+__global__ void __launch_bounds__(RT) k_bi_xr(T *x, T *__restrict__ r, const T *__restrict__ p, const T *__restrict__ s,
+                                              const T *__restrict__ t, const T *__restrict__ rhat, BiState *st,
+                                              int *flag, double *part, unsigned *tick, size_t n) {
     const int rh = blockIdx.y;
     if (flag[rh]) return;
     const T a = tc<T>(st[rh].alpha), om = tc<T>(st[rh].omega);
     const size_t o = rh * n;
+    x += o; r += o; p += o; s += o; t += o; rhat += o;
     using A = typename AccT<T>::A;
     A ac[3] = {0, 0, 0};
-    for (size_t i = (size_t)blockIdx.x * RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT) {
-        T si = s[o + i];
-        x[o + i] = cadd(x[o + i], cadd(cmul(a, p[o + i]), cmul(om, si)));
-        T ri = csub(si, cmul(om, t[o + i]));
-        r[o + i] = ri;
-        T h = rhat[o + i];
-        ac[0] += (A)h.x * ri.x + (A)h.y * ri.y;
-        ac[1] += (A)h.x * ri.y - (A)h.y * ri.x;
-        ac[2] += (A)ri.x * ri.x + (A)ri.y * ri.y;
-    }
+    struct In { Pack<T> x, p, s, t, h; };
+    for_packs<T>(
+        n, [&](size_t i) { return In{pk(x, i), pk(p, i), pk(s, i), pk(t, i), pk(rhat, i)}; },
+        [&](size_t i, In z) {
+#pragma unroll
+            for (int k = 0; k < PK<T>; k++) {
+                z.x.e[k] = cfma(a, z.p.e[k], cfma(om, z.s.e[k], z.x.e[k]));
+                const T ri = cfms(om, z.t.e[k], z.s.e[k]);
+                z.s.e[k] = ri;
+                dot_add(z.h.e[k], ri, ac[0], ac[1]);
+                norm_add(ri, ac[2]);
+            }
+            put(x, i, z.x);
+            put(r, i, z.s);
+        });
     double acc[3] = {ac[0], ac[1], ac[2]};
     if (partial_and_ticket<3>(acc, part + (size_t)rh * RBLK * NPART, tick + rh)) {
         double q[3];
@@ -206,8 +279,9 @@ __global__ void k_bi_xr(T *x, T *r, const T *p, const T *s, const T *t, const T 
         if (threadIdx.x != 0) return;
         BiState &S = st[rh];
         S.iters++;
-        S.rho_old = S.rho;
+        const double2 old = S.rho;
         S.rho = make_double2(q[0], q[1]);
+        S.beta = cmul(dcdiv(S.rho, old), dcdiv(S.alpha, S.omega));  // once here: FP64 divisions
         S.rr = q[2];
         if (!isfinite(q[0]) || !isfinite(q[1]) || !isfinite(q[2])) flag[rh] = 3;
         else if (q[2] <= S.tol2) flag[rh] = 1;
@@ -242,7 +316,8 @@ __global__ void k_bi_init(T *r, T *rhat, T *p, T *v, const T *b, int have_ax, Bi
         if (threadIdx.x != 0) return;
         BiState S;
         S.rho = make_double2(q[0], 0.0);
-        S.rho_old = S.alpha = S.omega = make_double2(1.0, 0.0);
+        S.alpha = S.omega = make_double2(1.0, 0.0);
+        S.beta = S.rho;
         S.rr = q[0];
         S.bb = q[1];
         S.tol2 = tol * tol * q[1];
@@ -433,13 +508,19 @@ static bri_status ensure_work(bri_ctx *ctx, int nrhs, bool need64, bool need32) 
 
 namespace {
 
+// two packs per thread, at most RBLK blocks per right-hand side
+template <typename T> dim3 vec_grid(size_t n, int nrhs) {
+    const size_t b = (n / PK<T> + 2 * RT - 1) / (2 * RT);
+    return dim3((unsigned)(b < 1 ? 1 : b < RBLK ? b : RBLK), (unsigned)nrhs);
+}
+
 // enqueue `iters` BiCGstab iterations on vectors vs (element T) for nrhs right-hand sides
 template <typename T>
 bri_status enqueue_iters(bri_ctx *ctx, const VecSet &vs, int nrhs, double m0, bri_prec prec, int iters,
                          cudaStream_t s) {
     SolverWork *w = ctx->work;
     const size_t n = w->n;
-    dim3 grid(RBLK, nrhs);
+    const dim3 grid = vec_grid<T>(n, nrhs);
     T *x = (T *)vs.x, *r = (T *)vs.r, *rh = (T *)vs.rhat, *p = (T *)vs.p, *v = (T *)vs.v, *sv = (T *)vs.s,
       *t = (T *)vs.t;
     const int thr = bri_dslash_threads(ctx, prec, nrhs);
