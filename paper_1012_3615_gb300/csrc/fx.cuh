@@ -83,8 +83,13 @@ BRI_D int fx_we(unsigned hi) {
 // = V rounded up to 32: the entries of a site lie at fixed offsets from its first
 BRI_D size_t fx_at(int site, int entries) { return (size_t)(site >> 5) * (32 * entries) + (site & 31); }
 
-// the limbs of one field matrix of site s (o: the field's start); info[1] = 1 if
-// it does not fit
+// the limbs of a unitary field matrix of one site (o: the field's start)
+BRI_D void fx_store_unitary(const double2 w[9], int4 *o, int site, int we) {
+    o += fx_at(site, 9);
+#pragma unroll
+    for (int e = 0; e < 9; e++) o[32 * e] = fx_split_f(w[e].x, w[e].y, FX_WB - we);
+}
+// the limbs of any field matrix of one site; info[1] = 1 if it does not fit
 BRI_D void fx_store(const double2 w[9], int4 *o, int site, unsigned *info) {
     const int we = fx_we(info[0]);
     if (we > 400 || norm_hi(w) > max(info[0], FX_ONE)) {  // infinities, NaN or huge entries

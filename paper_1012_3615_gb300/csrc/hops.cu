@@ -21,6 +21,7 @@
 #include "links.cuh"
 #include "paths.cuh"
 #include "project.cuh"
+#include "project_fx.cuh"
 
 using namespace bri;
 
@@ -208,23 +209,39 @@ __global__ void k_path_f64(const double2 *__restrict__ U, double2 *__restrict__ 
 }
 
 // fields from path sums, in place: W_j(x) = U (1-hop) or P_SU(3)(A) (2..4
-// hops), and their limbs where there is a fixed-point copy
-__global__ void k_project_hops(const double2 *__restrict__ U, double2 *__restrict__ hops64, int4 *__restrict__ fx,
+// hops), and their limbs where there is a fixed-point copy.  Path sums in fixed
+// point are projected in it (project_fx.cuh).  168 registers: the code is longer
+// than the instruction cache, three blocks an SM hide its fetches better than two
+// (16^3x32: 5.56 ms a build at 255 registers, 4.50 at 168 and at 128, 5.06 with
+// the FP64 refinement).
+__global__ void __launch_bounds__(128, 3) k_project_hops(const double2 *__restrict__ U, double2 *__restrict__ hops64, int4 *__restrict__ fx,
                                unsigned *info, int V) {
     const int site = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y;
     if (site >= V) return;
     M3<double2> w;
+    bool unitary = false;
     if (off_class(canon_k(j)) == 1) {
         const int mu = j == 0 ? 0 : j == 2 ? 1 : j == 8 ? 2 : 3;
 #pragma unroll
         for (int e = 0; e < 9; e++) w.e[e] = U[((size_t)site * 4 + mu) * 9 + e];
     } else {
-        w = project_su3(path_load(hops64, j, V, site, paths_fixed(info)));
+        const bool fixed = paths_fixed(info);
+        if (fixed) {
+            const int4 *p = reinterpret_cast<const int4 *>(hops64);
+            int4 A[9];
+#pragma unroll
+            for (int e = 0; e < 9; e++) A[e] = p[((size_t)j * 9 + e) * V + site];
+            unitary = project_fast_fx(A, w);
+        }
+        if (!unitary) w = project_su3(path_load(hops64, j, V, site, fixed));
     }
 #pragma unroll
     for (int e = 0; e < 9; e++) hops64[((size_t)j * 9 + e) * V + site] = w.e[e];
-    if (fx) fx_store(w.e, fx + (size_t)j * 9 * ((V + 31) & ~31), site, info);
+    if (!fx) return;
+    int4 *o = fx + (size_t)j * 9 * ((V + 31) & ~31);
+    if (unitary) fx_store_unitary(w.e, o, site, fx_we(info[0]));
+    else fx_store(w.e, o, site, info);
 }
 
 __global__ void k_project_batch(const M3<double2> *__restrict__ A, M3<double2> *__restrict__ Y, long n) {

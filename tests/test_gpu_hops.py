@@ -158,3 +158,30 @@ def test_path_sums_fixed_point_and_fp64(gpu, what):
     ref = oracle.force(L, AP, U, 0.0, chi, psi)
     dU = op.force(torch.as_tensor(chi, device=gpu), torch.as_tensor(psi, device=gpu)).cpu().numpy()
     assert np.abs(dU - ref).max() <= 1e-10 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("L,eps", [((4, 3, 3, 3), 0.3), ((3, 5, 3, 3), 1.0), ((3, 3, 3, 4), 3.0)])
+def test_projection_of_fixed_point_sums(gpu, L, eps):
+    """The off-axis fields of unitary links, projected in fixed point where the
+    FP32 seed settles and in the general form elsewhere: special unitary,
+    stationary and no worse than the oracle's maximum at the oracle's path sums.
+    Bounds as for the projection of single matrices, 16 2^-52."""
+    U = synth.random_su3_links(L, eps, 95)
+    op = Brillouin(L, AP)
+    op.build_hops(torch.as_tensor(U, device=gpu))
+    W = op.hops().cpu().numpy()
+    tol = 16 * 2.0**-52
+    for j in range(40):
+        d = [(j + 41) // 3**m % 3 - 1 for m in range(4)]
+        if sum(map(abs, d)) < 2:
+            continue
+        Y = W[:, j]
+        A = np.stack([a / n for a, n in (oracle.path_sum(L, U, s, d) for s in range(len(W)))])
+        assert np.abs(Y.conj().transpose(0, 2, 1) @ Y - np.eye(3)).max() <= tol
+        assert np.abs(np.linalg.det(Y) - 1).max() <= tol
+        B = A.conj().transpose(0, 2, 1) @ Y
+        T = 0.5 * (B - B.conj().transpose(0, 2, 1))
+        T -= np.eye(3) * (np.trace(T, axis1=1, axis2=2) / 3)[:, None, None]
+        assert np.abs(T).max() <= tol
+        for s in range(0, len(W), 20):
+            assert np.trace(B[s]).real >= np.trace(A[s].conj().T @ oracle.project_su3(A[s])).real - tol
