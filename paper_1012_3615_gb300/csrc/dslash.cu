@@ -87,7 +87,7 @@ static bri_status dslash_geom(bri_ctx *ctx, const Geom &g, void *out, const void
         if (!ctx->have64) return bri_fail(ctx, BRI_ESTATE, "FP64 hopping fields not built");
         if (ctx->have_fx) {
             int done = 0;
-            BRI_RETURN_IF(bri_dslash_fx(ctx, g, out, in, nrhs, m0, mode, skip, work, &done, s));
+            BRI_RETURN_IF(bri_dslash_fx(ctx, g, out, in, nrhs, m0, mode & 3, skip, work, &done, s));
             if (done == nrhs) return BRI_OK;
             const size_t field = (size_t)done * g.V * 12;
             out = (double2 *)out + field;
@@ -103,7 +103,7 @@ static bri_status dslash_geom(bri_ctx *ctx, const Geom &g, void *out, const void
         if ((threads >> 11) == 8) {
             // tensor-core apply: full link storage, whole lattice, no clover term
             if (st.comp == BRI_LINK_FULL && !g.clov64 && g.s0 == 0 && g.s1 == g.V)
-                return bri_dslash_tc(ctx, out, in, nrhs, m0, mode, prec, skip, threads & 2047, s);
+                return bri_dslash_tc(ctx, out, in, nrhs, m0, mode & 3, prec, skip, threads & 2047, s);
             threads = default_shape(ctx, prec);
         }
         const LinkStore &ps = prec == BRI_F32 ? ctx->p32 : ctx->p16;
@@ -115,14 +115,14 @@ static bri_status dslash_geom(bri_ctx *ctx, const Geom &g, void *out, const void
             const int H = g.V / 2;
             if (prec == BRI_F32) {
                 if (ps.comp == BRI_LINK_FULL)
-                    dslash_pair_launch(mode, PairF32<9>{(const float4 *)ps.a, H}, in, out, nrhs, g, diag, skip, thr, s);
+                    dslash_pair_launch(mode & 3, PairF32<9>{(const float4 *)ps.a, H}, in, out, nrhs, g, diag, skip, thr, s);
                 else
-                    dslash_pair_launch(mode, PairF32<6>{(const float4 *)ps.a, H}, in, out, nrhs, g, diag, skip, thr, s);
+                    dslash_pair_launch(mode & 3, PairF32<6>{(const float4 *)ps.a, H}, in, out, nrhs, g, diag, skip, thr, s);
             } else {
                 if (ps.comp == BRI_LINK_FULL)
-                    dslash_pair_launch(mode, PairF16<9>{(const uint2 *)ps.a, H}, in, out, nrhs, g, diag, skip, thr, s);
+                    dslash_pair_launch(mode & 3, PairF16<9>{(const uint2 *)ps.a, H}, in, out, nrhs, g, diag, skip, thr, s);
                 else
-                    dslash_pair_launch(mode, PairF16<6>{(const uint2 *)ps.a, H}, in, out, nrhs, g, diag, skip, thr, s);
+                    dslash_pair_launch(mode & 3, PairF16<6>{(const uint2 *)ps.a, H}, in, out, nrhs, g, diag, skip, thr, s);
             }
             BRI_LAUNCHED(ctx);
             return BRI_OK;

@@ -1491,10 +1491,12 @@ void dslash_launch(int mode, const LL &ll, const void *in, void *out, int nrhs, 
             return;
         }
     }
+    const bool parts = !(mode & DSLASH_ONE_PART) && dslash_in_parts(g.V);
+    mode &= 3;
     if constexpr (sizeof(T) == 8) {
         // pair loops on small lattices: the split form
         const int v = threads >> 11;
-        if (dslash_in_parts(g.V) && (g.clov64 || v == 5 || v == 6 || v == 9)) {
+        if (parts && (g.clov64 || v == 5 || v == 6 || v == 9)) {
             constexpr int VF = LL::COMP == BRI_LINK_8PARAM || LL::FULL32 ? 5 : 9;
             auto launch = [&](auto S, auto C) {
                 constexpr int spb = 128 / decltype(S)::value;

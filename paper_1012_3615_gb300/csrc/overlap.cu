@@ -33,6 +33,10 @@
 
 using namespace bri;
 
+// gamma5 D with the hop list of a site summed in one part on every lattice: what
+// is computed from FP32 applies here is handed out in FP64, with their rounding
+static constexpr int HERM = 2 | DSLASH_ONE_PART;
+
 namespace {
 
 constexpr int VT = 256;         // threads of the vector kernels
@@ -95,23 +99,23 @@ __global__ void k_mdot_part(const T *__restrict__ Vb, size_t ldv, const T *__res
     if (threadIdx.x == 0) part[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = acc;
 }
 
-// h[j] = sum of the partials of vector j (one warp per vector: lane l takes the
-// blocks l, l + 32, ... in order, then a fixed tree; one thread for all 152 took
-// 21 us); the real part of h[m - 1] is also added to *racc when racc is given
-// (Lanczos alpha)
+// h[j] = sum of the partials of vector j in block order; the real part of
+// h[m - 1] is also added to *racc when racc is given (Lanczos alpha).  One warp
+// per vector: it fetches the partials at once and lanes 0 and 1 add the real and
+// imaginary parts in order (one thread with a load per addition took 21 us)
 __global__ void k_mdot_final(const double2 *__restrict__ part, int nb, int m, double2 *h, double *racc) {
-    const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, l = threadIdx.x & 31;
+    __shared__ double2 p[4][DB];
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, j = blockIdx.x * 4 + w;
     if (j >= m) return;
-    double2 s = make_double2(0.0, 0.0);
-    for (int b = l; b < nb; b += 32) s = cadd(s, part[(size_t)j * nb + b]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
-        s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
-    }
-    if (l != 0) return;
-    h[j] = s;
-    if (racc && j == m - 1) *racc += s.x;
+    for (int b = l; b < nb; b += 32) p[w][b] = part[(size_t)j * nb + b];
+    __syncwarp();
+    if (l > 1) return;
+    const double *q = reinterpret_cast<const double *>(p[w]) + l;
+    double s = 0.0;
+#pragma unroll 8
+    for (int b = 0; b < nb; b++) s += q[2 * b];
+    reinterpret_cast<double *>(h + j)[l] = s;
+    if (racc && l == 0 && j == m - 1) *racc += s;
 }
 
 // w -= sum_j h_j V_j
@@ -527,8 +531,8 @@ bri_status lanczos(bri_ctx *ctx, bri_prec aprec, double m0, int nlow, int mmax, 
     res = LanczosResult();
     while (m < mmax) {
         T *vj = V + (size_t)m * n;
-        BRI_RETURN_IF(bri_dslash_impl(ctx, tmp, vj, 1, m0, 2, aprec, s));
-        BRI_RETURN_IF(bri_dslash_impl(ctx, w, tmp, 1, m0, 2, aprec, s));
+        BRI_RETURN_IF(bri_dslash_impl(ctx, tmp, vj, 1, m0, HERM, aprec, s));
+        BRI_RETURN_IF(bri_dslash_impl(ctx, w, tmp, 1, m0, HERM, aprec, s));
         res.applies += 2;
         // three-term step against v_{j-1}, v_j, then one Gram-Schmidt pass
         // against the whole basis (its coefficients are at rounding level)
@@ -637,8 +641,8 @@ bri_status poly_apply(bri_ctx *ctx, T *q, const T *v, T *b1, T *b2, T *Bb, T *tm
     // along Z can build up through the recurrence (there the polynomial is
     // evaluated at x = 0, far outside [lo, hi]).
     auto B = [&](T *out, const T *in) -> bri_status {  // out = H^2 in
-        BRI_RETURN_IF(bri_dslash_impl(ctx, tmp, in, 1, m0, 2, prec, s));
-        return bri_dslash_impl(ctx, out, tmp, 1, m0, 2, prec, s);
+        BRI_RETURN_IF(bri_dslash_impl(ctx, tmp, in, 1, m0, HERM, prec, s));
+        return bri_dslash_impl(ctx, out, tmp, 1, m0, HERM, prec, s);
     };
     // b_{N-1} = c_{N-1} v, then b_k = c_k v + 2 t(B) b_{k+1} - b_{k+2} down to k = 1
     k_cheb_step<T><<<nb, VT, 0, s>>>(b1, v, nullptr, nullptr, nullptr, o->coef[N - 1], 0.0, 0.0, 0, 0, n);
@@ -686,13 +690,13 @@ bri_status sign_one(bri_ctx *ctx, double2 *out, const double2 *in, cudaStream_t 
     if (o->prec == BRI_F64) {
         double2 *q = o->v64[1];
         BRI_RETURN_IF(poly_apply<double2>(ctx, q, vp, o->v64[2], o->v64[3], o->v64[4], o->v64[5], o->Z, BRI_F64, s));
-        BRI_RETURN_IF(bri_dslash_impl(ctx, out, q, 1, m0, 2, BRI_F64, s));
+        BRI_RETURN_IF(bri_dslash_impl(ctx, out, q, 1, m0, HERM, BRI_F64, s));
     } else {
         float2 **f = o->v32;
         k_f64_to_f32<<<vec_blocks(n), VT, 0, s>>>(f[0], vp, n);
         BRI_LAUNCHED(ctx);
         BRI_RETURN_IF(poly_apply<float2>(ctx, f[1], f[0], f[2], f[3], f[4], f[5], o->Z32, o->prec, s));
-        BRI_RETURN_IF(bri_dslash_impl(ctx, f[2], f[1], 1, m0, 2, o->prec, s));
+        BRI_RETURN_IF(bri_dslash_impl(ctx, f[2], f[1], 1, m0, HERM, o->prec, s));
         k_f32_to_f64<<<vec_blocks(n), VT, 0, s>>>(out, f[2], n);
         BRI_LAUNCHED(ctx);
     }
@@ -744,7 +748,7 @@ bri_status setup_modes(bri_ctx *ctx, bri_prec aprec, double m0, int nlow, int ma
         return bri_fail(ctx, BRI_ENOTCONV, "overlap setup: low modes of H^2 did not converge; raise max_krylov");
     // Rayleigh-Ritz of H on the Ritz vectors of H^2
     for (int b = 0; b < nlow; b++) {
-        BRI_RETURN_IF(bri_dslash_impl(ctx, HY + (size_t)b * n, Y + (size_t)b * n, 1, m0, 2, aprec, s));
+        BRI_RETURN_IF(bri_dslash_impl(ctx, HY + (size_t)b * n, Y + (size_t)b * n, 1, m0, HERM, aprec, s));
         st.applies++;
         BRI_RETURN_IF(mdot<T>(ctx, YHY + (size_t)b * nlow, Y, n, nlow, HY + (size_t)b * n, nullptr, s));
     }
@@ -760,7 +764,7 @@ bri_status setup_modes(bri_ctx *ctx, bri_prec aprec, double m0, int nlow, int ma
     for (int b = 0; b < nlow; b++) coefs[b] = make_double2(lam[b], 0.0);
     BRI_TRY_CUDA(ctx, cudaMemcpyAsync(o->cdef, coefs.data(), sizeof(double2) * nlow, cudaMemcpyHostToDevice, s));
     for (int b = 0; b < nlow; b++) {
-        BRI_RETURN_IF(bri_dslash_impl(ctx, HY, Z + (size_t)b * n, 1, m0, 2, aprec, s));
+        BRI_RETURN_IF(bri_dslash_impl(ctx, HY, Z + (size_t)b * n, 1, m0, HERM, aprec, s));
         st.applies++;
         BRI_RETURN_IF(maxpy<T>(ctx, HY, Z + (size_t)b * n, n, o->cdef + b, 1, s));
         k_norm_part<T><<<DB, VT, 0, s>>>(HY, n, o->part);

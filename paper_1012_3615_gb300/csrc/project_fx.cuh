@@ -2,8 +2,8 @@
 // unitary start, residual, first update) as integer multiply-adds on two-limb
 // numbers (see dslash_fx.cu), for path sums that are in that form.  About 1,500
 // wide multiply-adds of 4 clocks in place of 440 FP64 operations of 64; what
-// bounds it now is the instruction count (13,000 a matrix, half of them the FP32
-// seed) and their fetch.  16^3x32: 4.50 ms a build, 5.06 with FP64; distance from
+// bounds it now is the instruction count (13,000 a matrix, the FP32 seed among
+// them) and their fetch.  16^3x32: 4.50 ms a build, 5.06 with FP64; distance from
 // the 64-bit eigenvector projection 0.7e-16 rms, it was 1.6e-16.
 // Bounds: rows and columns of A, Y have norms <= 1 (and their rounding), so high
 // limbs are below 2^29 and 2^28 and every sum of six products below 2^62; low

@@ -35,7 +35,7 @@ def _op(L, U, gpu):
 
 
 # volumes on both sides of the lines between 4, 2 and 1 splits of the hop list
-# (2 ceil(V / 32) nrhs warps at 1216 and 2432), ragged last groups
+# (2 ceil(V / 32) warps at 1216 and 2432), ragged last groups
 @pytest.mark.parametrize("L,nrhs", [((3, 3, 3, 3), 1), ((5, 3, 7, 3), 2), ((11, 12, 12, 12), 1), ((11, 11, 12, 13), 1),
                                     ((13, 14, 14, 15), 1), ((14, 14, 14, 15), 1), ((4, 5, 3, 4), 40)])
 def test_splits_against_oracle(gpu, L, nrhs):
@@ -105,3 +105,28 @@ def test_infinities_and_nan_stay_local(gpu):
         far &= (np.minimum(d, np.array(L) - d) > 1).any(1)
     assert np.array_equal(out[far], clean[far])
     assert not np.isfinite(out[~far]).all(axis=(1, 2)).any()
+
+
+def test_capture_and_streams(gpu):
+    """The work space of an apply follows its stream: equal bits from a captured
+    apply, replayed on new input, and from two streams at once."""
+    L = (8, 6, 6, 8)
+    op, _ = _op(L, synth.random_su3_links(L, 0.3, 14), gpu)
+    x = torch.as_tensor(synth.gaussian_spinor(L, 8, 15), device=gpu)
+    want = [op.apply(x[r:r + 1], m0=0.1) for r in range(8)]
+    static = x[:1].clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        out = op.apply(static, m0=0.1)
+    for r in (1, 2, 3):
+        static.copy_(x[r:r + 1])
+        graph.replay()
+        assert torch.equal(out, want[r])
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    got = []
+    for r in range(8):
+        with torch.cuda.stream(streams[r % 2]):
+            got.append(op.apply(x[r:r + 1], m0=0.1))
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
