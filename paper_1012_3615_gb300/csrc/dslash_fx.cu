@@ -448,6 +448,9 @@ __global__ void __maxnreg__(FX_REGS) k_dslash_fx(int mode, const int4 *__restric
             else if (dm < 0) gamma_add(mu, false);
         }
     }
+    // the partner may still be adding to this warp's rows: with some classes
+    // switched off the last pair of a split starts a class of its own
+    asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");
     flush(cls);
     __syncthreads();
     if (split != 0 || !active) return;

@@ -130,3 +130,24 @@ def test_capture_and_streams(gpu):
             got.append(op.apply(x[r:r + 1], m0=0.1))
     torch.cuda.synchronize()
     assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("classes", [(1, 3), (1, 3, 4), (2,), (4,), (1, 2, 4), (2, 3, 4)])
+def test_classes_switched_off(gpu, oracle_weights, classes):
+    """Weights that leave out whole hop classes move the ends of the splits: with
+    classes 1, 3 and with 1, 3, 4 the last pair of a split is the only one of its
+    class, so that its sums follow the class before with no pair between."""
+    lam = [1.9] + [-0.1 * n if n in classes else 0.0 for n in range(1, 5)]
+    rho = [0.0] + [0.3 / n if n in classes else 0.0 for n in range(1, 5)]
+    L = (4, 5, 3, 4)  # four splits
+    U = synth.random_su3_links(L, 0.3, 16)
+    psi = synth.gaussian_spinor(L, 9, 17)
+    op, W = _op(L, U, gpu)
+    op.set_weights(lam, rho)
+    oracle_weights(lam, rho)
+    x = torch.as_tensor(psi, device=gpu)
+    for dag in (False, True):
+        out = op.apply(x, m0=0.1, dagger=dag).cpu().numpy()
+        for r in range(9):
+            ref = oracle.apply(L, AP, W, 0.1, psi[r], dagger=dag)
+            assert np.abs(out[r] - ref).max() <= 4e-15 * np.abs(ref).max()
