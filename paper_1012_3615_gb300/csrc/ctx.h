@@ -29,6 +29,7 @@ struct bri_ctx {
     int4 *hopsfx = nullptr;      // fixed-point copy of hops64 (dslash_fx.cu), [40][9][V]; null without memory for it
     unsigned *fxinfo = nullptr;  // its scale and validity (device)
     bool have_fx = false, fx_tried = false;
+    unsigned fx_attr = 0;        // its kernels whose shared-memory limit is raised on this device
     cudaMemPool_t pool = nullptr;  // stream-ordered work space of the calls, released by bri_destroy
     LinkStore f32, f16;
     LinkStore p32, p16;  // site-pair interleaved copies (full / 2-row, even t extent)

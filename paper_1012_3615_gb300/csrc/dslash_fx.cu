@@ -498,17 +498,21 @@ size_t fx_vp(const Geom &g) { return (size_t)((g.V + 31) & ~31); }
 size_t fx_bytes(const Geom &g, int nrhs) { return (sizeof(int4) * 12 + sizeof(int)) * fx_vp(g) * nrhs; }
 
 template <int S, bool CLOV>
-void fx_launch(int mode, bri_ctx *ctx, const Geom &g, const int4 *P, const int *ex, const void *in, void *out, int nrhs,
-               double diag, const int *skip, cudaStream_t s) {
+bri_status fx_launch(int mode, bri_ctx *ctx, const Geom &g, const int4 *P, const int *ex, const void *in, void *out,
+                     int nrhs, double diag, const int *skip, cudaStream_t s) {
     constexpr int T = FX_T<S>, SPB = T / (2 * S);
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k_dslash_fx<S, CLOV>, cudaFuncAttributeMaxDynamicSharedMemorySize, FX_SMEM<S>);
-        attr = true;
+    // the opt-in to more than 48 KB belongs to the device, as a context does
+    constexpr unsigned bit = 1u << (S + (CLOV ? 8 : 0));
+    if (!(ctx->fx_attr & bit)) {
+        BRI_TRY_CUDA(ctx, cudaFuncSetAttribute(k_dslash_fx<S, CLOV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               FX_SMEM<S>));
+        ctx->fx_attr |= bit;
     }
     const unsigned nb = (unsigned)((g.s1 - g.s0 + SPB - 1) / SPB) * (unsigned)nrhs;
     k_dslash_fx<S, CLOV><<<nb, T, FX_SMEM<S>, s>>>(mode, ctx->hopsfx, ctx->fxinfo, LinkF64{ctx->hops64, g.V}, P, ex,
                                                    (const double2 *)in, (double2 *)out, g, fx_order(g), diag, skip);
+    BRI_LAUNCHED(ctx);
+    return BRI_OK;
 }
 
 }  // namespace
@@ -574,9 +578,12 @@ bri_status bri_dslash_fx(bri_ctx *ctx, const Geom &g, void *out, const void *in,
     const bool all = g.s0 == 0 && g.s1 == g.V;
     const long long span = (long long)g.s1 - g.s0 + 2 * S3;
     const int n = all || span >= g.V ? g.V : (int)span, first = n == g.V ? 0 : (g.s0 - S3 + g.V) % g.V;
-    k_fx_spinor<<<dim3((unsigned)((n + 127) / 128), (unsigned)nrhs), 128, 0, s>>>((const double2 *)in, P, ex, g.V,
-                                                                                  first, n, skip);
-    BRI_LAUNCHED(ctx);
+    auto convert = [&]() -> bri_status {
+        k_fx_spinor<<<dim3((unsigned)((n + 127) / 128), (unsigned)nrhs), 128, 0, s>>>((const double2 *)in, P, ex, g.V,
+                                                                                      first, n, skip);
+        BRI_LAUNCHED(ctx);
+        return BRI_OK;
+    };
     // splits of the hop list, so that the 608 schedulers have two warps or more;
     // by the lattice alone, so that a right-hand side gives the same bits alone, in
     // a batch and on a range of sites
@@ -584,9 +591,10 @@ bri_status bri_dslash_fx(bri_ctx *ctx, const Geom &g, void *out, const void *in,
     const int S = warps >= 2432 ? 1 : warps >= 1216 ? 2 : 4;
     auto launch = g.clov64 ? (S == 1 ? fx_launch<1, true> : S == 2 ? fx_launch<2, true> : fx_launch<4, true>)
                            : (S == 1 ? fx_launch<1, false> : S == 2 ? fx_launch<2, false> : fx_launch<4, false>);
-    launch(mode, ctx, g, P, ex, in, out, nrhs, diag, skip, s);
-    BRI_LAUNCHED(ctx);
+    bri_status st = convert();
+    if (st == BRI_OK) st = launch(mode, ctx, g, P, ex, in, out, nrhs, diag, skip, s);
     if (own) BRI_TRY_CUDA(ctx, cudaFreeAsync(own, s));
+    BRI_RETURN_IF(st);
     *ndone += nrhs;
     return BRI_OK;
 }

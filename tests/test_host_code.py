@@ -1,0 +1,97 @@
+"""The library's host code without a GPU: its objects linked with a stand-in for
+the CUDA runtime (fake_cudart.cpp) that records launches, counts memory and
+refuses what the runtime refuses.  Nothing is computed."""
+import ctypes
+import glob
+import os
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    from paper_1012_3615_gb300 import abi, build
+
+    build.build()
+    out = str(tmp_path_factory.mktemp("fake") / "libbrillouin_fake.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build_nvcc()))), "include")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", cuda, "-o", out,
+                    os.path.join(HERE, "fake_cudart.cpp")] + sorted(glob.glob(os.path.join(build.BUILD, "*.o"))),
+                   check=True, capture_output=True, text=True)
+    lib = ctypes.CDLL(out)
+    for name, (res, args) in abi.SIGNATURES.items():
+        f = getattr(lib, name)
+        f.restype, f.argtypes = res, args
+    lib.fake_log.restype = ctypes.c_char_p
+    lib.fake_used.restype = ctypes.c_size_t
+    lib.fake_budget.argtypes = [ctypes.c_size_t]
+    lib.fake_refuse.argtypes = [ctypes.c_long, ctypes.c_long]
+    lib.cudaMemGetInfo.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
+    lib.cudaStreamBeginCapture.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    lib.cudaStreamEndCapture.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
+    lib.cudaGraphInstantiate.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_ulonglong]
+    for n in ("cudaGraphLaunch",):
+        getattr(lib, n).argtypes = [ctypes.c_void_p, ctypes.c_void_p]
+    for n in ("cudaGraphDestroy", "cudaGraphExecDestroy"):
+        getattr(lib, n).argtypes = [ctypes.c_void_p]
+    return lib
+
+
+def build_nvcc():
+    import shutil
+
+    from paper_1012_3615_gb300 import build
+
+    return shutil.which(build.NVCC) or "/usr/local/cuda/bin/nvcc"
+
+
+@pytest.fixture
+def fake(lib):
+    lib.fake_reset()
+    made = []
+
+    class Fake:
+        def __init__(self):
+            self.lib = lib
+
+        def op(self, L=(8, 8, 8, 8), device=0, comp=0, prec=0):
+            """a context on a device with hopping fields built from links somewhere"""
+            from paper_1012_3615_gb300 import abi
+
+            lib.fake_device(device)
+            lat = abi.bri_lattice((ctypes.c_int * 4)(*L), (ctypes.c_int * 4)(1, 1, 1, -1))
+            h = ctypes.c_void_p()
+            assert lib.bri_create(ctypes.byref(lat), ctypes.byref(h)) == 0
+            made.append((device, h))
+            return h
+
+        def apply(self, h, nrhs=1, prec=0, stream=None):
+            return lib.bri_apply(h, 1 << 50, 1 << 56, nrhs, 0.1, 0, prec, stream)
+
+        def build(self, h, prec=0, comp=0):
+            return lib.bri_build_hops(h, 1 << 57, prec, comp, None)
+
+        def log(self):
+            text = lib.fake_log().decode().split("\n")
+            lib.fake_clear_log()
+            return [t for t in text if t]
+
+    yield Fake()
+    lib.fake_reset()
+    for device, h in made:
+        lib.fake_device(device)
+        lib.bri_destroy(h)
+    assert lib.fake_used() == 0  # nothing outlives its context
+
+
+@pytest.mark.parametrize("L", [(8, 8, 8, 8), (11, 12, 12, 12), (16, 16, 16, 32)])
+def test_fp64_apply_on_two_devices(fake, L):
+    """the opt-in to the FP64 apply's shared memory belongs to each device"""
+    for device in (0, 1):
+        h = fake.op(L, device)
+        assert fake.build(h) == 0
+        assert fake.apply(h) == 0, fake.lib.bri_last_error(h)
+        assert any("k_dslash_fx" in t for t in fake.log())
