@@ -5,18 +5,18 @@
 // the 17,016 FP64 operations of a site, are taken on two-limb fixed-point
 // numbers with exact integer sums:
 //
-//   link entries  w  = fw 2^(we - 62),    fw = (wh + wl) 2^32, |wh| <= 2^30
+//   link entries  w  = fw 2^-62,          fw = (wh + wl) 2^32, |wh| <= 2^30
 //   spinors       p  = fp 2^(e(y) - 60),  fp = (ph + pl) 2^32, |ph| <= 2^28,
 //                 e(y) the exponent of the largest component of site y
-//   products      w p = (wh ph + wh pl + wl ph) 2^(we + e - 58)
+//   products      w p = (wh ph + wh pl + wl ph) 2^(e - 58)
 //
 // with integers wh, ph and |wl|, |pl| <= 1/2 kept as FP32 numbers; wl pl is
 // below 2^-60 of the largest product and dropped.  A 64-bit accumulator holds
 // the six high products of a colour row exactly; the twelve cross products, at
 // most 2^-30 of the largest product, are summed in packed FP32 FMAs (rounded to
 // 2^-24 of themselves) and added as an integer: rows and columns of a link
-// have norm <= 2^we, so |sum wh pl + wl ph| <= 7.9 2^28 < 2^31.  The row is
-// rounded to the unit 2^(we + X_n - 58) of its hop class n, X_n = the largest
+// have norm <= 1, so |sum wh pl + wl ph| <= 7.9 2^28 < 2^31.  The row is
+// rounded to the unit 2^(X_n - 58) of its hop class n, X_n = the largest
 // e(y) of the class's neighbours + h_n, and the rows are summed as 64-bit
 // integers: once with the class weight lambda and once through gamma_d (entries
 // +-1, +-i: additions only).  A class sum holds at most 8, 48, 96, 64 rows
@@ -34,8 +34,8 @@
 // scoreboard and fixed-latency waits the top stalls).
 //
 // A site that meets an infinity, a NaN or an exponent outside the range of
-// FP64 scales takes the FP64 loop (fx_slow), as every site does when the links
-// hold such an entry.
+// FP64 scales takes the FP64 loop (fx_slow), as every site does when a link is
+// not of unit norm or a field holds a NaN.
 #include <algorithm>
 #include <string>
 
@@ -84,7 +84,7 @@ __global__ void k_fx_spinor(const double2 *__restrict__ in, int4 *__restrict__ p
 
 // one colour row of W p (SGN = 1, w = row c of W) or W^dagger p (SGN = -1,
 // w = column c of W) for the two spins in p, rounded to units of
-// 2^(we + e - 58 + sh).  pf: the spinor's high limbs as FP32 numbers
+// 2^(e - 58 + sh).  pf: the spinor's high limbs as FP32 numbers
 template <int SGN>
 BRI_D void fx_row(const int4 w[3], const int4 p[6], const float2 pf[6], int sh, long long half, long long re[2],
                   long long im[2]) {
@@ -123,66 +123,104 @@ BRI_D void fx_negate(int4 p[6]) {
         p[k] = make_int4(-p[k].x, p[k].y ^ (int)0x80000000, -p[k].z, p[k].w ^ (int)0x80000000);
 }
 
-// the FP64 loop for one site, whole spinor (the arithmetic of hop_pair with
-// run-time offsets)
+// out = diag p + v, the clover term and the sign of mode 2, for the spins 2h, 2h + 1
+template <bool CLOV>
+BRI_D void fx_finish(int mode, const double2 *__restrict__ in, double2 *__restrict__ out, int site, int h,
+                     const Geom &g, double diag, const double2 v[6]) {
+    double2 o[6], p[6];
+#pragma unroll
+    for (int i = 0; i < 6; i++) p[i] = in[(size_t)site * 12 + 6 * h + i];
+#pragma unroll
+    for (int i = 0; i < 6; i++) o[i] = make_double2(fma(diag, p[i].x, v[i].x), fma(diag, p[i].y, v[i].y));
+    if constexpr (CLOV) {
+        double2 c[18];
+#pragma unroll
+        for (int e = 0; e < 18; e++) c[e] = g.clov64[(size_t)(18 * h + e) * g.V + site];
+        clover_block(c, p, o);
+    }
+    const double s5 = mode == 2 && h == 1 ? -1.0 : 1.0;
+#pragma unroll
+    for (int i = 0; i < 6; i++) out[(size_t)site * 12 + 6 * h + i] = make_double2(s5 * o[i].x, s5 * o[i].y);
+}
+
+// The FP64 loop (the arithmetic of hop_pair with run-time offsets) for one site:
+// its threads part = 2 split + h share the list, leave their sums in sum (entry i
+// of thread part at [12 part + i][32]) and threads 0 and 1 add them.  Called by whole
+// blocks; slow: this thread's site takes part.  Bound by the FP64 pipe; every site
+// this way (links of norm 1.5) on 8^4, 12^4, 16^3x32: 0.17, 0.75, 3.99 ms; one
+// thread with the whole list 0.61, 1.29, 4.13; the FP64 kernel 0.63, 1.17, 4.12
+template <bool CLOV>
 __device__ __noinline__ void fx_slow(int mode, const LinkF64 &ll, const double2 *__restrict__ in,
-                                     double2 *__restrict__ out, int site, const Geom &g, double diag) {
-    int x[4];
-    const SiteNb nb = site_nb(g, site, x);
-    AccD acc;
-    for (int i = 0; i < 12; i++) acc.a[i] = make_double2(0.0, 0.0);
-    const double rsign = mode == 1 ? -1.0 : 1.0;
+                                     double2 *__restrict__ out, double2 *sum, int site, const Geom &g, double diag,
+                                     int part, int parts, bool slow) {
+    if (slow) {
+        int x[4];
+        const SiteNb nb = site_nb(g, site, x);
+        AccD acc;
+#pragma unroll
+        for (int i = 0; i < 12; i++) acc.a[i] = make_double2(0.0, 0.0);
+        const double rsign = mode == 1 ? -1.0 : 1.0;
 #pragma unroll 1
-    for (int t = 0; t < g.nhop; t++) {
-        const HopArg &h = g.hop[t];
-        int yf, yb;
-        float phf, phb;
-        hop_nb(h.dm, site, nb, yf, phf, yb, phb);
-        const int n = abs(h.dm[0]) + abs(h.dm[1]) + abs(h.dm[2]) + abs(h.dm[3]);
-        const double q = (double)(phf * phb), L = g.lamd[n] * (double)phf, R = g.rhod[n] * (double)phf * rsign;
-        double2 cf[12];
-        {
-            const M3<double2> W = ll.load(h.j, site);
-            double2 p[12];
-            load_spinor(in + (size_t)yf * 12, p);
+        for (int t = part * g.nhop / parts; t < (part + 1) * g.nhop / parts; t++) {
+            const HopArg &h = g.hop[t];
+            int yf, yb;
+            float phf, phb;
+            hop_nb(h.dm, site, nb, yf, phf, yb, phb);
+            const int n = abs(h.dm[0]) + abs(h.dm[1]) + abs(h.dm[2]) + abs(h.dm[3]);
+            const double q = (double)(phf * phb), L = g.lamd[n] * (double)phf, R = g.rhod[n] * (double)phf * rsign;
+            double2 cf[12];
+            {
+                const M3<double2> W = ll.load(h.j, site);
+                double2 p[12];
+                load_spinor(in + (size_t)yf * 12, p);
 #pragma unroll
-            for (int sp = 0; sp < 4; sp++) mv64<1>(W, p, sp, cf + 3 * sp);
-        }
-        const M3<double2> W = ll.load(h.j, yb);
-        double2 p[12];
-        load_spinor(in + (size_t)yb * 12, p);
-#pragma unroll
-        for (int sp = 0; sp < 4; sp++) {
-            double2 cb[3];
-            mv64<-1>(W, p, sp, cb);
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                double2 &f = cf[3 * sp + c];
-                const double sx = fma(q, cb[c].x, f.x), sy = fma(q, cb[c].y, f.y);
-                f.x = fma(-q, cb[c].x, f.x);
-                f.y = fma(-q, cb[c].y, f.y);
-                acc.a[3 * sp + c].x = fma(L, sx, acc.a[3 * sp + c].x);
-                acc.a[3 * sp + c].y = fma(L, sy, acc.a[3 * sp + c].y);
+                for (int sp = 0; sp < 4; sp++) mv64<1>(W, p, sp, cf + 3 * sp);
             }
-        }
-#pragma unroll
-        for (int mu = 0; mu < 4; mu++) {
-            if (h.dm[mu] == 0) continue;
-            const double rd = R * (double)h.dm[mu];
+            const M3<double2> W = ll.load(h.j, yb);
+            double2 p[12];
+            load_spinor(in + (size_t)yb * 12, p);
 #pragma unroll
             for (int sp = 0; sp < 4; sp++) {
-                const int s = gcol(mu, sp);
-                const int gr = gre(mu, s), gi = gim(mu, s);
+                double2 cb[3];
+                mv64<-1>(W, p, sp, cb);
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
-                    if (gr != 0) acc_re(acc.a[3 * s + c], rd * (double)gr, cf[3 * sp + c]);
-                    else acc_im(acc.a[3 * s + c], rd * (double)gi, cf[3 * sp + c]);
+                    double2 &f = cf[3 * sp + c];
+                    const double sx = fma(q, cb[c].x, f.x), sy = fma(q, cb[c].y, f.y);
+                    f.x = fma(-q, cb[c].x, f.x);
+                    f.y = fma(-q, cb[c].y, f.y);
+                    acc.a[3 * sp + c].x = fma(L, sx, acc.a[3 * sp + c].x);
+                    acc.a[3 * sp + c].y = fma(L, sy, acc.a[3 * sp + c].y);
+                }
+            }
+#pragma unroll
+            for (int mu = 0; mu < 4; mu++) {
+                if (h.dm[mu] == 0) continue;
+                const double rd = R * (double)h.dm[mu];
+#pragma unroll
+                for (int sp = 0; sp < 4; sp++) {
+                    const int s = gcol(mu, sp);
+                    const int gr = gre(mu, s), gi = gim(mu, s);
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        if (gr != 0) acc_re(acc.a[3 * s + c], rd * (double)gr, cf[3 * sp + c]);
+                        else acc_im(acc.a[3 * s + c], rd * (double)gi, cf[3 * sp + c]);
+                    }
                 }
             }
         }
+#pragma unroll
+        for (int i = 0; i < 12; i++) sum[32 * (12 * part + i)] = acc.a[i];
     }
-    if (g.clov64) dslash_finish<double2, true>(mode, in, out, site, g, diag, acc);
-    else dslash_finish<double2, false>(mode, in, out, site, g, diag, acc);
+    __syncthreads();
+    if (!slow || part > 1) return;
+    double2 v[6];
+#pragma unroll
+    for (int i = 0; i < 6; i++) {
+        v[i] = make_double2(0.0, 0.0);
+        for (int k = 0; k < parts; k++) v[i] = cadd(v[i], sum[32 * (12 * k + 6 * part + i)]);
+    }
+    fx_finish<CLOV>(mode, in, out, site, part, g, diag, v);
 }
 
 // One thread per (site, chirality, split): a warp holds 32 sites, its spins
@@ -291,13 +329,10 @@ __global__ void __maxnreg__(FX_REGS) k_dslash_fx(int mode, const int4 *__restric
 #pragma unroll
     for (int k = 0; k < 4; k++) se[k * T + tid] = X[k];
     __syncthreads();
-    const int we = fx_we(info[0]);
-    bool slow = info[1] != 0;
 #pragma unroll
     for (int k = 0; k < 4; k++) {
         for (int q = 0; q < 2 * S; q++) X[k] = max(X[k], se[k * T + (sgrp * 2 * S + q) * 32 + lane]);
         X[k] = X[k] == FX_ZERO ? 0 : X[k] + fx_head(k + 1);
-        slow = slow || we + X[k] > 900 || we + X[k] < -900;
     }
     __syncthreads();
     int *sx = (int *)(fx_sm + T * 12 * 8 + (T / 64) * 2 * FX_STAGE * 16) + tid;  // the four exponents
@@ -314,11 +349,11 @@ __global__ void __maxnreg__(FX_REGS) k_dslash_fx(int mode, const int4 *__restric
         La[i] = Ga[i] = 0;
         sm[i * T + tid] = 0.0;
     }
-    const int i0 = split * nh / S, i1 = (split + 1) * nh / S;
+    const int i0 = split * nh / S, i1 = info[1] ? i0 : (split + 1) * nh / S;
     int cls = i0 < i1 ? ord.cls[i0] : 1;
     int Xn = sx[(cls - 1) * T];
     auto flush = [&](int n) {
-        const double scale = slow ? 0.0 : __hiloint2double((1023 + we + Xn - FX_AB) << 20, 0);
+        const double scale = __hiloint2double((1023 + Xn - FX_AB) << 20, 0);
         const double cl = g.lamd[n] * scale, cg = g.rhod[n] * (mode == 1 ? -scale : scale);
 #pragma unroll
         for (int i = 0; i < 12; i++) sm[i * T + tid] = fma(fx_double(La[i], 0), cl, sm[i * T + tid]);
@@ -453,32 +488,26 @@ __global__ void __maxnreg__(FX_REGS) k_dslash_fx(int mode, const int4 *__restric
     asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");
     flush(cls);
     __syncthreads();
-    if (split != 0 || !active) return;
-    if (slow) {
-        if (h == 0) fx_slow(mode, ll, in, out, site, g, diag);
-        return;
-    }
-    double2 o[6], p[6];
+    // a site out of the fixed-point range: its sums so far are worth nothing
+    bool slow = info[1] != 0;
 #pragma unroll
-    for (int i = 0; i < 6; i++) p[i] = in[(size_t)site * 12 + 6 * h + i];
+    for (int k = 0; k < 4; k++) slow = slow || abs(sx[k * T]) > 900;
+    if (split == 0 && active && !slow) {
+        double2 v[6];
 #pragma unroll
-    for (int i = 0; i < 6; i++) {
-        double2 v = make_double2(0.0, 0.0);
-        for (int k = 0; k < S; k++) {
-            v.x += sm[(2 * i) * T + tid + 64 * k];
-            v.y += sm[(2 * i + 1) * T + tid + 64 * k];
+        for (int i = 0; i < 6; i++) {
+            v[i] = make_double2(0.0, 0.0);
+            for (int k = 0; k < S; k++) {
+                v[i].x += sm[(2 * i) * T + tid + 64 * k];
+                v[i].y += sm[(2 * i + 1) * T + tid + 64 * k];
+            }
         }
-        o[i] = make_double2(fma(diag, p[i].x, v.x), fma(diag, p[i].y, v.y));
+        fx_finish<CLOV>(mode, in, out, site, h, g, diag, v);
     }
-    if constexpr (CLOV) {
-        double2 c[18];
-#pragma unroll
-        for (int e = 0; e < 18; e++) c[e] = g.clov64[(size_t)(18 * h + e) * V + site];
-        clover_block(c, p, o);
-    }
-    const double s5 = mode == 2 && h == 1 ? -1.0 : 1.0;
-#pragma unroll
-    for (int i = 0; i < 6; i++) out[(size_t)site * 12 + 6 * h + i] = make_double2(s5 * o[i].x, s5 * o[i].y);
+    if (!__syncthreads_or(slow && active)) return;
+    // the spinor stages of the group's 2 S warps lie behind one another
+    double2 *sum = (double2 *)(fx_sm + T * (12 * 8 + 4 * 4) + (T / 64) * 2 * FX_STAGE * 16) + sgrp * 2 * S * 12 * 32 + lane;
+    fx_slow<CLOV>(mode, ll, in, out, sum, site, g, diag, 2 * split + h, 2 * S, slow && active);
 }
 
 FxOrder fx_order(const Geom &g) {

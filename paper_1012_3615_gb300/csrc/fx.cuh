@@ -72,33 +72,22 @@ BRI_D unsigned norm_hi(const double2 w[9]) {
     }
     return m;
 }
+// Links of unit norm: info[0] and info[2] hold the largest norm of a row or
+// column and the complement of the smallest.  Their limbs keep every digit that
+// matters; with one exponent for all, a link of another size would take digits
+// from the rest of the lattice, so that others keep their FP64 numbers
 constexpr unsigned FX_ONE = 0x3ff00010u;  // 1 + 2^-16: a unitary matrix and its rounding
-// exponent we: norms are at most 2^we
-BRI_D int fx_we(unsigned hi) {
-    if (hi <= FX_ONE) return 0;
-    return ((int)(hi >> 20) - 1022 + 1) >> 1;  // |.|^2 < 2^(exponent field - 1022)
-}
+BRI_D bool fx_unit_links(const unsigned *info) { return info[0] <= FX_ONE && ~info[2] >= 0x3fefffe0u; }
 
 // limb copies are stored in blocks of 32 sites, [..][Vp/32][entries][32] with Vp
 // = V rounded up to 32: the entries of a site lie at fixed offsets from its first
 BRI_D size_t fx_at(int site, int entries) { return (size_t)(site >> 5) * (32 * entries) + (site & 31); }
 
-// the limbs of a unitary field matrix of one site (o: the field's start)
-BRI_D void fx_store_unitary(const double2 w[9], int4 *o, int site, int we) {
+// the limbs of a field matrix of one site (o: the field's start)
+BRI_D void fx_store(const double2 w[9], int4 *o, int site) {
     o += fx_at(site, 9);
 #pragma unroll
-    for (int e = 0; e < 9; e++) o[32 * e] = fx_split_f(w[e].x, w[e].y, FX_WB - we);
-}
-// the limbs of any field matrix of one site; info[1] = 1 if it does not fit
-BRI_D void fx_store(const double2 w[9], int4 *o, int site, unsigned *info) {
-    const int we = fx_we(info[0]);
-    if (we > 400 || norm_hi(w) > max(info[0], FX_ONE)) {  // infinities, NaN or huge entries
-        info[1] = 1;
-        return;
-    }
-    o += fx_at(site, 9);
-#pragma unroll
-    for (int e = 0; e < 9; e++) o[32 * e] = fx_split_f(w[e].x, w[e].y, FX_WB - we);
+    for (int e = 0; e < 9; e++) o[32 * e] = fx_split_f(w[e].x, w[e].y, FX_WB);
 }
 
 }  // namespace bri

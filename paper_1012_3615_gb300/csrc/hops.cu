@@ -38,10 +38,8 @@ namespace {
 // 16^3x32: 0.90 ms (FP64 products: 2.7), the whole build 5.1 ms (7.7), of which
 // the projection takes 3.7.
 // Links whose rows and columns are not of norm 1 to 2^-16 (only their user
-// knows what they are) take the FP64 form: info[0] and info[2] hold the largest
-// and the smallest norm, and every kernel takes the same branch.
+// knows what they are) take the FP64 form; every kernel takes the same branch.
 constexpr int PS_B = 61;
-BRI_D bool paths_fixed(const unsigned *info) { return info[0] <= FX_ONE && ~info[2] >= 0x3fefffe0u; }
 
 // smallest |row|^2, |column|^2 of a matrix, as the high word of a double
 BRI_D unsigned norm_lo(const double2 w[9]) {
@@ -53,8 +51,8 @@ BRI_D unsigned norm_lo(const double2 w[9]) {
     }
     return m;
 }
-// info[0]: largest norm of the links (the other fields are unitary), info[1]: 1
-// if a field matrix does not fit its limbs, info[2]: complement of the smallest
+// info[0]: largest norm of the links, info[2]: complement of the smallest;
+// info[1] becomes 1 where the apply has to read the FP64 fields
 __global__ void k_link_norms(const double2 *__restrict__ U, int n, unsigned *info) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     unsigned m = 0, l = 0;
@@ -135,7 +133,7 @@ __global__ void k_path_level(int n, FieldList f, double2 *__restrict__ A, const 
     const int j = f.j[blockIdx.y], k = canon_k(j), V = g.V;
     int x[4];
     const SiteNb nb = site_nb(g, site, x);
-    if (paths_fixed(info)) {
+    if (fx_unit_links(info)) {
         long long sum[18];
 #pragma unroll
         for (int i = 0; i < 18; i++) sum[i] = 0;
@@ -179,7 +177,7 @@ __global__ void k_path_links(const double2 *__restrict__ U, double2 *__restrict_
                              const unsigned *__restrict__ info) {
     const int site = blockIdx.x * blockDim.x + threadIdx.x, mu = blockIdx.y;
     if (site >= V) return;
-    const bool fixed = paths_fixed(info);
+    const bool fixed = fx_unit_links(info);
     int4 *o = reinterpret_cast<int4 *>(A);
 #pragma unroll
     for (int e = 0; e < 9; e++) {
@@ -194,7 +192,7 @@ __global__ void k_path_links(const double2 *__restrict__ U, double2 *__restrict_
 __global__ void k_path_f64(const double2 *__restrict__ U, double2 *__restrict__ A, int V,
                            const unsigned *__restrict__ info) {
     const int site = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-    if (site >= V || !paths_fixed(info)) return;
+    if (site >= V || !fx_unit_links(info)) return;
     const int n = off_class(canon_k(j));
     if (n == 1) {
         const int mu = j == 0 ? 0 : j == 2 ? 1 : j == 8 ? 2 : 3;
@@ -219,14 +217,15 @@ __global__ void __launch_bounds__(128, 3) k_project_hops(const double2 *__restri
     const int site = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y;
     if (site >= V) return;
+    const bool fixed = fx_unit_links(info);
     M3<double2> w;
     bool unitary = false;
     if (off_class(canon_k(j)) == 1) {
         const int mu = j == 0 ? 0 : j == 2 ? 1 : j == 8 ? 2 : 3;
+        unitary = fixed;
 #pragma unroll
         for (int e = 0; e < 9; e++) w.e[e] = U[((size_t)site * 4 + mu) * 9 + e];
     } else {
-        const bool fixed = paths_fixed(info);
         if (fixed) {
             const int4 *p = reinterpret_cast<const int4 *>(hops64);
             int4 A[9];
@@ -234,14 +233,16 @@ __global__ void __launch_bounds__(128, 3) k_project_hops(const double2 *__restri
             for (int e = 0; e < 9; e++) A[e] = p[((size_t)j * 9 + e) * V + site];
             unitary = project_fast_fx(A, w);
         }
-        if (!unitary) w = project_su3(path_load(hops64, j, V, site, fixed));
+        if (!unitary) {
+            w = project_su3(path_load(hops64, j, V, site, fixed));
+            unitary = norm_hi(w.e) <= FX_ONE;  // not of a NaN
+        }
     }
 #pragma unroll
     for (int e = 0; e < 9; e++) hops64[((size_t)j * 9 + e) * V + site] = w.e[e];
     if (!fx) return;
-    int4 *o = fx + (size_t)j * 9 * ((V + 31) & ~31);
-    if (unitary) fx_store_unitary(w.e, o, site, fx_we(info[0]));
-    else fx_store(w.e, o, site, info);
+    if (!fixed || !unitary) info[1] = 1;
+    else fx_store(w.e, fx + (size_t)j * 9 * ((V + 31) & ~31), site);
 }
 
 __global__ void k_project_batch(const M3<double2> *__restrict__ A, M3<double2> *__restrict__ Y, long n) {

@@ -151,3 +151,33 @@ def test_classes_switched_off(gpu, oracle_weights, classes):
         for r in range(9):
             ref = oracle.apply(L, AP, W, 0.1, psi[r], dagger=dag)
             assert np.abs(out[r] - ref).max() <= 4e-15 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("size", [2.0**10, 2.0**30, 2.0**62, 2.0**200])
+def test_one_large_link_stays_local(gpu, size):
+    """a link of any norm takes no digits from the sites that do not see it, nor
+    from the unitary fields of those that do"""
+    L = (6, 5, 7, 6)
+    U = synth.random_su3_links(L, 0.3, 18)
+    psi = synth.gaussian_spinor(L, 1, 19)
+    U[100, 1] *= size
+    op, W = _op(L, U, gpu)
+    out = op.apply(torch.as_tensor(psi, device=gpu), m0=0.1).cpu().numpy()[0]
+    ref = oracle.apply(L, AP, W, 0.1, psi[0])
+    assert (np.abs(out - ref) <= 4e-15 * np.abs(ref).max(axis=(1, 2), keepdims=True)).all()
+
+
+@pytest.mark.parametrize("scale", [1e-3, 1e-9, 1e-100])
+def test_small_links_keep_their_digits(gpu, oracle_weights, scale):
+    """links of a small norm where they are the whole result: Wilson weights,
+    diagonal zero"""
+    L = (4, 3, 5, 4)
+    lam, rho = [4.0, -0.5, 0, 0, 0], [0, 0.5, 0, 0, 0]
+    U = scale * synth.random_su3_links(L, 0.3, 20)
+    psi = synth.gaussian_spinor(L, 1, 21)
+    op, W = _op(L, U, gpu)
+    op.set_weights(lam, rho)
+    oracle_weights(lam, rho)
+    out = op.apply(torch.as_tensor(psi, device=gpu), m0=-4.0).cpu().numpy()[0]
+    ref = oracle.apply(L, AP, W, -4.0, psi[0])
+    assert np.abs(out - ref).max() <= 4e-15 * np.abs(ref).max()
