@@ -27,7 +27,7 @@ struct bri_ctx {
     double2 *hops64 = nullptr;  // FP64 hops, [40][9][V]
     bool have64 = false;
     int4 *hopsfx = nullptr;      // fixed-point copy of hops64 (dslash_fx.cu), [40][9][V]; null without memory for it
-    unsigned *fxinfo = nullptr;  // its scale and validity (device)
+    unsigned *fxinfo = nullptr;  // whether the links are not unitary, the copy not usable (device)
     bool have_fx = false, fx_tried = false;
     unsigned fx_attr = 0;        // its kernels whose shared-memory limit is raised on this device
     cudaMemPool_t pool = nullptr;  // stream-ordered work space of the calls, released by bri_destroy

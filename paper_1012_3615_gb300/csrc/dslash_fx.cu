@@ -35,7 +35,8 @@
 //
 // A site that meets an infinity, a NaN or an exponent outside the range of
 // FP64 scales takes the FP64 loop (fx_slow), as every site does when a link is
-// not of unit norm or a field holds a NaN.
+// not unitary (one exponent serves all links: one of another size would take
+// digits from the rest of the lattice) or a field holds a NaN.
 #include <algorithm>
 #include <string>
 
@@ -558,7 +559,7 @@ bri_status bri_fx_reserve(bri_ctx *ctx) {
             ctx->hopsfx = nullptr;
         }
     }
-    if (!ctx->fxinfo) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->fxinfo, 3 * sizeof(unsigned)));
+    if (!ctx->fxinfo) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->fxinfo, 2 * sizeof(unsigned)));
     if (!ctx->pool) {
         cudaMemPoolProps pp{};
         pp.allocType = cudaMemAllocationTypePinned;

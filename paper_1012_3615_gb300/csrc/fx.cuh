@@ -72,12 +72,7 @@ BRI_D unsigned norm_hi(const double2 w[9]) {
     }
     return m;
 }
-// Links of unit norm: info[0] and info[2] hold the largest norm of a row or
-// column and the complement of the smallest.  Their limbs keep every digit that
-// matters; with one exponent for all, a link of another size would take digits
-// from the rest of the lattice, so that others keep their FP64 numbers
 constexpr unsigned FX_ONE = 0x3ff00010u;  // 1 + 2^-16: a unitary matrix and its rounding
-BRI_D bool fx_unit_links(const unsigned *info) { return info[0] <= FX_ONE && ~info[2] >= 0x3fefffe0u; }
 
 // limb copies are stored in blocks of 32 sites, [..][Vp/32][entries][32] with Vp
 // = V rounded up to 32: the entries of a site lie at fixed offsets from its first

@@ -37,38 +37,42 @@ namespace {
 // is scaled by 2^-1, 2^-2, 2^-2 (n = 2, 3, 4) instead of 1/n.  Known to 2^-57.
 // 16^3x32: 0.90 ms (FP64 products: 2.7), the whole build 5.1 ms (7.7), of which
 // the projection takes 3.7.
-// Links whose rows and columns are not of norm 1 to 2^-16 (only their user
-// knows what they are) take the FP64 form; every kernel takes the same branch.
+// Links that are not unitary to 2^-16 (only their user knows what they are)
+// take the FP64 form; every kernel takes the same branch.  Norms alone would not
+// do: products of matrices with rows and columns of norm 1 grow to 1.73^n.
 constexpr int PS_B = 61;
 
-// smallest |row|^2, |column|^2 of a matrix, as the high word of a double
-BRI_D unsigned norm_lo(const double2 w[9]) {
-    unsigned m = 0xffffffffu;
+// unitary to 2^-16: rows of norm 1 and orthogonal, in FP32 (with the norms in
+// FP64 a build of 16^3x32 took 62 us more).  to_f32 wants numbers in its range
+BRI_D bool unitary_link(const double2 w[9]) {
+    float2 f[9];
+    unsigned m = 0;
 #pragma unroll
-    for (int i = 0; i < 3; i++) {
-        m = min(m, abs_hi(cnorm2(w[3 * i]) + cnorm2(w[3 * i + 1]) + cnorm2(w[3 * i + 2])));
-        m = min(m, abs_hi(cnorm2(w[i]) + cnorm2(w[3 + i]) + cnorm2(w[6 + i])));
+    for (int e = 0; e < 9; e++) {
+        m = max(m, max(abs_hi(w[e].x), abs_hi(w[e].y)));
+        f[e] = to_f32(w[e]);
     }
-    return m;
+    bool ok = m <= FX_ONE;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = i; j < 3; j++) {
+            float2 d = make_float2(i == j ? -1.f : 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 3; k++) d = cadd(d, cmulc(f[3 * i + k], f[3 * j + k]));
+            ok = ok && d.x * d.x + d.y * d.y <= 0x1p-32f;
+        }
+    return ok;
 }
-// info[0]: largest norm of the links, info[2]: complement of the smallest;
-// info[1] becomes 1 where the apply has to read the FP64 fields
-__global__ void k_link_norms(const double2 *__restrict__ U, int n, unsigned *info) {
+// info[0] becomes 1 if a link is not unitary, info[1] if the apply has to read
+// the FP64 fields
+__global__ void k_link_check(const double2 *__restrict__ U, int n, unsigned *info) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned m = 0, l = 0;
-    if (i < n) {
-        double2 w[9];
+    if (i >= n) return;
+    double2 w[9];
 #pragma unroll
-        for (int e = 0; e < 9; e++) w[e] = U[(size_t)i * 9 + e];
-        m = norm_hi(w);
-        l = ~norm_lo(w);
-    }
-    m = __reduce_max_sync(0xffffffffu, m);
-    l = __reduce_max_sync(0xffffffffu, l);
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(info, m);
-        atomicMax(info + 2, l);
-    }
+    for (int e = 0; e < 9; e++) w[e] = U[(size_t)i * 9 + e];
+    if (!unitary_link(w)) info[0] = 1;
 }
 
 template <bool DAG> BRI_D M3<int4> field_load_fx(const double2 *__restrict__ A, int j, int V, int site) {
@@ -133,7 +137,7 @@ __global__ void k_path_level(int n, FieldList f, double2 *__restrict__ A, const 
     const int j = f.j[blockIdx.y], k = canon_k(j), V = g.V;
     int x[4];
     const SiteNb nb = site_nb(g, site, x);
-    if (fx_unit_links(info)) {
+    if (info[0] == 0) {
         long long sum[18];
 #pragma unroll
         for (int i = 0; i < 18; i++) sum[i] = 0;
@@ -177,7 +181,7 @@ __global__ void k_path_links(const double2 *__restrict__ U, double2 *__restrict_
                              const unsigned *__restrict__ info) {
     const int site = blockIdx.x * blockDim.x + threadIdx.x, mu = blockIdx.y;
     if (site >= V) return;
-    const bool fixed = fx_unit_links(info);
+    const bool fixed = info[0] == 0;
     int4 *o = reinterpret_cast<int4 *>(A);
 #pragma unroll
     for (int e = 0; e < 9; e++) {
@@ -192,7 +196,7 @@ __global__ void k_path_links(const double2 *__restrict__ U, double2 *__restrict_
 __global__ void k_path_f64(const double2 *__restrict__ U, double2 *__restrict__ A, int V,
                            const unsigned *__restrict__ info) {
     const int site = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-    if (site >= V || !fx_unit_links(info)) return;
+    if (site >= V || info[0]) return;
     const int n = off_class(canon_k(j));
     if (n == 1) {
         const int mu = j == 0 ? 0 : j == 2 ? 1 : j == 8 ? 2 : 3;
@@ -217,7 +221,7 @@ __global__ void __launch_bounds__(128, 3) k_project_hops(const double2 *__restri
     const int site = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y;
     if (site >= V) return;
-    const bool fixed = fx_unit_links(info);
+    const bool fixed = info[0] == 0;
     M3<double2> w;
     bool unitary = false;
     if (off_class(canon_k(j)) == 1) {
@@ -401,8 +405,8 @@ bri_status bri_hops_build_impl(bri_ctx *ctx, cudaStream_t s) {
     if (!ctx->hops64) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->hops64, sizeof(double2) * 9 * NCANON * (size_t)g.V));
     BRI_RETURN_IF(bri_fx_reserve(ctx));
     ctx->have64 = false;
-    BRI_TRY_CUDA(ctx, cudaMemsetAsync(ctx->fxinfo, 0, 3 * sizeof(unsigned), s));
-    k_link_norms<<<(unsigned)(((size_t)g.V * 4 + 127) / 128), 128, 0, s>>>(ctx->U, 4 * g.V, ctx->fxinfo);
+    BRI_TRY_CUDA(ctx, cudaMemsetAsync(ctx->fxinfo, 0, 2 * sizeof(unsigned), s));
+    k_link_check<<<(unsigned)(((size_t)g.V * 4 + 127) / 128), 128, 0, s>>>(ctx->U, 4 * g.V, ctx->fxinfo);
     BRI_LAUNCHED(ctx);
     BRI_RETURN_IF(path_levels(ctx, ctx->hops64, s));
     const int T = 128;

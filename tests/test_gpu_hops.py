@@ -185,3 +185,38 @@ def test_projection_of_fixed_point_sums(gpu, L, eps):
         assert np.abs(T).max() <= tol
         for s in range(0, len(W), 20):
             assert np.trace(B[s]).real >= np.trace(A[s].conj().T @ oracle.project_su3(A[s])).real - tol
+
+
+@pytest.mark.parametrize("a,b", [(0.0, 3**-0.5), (0.612, 0.296), (0.3, 0.46)])
+def test_unit_norms_without_orthogonality(gpu, a, b):
+    """Links whose rows and columns have norm 1 without being unitary, a + b J in
+    any order with any phases: path sums of norm up to 1.73^4, beyond the bounds
+    of the fixed-point form.  They take the FP64 form, like twice those links,
+    whose off-axis fields are therefore the same bits (all steps scale by powers
+    of 2; an entry in a hundred may differ where a threshold of the projection
+    does not), and agree with the oracle's to the bound of the other tests."""
+    L = (3, 4, 3, 5)
+    rng = np.random.default_rng(96)
+    n = synth.volume(L) * 4
+    A = a * np.eye(3) + b * np.ones((3, 3))
+    A = A / np.linalg.norm(A[0])
+    perm = np.array([rng.permutation(3) for _ in range(n)])
+    ph = np.exp(0.4j * rng.standard_normal((2, n, 3)))
+    U = (A[perm] * ph[0][:, :, None] * ph[1][:, None, :]).reshape(-1, 4, 3, 3)
+    assert np.allclose(np.linalg.norm(U, axis=-1), 1) and np.allclose(np.linalg.norm(U, axis=-2), 1)
+    op = Brillouin(L, AP)
+    off = [j for j in range(40) if sum((j + 41) // 3**m % 3 != 1 for m in range(4)) > 1]
+    op.build_hops(torch.as_tensor(U, device=gpu))
+    W = op.hops().cpu().numpy()[:, off]
+    op.build_hops(torch.as_tensor(2 * U, device=gpu))
+    assert (op.hops().cpu().numpy()[:, off] == W).mean() > 0.99
+    ref = oracle.build_hops(L, U)[:, [j + 41 for j in off]]
+    # where the maximum is unique to 64 bits: the path sum's singular values apart from zero
+    fine = np.isfinite(ref).all(axis=(-1, -2))
+    for i, j in enumerate(off):
+        d = [(j + 41) // 3**m % 3 - 1 for m in range(4)]
+        for s in range(0, len(W), 7):
+            P, m = oracle.path_sum(L, U, s, d)
+            sv = np.linalg.svd(P / m, compute_uv=False)
+            if fine[s, i] and sv[2] > 1e-3:
+                assert np.abs(W[s, i] - ref[s, i]).max() < 1e-12 / sv[2], (s, j)
