@@ -116,6 +116,7 @@ bri_status bri_dslash_raw(bri_ctx *ctx, void *out, const void *in, int nrhs, dou
                           const int *skip, int threads, cudaStream_t s, void *work = nullptr);
 // FP64 apply in fixed point (dslash_fx.cu)
 bri_status bri_fx_reserve(bri_ctx *ctx);
+bool bri_fx_ready(const bri_ctx *ctx);
 size_t bri_fx_work_bytes(bri_ctx *ctx, int nrhs);
 bri_status bri_dslash_fx(bri_ctx *ctx, const bri::Geom &g, void *out, const void *in, int nrhs, double m0, int mode,
                          const int *skip, void *work, int *ndone, cudaStream_t s);

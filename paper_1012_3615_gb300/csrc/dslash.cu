@@ -85,7 +85,7 @@ static bri_status dslash_geom(bri_ctx *ctx, const Geom &g, void *out, const void
     const double diag = m0 + g.lamd[0];
     if (prec == BRI_F64) {
         if (!ctx->have64) return bri_fail(ctx, BRI_ESTATE, "FP64 hopping fields not built");
-        if (ctx->have_fx) {
+        if (bri_fx_ready(ctx)) {
             int done = 0;
             BRI_RETURN_IF(bri_dslash_fx(ctx, g, out, in, nrhs, m0, mode & 3, skip, work, &done, s));
             if (done == nrhs) return BRI_OK;

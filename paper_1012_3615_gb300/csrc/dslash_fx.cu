@@ -38,6 +38,7 @@
 // not unitary (one exponent serves all links: one of another size would take
 // digits from the rest of the lattice) or a field holds a NaN.
 #include <algorithm>
+#include <cmath>
 #include <string>
 
 #include "dslash_kernel.cuh"
@@ -570,6 +571,17 @@ bri_status bri_fx_reserve(bri_ctx *ctx) {
         BRI_TRY_CUDA(ctx, cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep));
     }
     return BRI_OK;
+}
+
+// the fixed-point apply can be used: its fields are there, and the class weights
+// lie within 2^+-60 or are zero, so that their products with the class scales
+// (2^+-958) stay normal numbers with all their digits
+bool bri_fx_ready(const bri_ctx *ctx) {
+    if (!ctx->have_fx) return false;
+    for (int n = 1; n <= 4; n++)
+        for (double w : {std::fabs(ctx->g.lamd[n]), std::fabs(ctx->g.rhod[n])})
+            if (w != 0.0 && !(w >= 0x1p-60 && w <= 0x1p60)) return false;
+    return true;
 }
 
 size_t bri_fx_work_bytes(bri_ctx *ctx, int nrhs) { return fx_bytes(ctx->g, nrhs); }

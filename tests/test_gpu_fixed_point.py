@@ -181,3 +181,75 @@ def test_small_links_keep_their_digits(gpu, oracle_weights, scale):
     out = op.apply(torch.as_tensor(psi, device=gpu), m0=-4.0).cpu().numpy()[0]
     ref = oracle.apply(L, AP, W, -4.0, psi[0])
     assert np.abs(out - ref).max() <= 4e-15 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("size", [1e-290, 1e-200, 1e200])
+def test_weights_of_any_size(gpu, oracle_weights, size):
+    """weights whose products with the spinors' scales would leave the range of
+    normal FP64 numbers lose no digits"""
+    L = (4, 3, 5, 4)
+    lam, rho = [0] + [size * v for v in (-0.5, -0.2, 0.1, 0.3)], [0] + [size * v for v in (0.3, 0.2, 0.1, 0.05)]
+    U = synth.random_su3_links(L, 0.3, 22)
+    psi = synth.gaussian_spinor(L, 1, 23) * 1e-10
+    op, W = _op(L, U, gpu)
+    op.set_weights(lam, rho)
+    oracle_weights(lam, rho)
+    out = op.apply(torch.as_tensor(psi, device=gpu), m0=0.0).cpu().numpy()[0]
+    ref = oracle.apply(L, AP, W, 0.0, psi[0])
+    assert np.abs(out - ref).max() <= 4e-15 * np.abs(ref).max()
+
+
+def _scaled_weights(op, oracle_weights, f):
+    lam, rho = op.weights()
+    lam, rho = [f * v for v in lam], [f * v for v in rho]
+    op.set_weights(lam, rho)
+    oracle_weights(lam, rho)
+
+
+@pytest.mark.parametrize("L,nrhs", [((3, 3, 3, 3), 1), ((4, 5, 3, 4), 7), ((11, 12, 12, 12), 1), ((14, 14, 14, 15), 1)])
+@pytest.mark.parametrize("f", [2.0**-61, 2.0**-59])
+def test_fp64_kernel_and_fixed_point(gpu, oracle_weights, L, nrhs, f):
+    """The operator times a power of 2, just out of and just in the range of the
+    fixed-point apply: the FP64 kernel, which also runs without memory for the
+    fixed-point copy, and the fixed-point one, through D, D^dagger, the overlap
+    kernel, the clover term and slabs of time slices"""
+    U = synth.random_su3_links(L, 0.3, 24)
+    psi = synth.gaussian_spinor(L, nrhs, 25)
+    op, W = _op(L, U, gpu)
+    _scaled_weights(op, oracle_weights, f)
+    x = torch.as_tensor(psi, device=gpu)
+
+    def check(out, ref):
+        assert np.abs(out - ref).max() <= 4e-15 * np.abs(ref).max()
+
+    r = nrhs - 1
+    for dag in (False, True):
+        ref = oracle.apply(L, AP, W, 0.1 * f, psi[r], dagger=dag)
+        check(op.apply(x, m0=0.1 * f, dagger=dag)[r].cpu().numpy(), ref)
+    host = op.apply_host(torch.as_tensor(psi).pin_memory(), m0=0.1 * f, dagger=True)
+    torch.cuda.synchronize()
+    check(host[r].numpy(), ref)
+    check(op.overlap_kernel(x, rho=1.5 * f)[r].cpu().numpy(), oracle.overlap_kernel(L, AP, W, 0.0, 1.5 * f, psi[r]))
+    if len(psi[0]) < 1000:
+        op.set_clover(f)
+        check(op.apply(x, m0=0.1 * f)[r].cpu().numpy(), oracle.apply_clover(L, AP, W, U, 0.1 * f, f, psi[r]))
+
+
+@pytest.mark.parametrize("f", [2.0**61, 2.0**59])
+@pytest.mark.parametrize("mode,nrhs", [(0, 1), (1, 2), (4, 3)])
+def test_solves_with_either_apply(gpu, oracle_weights, f, mode, nrhs):
+    """solver iterations and residuals (with right-hand sides skipped as they
+    converge) on the FP64 kernel and on the fixed-point apply"""
+    L = (4, 4, 5, 4)
+    U = synth.random_su3_links(L, 0.3, 26)
+    b = synth.z2_spinor(L, nrhs, 27)
+    b[-1] = 0
+    b[-1, 5, 1, 2] = 1.0
+    op, W = _op(L, U, gpu)
+    _scaled_weights(op, oracle_weights, f)
+    op.store_hops("f32", "2row")
+    x, info = op.solve(torch.as_tensor(b, device=gpu), m0=0.1 * f, tol=1e-10, mode=mode)
+    assert all(i["status"] == "BRI_OK" for i in info)
+    for r in range(nrhs):
+        res = b[r] - oracle.apply(L, AP, W, 0.1 * f, x.cpu().numpy()[r])
+        assert np.linalg.norm(res) <= 1.01e-10 * np.linalg.norm(b[r])
