@@ -120,7 +120,14 @@ bri_status bri_get_hops(bri_ctx *ctx, double *out, void *stream);
  * Sec. 1), for nrhs right-hand sides, with the hopping fields stored in prec
  * (for BRI_F32 / BRI_F16 the compression of the last build/store in that
  * precision).  in/out: device, [nrhs][V][4][3] complex (see conventions),
- * 16-byte aligned, must not overlap.  Errors: BRI_EINVAL, BRI_ESTATE
+ * 16-byte aligned, must not overlap.  BRI_F64: products are summed in fixed
+ * point, exactly over the hops of a class, at sites where the links (unitary
+ * to 2^-16), the weights and the spinors that the site sees allow it, in FP64
+ * elsewhere.  In fixed point the error is at most that of FP64 arithmetic
+ * relative to the largest component of the site's neighbours; a result
+ * component that only gets contributions of components 2^-k of those (links
+ * near the identity; k is at most 20) may have an error 2^k times larger
+ * relative to itself.  Errors: BRI_EINVAL, BRI_ESTATE
  * (fields of that precision not built), BRI_ECUDA. */
 bri_status bri_apply(bri_ctx *ctx, void *out, const void *in, int nrhs, double m0, int dagger,
                      bri_prec prec, void *stream);

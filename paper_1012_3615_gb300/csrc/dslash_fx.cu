@@ -33,8 +33,9 @@
 // instructions; latency at 12 warps per SM bounds it (issue 42%, long
 // scoreboard and fixed-latency waits the top stalls).
 //
-// A site that meets an infinity, a NaN or an exponent outside the range of
-// FP64 scales takes the FP64 loop (fx_slow), as every site does when a link is
+// A site that meets an infinity, a NaN, a spinor whose components differ by too
+// many orders of magnitude (FX_WIDE) or an exponent outside the range of FP64
+// scales takes the FP64 loop (fx_slow), as every site does when a link is
 // not unitary (one exponent serves all links: one of another size would take
 // digits from the rest of the lattice) or a field holds a NaN.
 #include <algorithm>
@@ -57,6 +58,14 @@ namespace {
 // head room h_n of the class sums
 BRI_D int fx_head(int n) { return n == 1 ? 0 : n == 2 ? 2 : 3; }
 
+// A site's components share an exponent, so that one 2^-k of the largest keeps
+// 53 - k bits.  A site where a component lies more than this many binary orders
+// below the largest of its chirality (zeros included, unless all six are) is
+// marked as out of range, and those that see it take the FP64 loop: out of a
+// Gaussian field one site in 10^9.  The chiralities may differ by any factor:
+// through gamma_d both enter every row.
+constexpr unsigned FX_WIDE = 20;
+
 // spinors to limbs [nrhs][Vp/32][12][32] and block exponents [nrhs][V], for n
 // sites from s0 on (modulo V)
 __global__ void k_fx_spinor(const double2 *__restrict__ in, int4 *__restrict__ p, int *__restrict__ ex, int V, int s0,
@@ -68,14 +77,22 @@ __global__ void k_fx_spinor(const double2 *__restrict__ in, int4 *__restrict__ p
     double2 v[12];
     load_spinor(in + ((size_t)rhs * V + site) * 12, v);
     unsigned m = 0;
-    bool zero = true;
+    bool zero = true, wide = false;
 #pragma unroll
-    for (int k = 0; k < 12; k++) {
-        m = max(m, max(abs_hi(v[k].x), abs_hi(v[k].y)));
-        zero = zero && v[k].x == 0.0 && v[k].y == 0.0;
+    for (int h = 0; h < 2; h++) {
+        unsigned lo = 0xffffffffu, hi = 0;
+#pragma unroll
+        for (int k = 6 * h; k < 6 * h + 6; k++) {
+            const unsigned a = max(abs_hi(v[k].x), abs_hi(v[k].y));
+            lo = min(lo, a);
+            hi = max(hi, a);
+            zero = zero && v[k].x == 0.0 && v[k].y == 0.0;
+        }
+        wide = wide || (hi >> 20) > (lo >> 20) + FX_WIDE;
+        m = max(m, hi);
     }
     const int f = (int)(m >> 20);
-    const bool bad = f == 2047;
+    const bool bad = f == 2047 || wide;
     const int e = bad ? FX_BAD : zero ? FX_ZERO : f - 1022;
     ex[(size_t)rhs * V + site] = e;
     p += (size_t)rhs * 12 * ((V + 31) & ~31) + fx_at(site, 12);
@@ -575,13 +592,17 @@ bri_status bri_fx_reserve(bri_ctx *ctx) {
 
 // the fixed-point apply can be used: its fields are there, and the class weights
 // lie within 2^+-60 or are zero, so that their products with the class scales
-// (2^+-958) stay normal numbers with all their digits
+// (2^+-958) stay normal numbers with all their digits.  rho all zero leaves the
+// chiralities apart, which share an exponent (FX_WIDE)
 bool bri_fx_ready(const bri_ctx *ctx) {
     if (!ctx->have_fx) return false;
-    for (int n = 1; n <= 4; n++)
+    bool mixes = false;
+    for (int n = 1; n <= 4; n++) {
         for (double w : {std::fabs(ctx->g.lamd[n]), std::fabs(ctx->g.rhod[n])})
             if (w != 0.0 && !(w >= 0x1p-60 && w <= 0x1p60)) return false;
-    return true;
+        mixes = mixes || ctx->g.rhod[n] != 0.0;
+    }
+    return mixes;
 }
 
 size_t bri_fx_work_bytes(bri_ctx *ctx, int nrhs) { return fx_bytes(ctx->g, nrhs); }

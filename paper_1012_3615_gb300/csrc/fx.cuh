@@ -5,7 +5,7 @@
 
 namespace bri {
 
-constexpr int FX_BAD = 1 << 20;     // block exponent of a site with an infinity or a NaN
+constexpr int FX_BAD = 1 << 20;     // block exponent of a site out of range: an infinity, a NaN, or FX_WIDE
 constexpr int FX_ZERO = -(1 << 20);  // ... of a site that is zero
 constexpr int FX_WB = 62, FX_PB = 60;  // fraction bits of links and spinors
 constexpr int FX_AB = FX_WB + FX_PB - 64;  // of the row sums

@@ -253,3 +253,43 @@ def test_solves_with_either_apply(gpu, oracle_weights, f, mode, nrhs):
     for r in range(nrhs):
         res = b[r] - oracle.apply(L, AP, W, 0.1 * f, x.cpu().numpy()[r])
         assert np.linalg.norm(res) <= 1.01e-10 * np.linalg.norm(b[r])
+
+
+@pytest.mark.parametrize("what", ["spin", "colour", "zero beside small", "laplacian", "near the line"])
+def test_components_of_different_size(gpu, oracle_weights, what):
+    """Components that stay apart (one chirality and its spins, colours over unit
+    links, chiralities without gamma terms) keep their own digits next to ones
+    that are many orders larger: against the largest result of their own kind.
+    Within the line of 2^-20 the block exponent takes at most that factor, 2^-54
+    of the largest component and 80 hops of weight 1/16 or less."""
+    L = (4, 4, 3, 5)
+    U = synth.unit_links(L) if what in ("colour", "near the line") else synth.random_su3_links(L, 0.3, 28)
+    psi = synth.gaussian_spinor(L, 1, 29)
+    if what in ("spin", "zero beside small"):
+        psi[:, :, 2:] = 0
+    if what == "spin":
+        psi[:, :, 1] *= 1e-14
+    elif what == "colour":
+        psi[..., 2] *= 1e-14
+    elif what == "near the line":
+        psi[..., 2] *= 1e-4
+    elif what == "zero beside small":
+        psi *= 1e-14
+        psi[0, 100] = 0
+        psi[0, 100, 0, 0] = 1.0
+    else:
+        psi[:, :, 2:] *= 1e-14
+    op, W = _op(L, U, gpu)
+    if what == "laplacian":
+        lam, rho = [1.9, -0.1, -0.05, -0.02, -0.01], [0] * 5
+        op.set_weights(lam, rho)
+        oracle_weights(lam, rho)
+    out = op.apply(torch.as_tensor(psi, device=gpu), m0=0.1).cpu().numpy()[0]
+    ref = oracle.apply(L, AP, W, 0.1, psi[0])
+    size = np.abs(ref).max(axis=0)
+    tol = 4e-15 if what != "near the line" else 4e-15 + 2.0**-54 * 5 * np.abs(psi).max() / size
+    assert (np.abs(out - ref).max(axis=0) <= tol * size).all()
+    if what == "zero beside small":  # far from the point, each site by itself
+        far = np.abs(ref).max(axis=(1, 2)) < 1e-10
+        assert far.any()
+        assert (np.abs(out - ref)[far] <= 4e-15 * np.abs(ref[far]).max(axis=(1, 2), keepdims=True)).all()
