@@ -441,6 +441,13 @@ struct SolverWork {
     std::map<std::string, Captured> graphs;
 };
 
+static void drop_graphs(SolverWork *w) {
+    for (auto &kv : w->graphs) cudaGraphExecDestroy(kv.second.exec);
+    w->graphs.clear();
+}
+// most graphs kept: a program that keeps changing the operator starts again
+static constexpr size_t MAX_GRAPHS = 32;
+
 static void free_vecs(VecSet &v) {
     void **a[] = {&v.x, &v.r, &v.rhat, &v.p, &v.v, &v.s, &v.t};
     for (void **p : a) {
@@ -452,7 +459,7 @@ static void free_vecs(VecSet &v) {
 void bri_solver_free(bri_ctx *ctx) {
     SolverWork *w = ctx->work;
     if (!w) return;
-    for (auto &kv : w->graphs) cudaGraphExecDestroy(kv.second.exec);
+    drop_graphs(w);
     free_vecs(w->v64);
     free_vecs(w->v32);
     cudaFree(w->r64);
@@ -541,6 +548,19 @@ bri_status enqueue_iters(bri_ctx *ctx, const VecSet &vs, int nrhs, double m0, br
     return BRI_OK;
 }
 
+// everything that captured iterations hold by value: weights, clover term and
+// boundary phases (Geom), and the buffers that the stencil reads or works in
+std::string graph_key(bri_ctx *ctx, const VecSet &vs, int elt, bri_prec prec, int nrhs, double m0, int thr) {
+    const LinkStore &st = prec == BRI_F32 ? ctx->f32 : ctx->f16, &ps = prec == BRI_F32 ? ctx->p32 : ctx->p16;
+    char text[512];
+    snprintf(text, sizeof text, "bi:%d:%d:%d:%.17g:%p:%p:%p:%d:%d:%p:%p:%d:%p:%d:%p:%p:%p:%d", elt, (int)prec, nrhs, m0,
+             vs.x, vs.s, vs.t, thr, (int)st.comp, st.a, st.b, (int)ps.comp, ps.a, (int)ps.valid, ctx->tc_f,
+             (void *)ctx->tc_amax, (void *)ctx->hopsfx, (int)bri_fx_ready(ctx));
+    std::string key(text);
+    key.append((const char *)&ctx->g, sizeof ctx->g);
+    return key;
+}
+
 // Run BiCGstab on (vs.x, b) in element type T until every right-hand side has a
 // flag (converged / breakdown / nan) or maxit iterations were done.  x is the
 // initial guess when have_x0.  Returns the iterations performed.
@@ -561,21 +581,19 @@ bri_status bicgstab(bri_ctx *ctx, const VecSet &vs, const T *b, bool have_x0, in
     BRI_LAUNCHED(ctx);
     // block of iterations per graph replay: short for expensive FP64 applies
     const int K = sizeof(T) == 16 ? 4 : 16;
-    char key[192];
-    snprintf(key, sizeof key, "bi:%d:%d:%d:%.17g:%p:%p:%p:%d", (int)sizeof(T), (int)prec, nrhs, m0, vs.x, vs.s,
-             vs.t, bri_dslash_threads(ctx, prec, nrhs));
+    // the tensor-core apply and the site-pair kernel allocate or store on first
+    // use: not inside the capture
+    const int thr = bri_dslash_threads(ctx, prec, nrhs);
+    if ((thr >> 11) == 8) BRI_RETURN_IF(bri_tc_reserve(ctx, nrhs, thr & 2047));
+    if ((thr >> 11) == 3 && prec != BRI_F64 && !(prec == BRI_F32 ? ctx->p32 : ctx->p16).valid && !ctx->g.clov64)
+        BRI_RETURN_IF(bri_pair_store_impl(ctx, prec, s));
+    const std::string key = graph_key(ctx, vs, (int)sizeof(T), prec, nrhs, m0, thr);
     SolverWork::Captured run{};
     auto it = w->graphs.find(key);
     if (it != w->graphs.end()) {
         run = it->second;
     } else {
-        // the tensor-core apply and the site-pair kernel allocate on first use:
-        // not inside the capture
-        const int thr = bri_dslash_threads(ctx, prec, nrhs);
-        if ((thr >> 11) == 8) BRI_RETURN_IF(bri_tc_reserve(ctx, nrhs, thr & 2047));
-        if ((thr >> 11) == 3 && prec != BRI_F64 && !(prec == BRI_F32 ? ctx->p32 : ctx->p16).valid &&
-            !ctx->g.clov64)
-            BRI_RETURN_IF(bri_pair_store_impl(ctx, prec, s));
+        if (w->graphs.size() >= MAX_GRAPHS) drop_graphs(w);
         cudaGraph_t graph;
         const long before = ctx->launches;
         BRI_TRY_CUDA(ctx, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));

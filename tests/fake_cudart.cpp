@@ -55,6 +55,7 @@ std::map<std::pair<int, const void *>, int> smem_limit;
 std::map<cudaStream_t, Graph *> capturing;
 std::set<Pool *> pools;
 int capture_mode = cudaStreamCaptureModeGlobal;
+int fill = 0;  // byte that results of 16 bytes or more consist of
 long fail_skip = -1, fail_count = 0;
 std::string record;
 struct Config {
@@ -106,6 +107,7 @@ void fake_reset() {
     budget = (size_t)1 << 40;
     fail_skip = -1;
     fail_count = 0;
+    fill = 0;
     capture_mode = cudaStreamCaptureModeGlobal;
     record.clear();
 }
@@ -116,6 +118,7 @@ void fake_refuse(long skip, long count) {
     fail_skip = skip;
     fail_count = count;
 }
+void fake_fill(int byte) { fill = byte; }
 void fake_device(int d) { device = d; }
 const char *fake_log() { return record.c_str(); }
 void fake_clear_log() { record.clear(); }
@@ -153,8 +156,9 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3 block, void **arg
     if (smem > 48 * 1024 && (lim == smem_limit.end() || (size_t)lim->second < smem)) return fail(cudaErrorInvalidValue);
     Launch l;
     l.name = names[fun];
-    if (l.name.find("k_dslash_fx") != std::string::npos)  // (mode, link limbs, info, fields, spinor limbs, ...)
-        for (int i : {1, 4}) l.needs.push_back(*(uintptr_t *)args[i]);
+    // (mode, fields, ...), in fixed point (mode, limbs, info, fields, spinor limbs, ...)
+    if (l.name.find("k_dslash") != std::string::npos) l.needs.push_back(*(uintptr_t *)args[1]);
+    if (l.name.find("k_dslash_fx") != std::string::npos) l.needs.push_back(*(uintptr_t *)args[4]);
     auto c = capturing.find(stream);
     if (c != capturing.end()) {
         c->second->launches.push_back(l);
@@ -247,7 +251,7 @@ cudaError_t cudaHostGetDevicePointer(void **d, void *h, unsigned) {
     return cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void *dst, const void *, size_t n, cudaMemcpyKind kind, cudaStream_t) {
-    if (kind == cudaMemcpyDeviceToHost) memset(dst, 0, n);
+    if (kind == cudaMemcpyDeviceToHost) memset(dst, n >= 16 ? fill : 0, n);
     return cudaSuccess;
 }
 cudaError_t cudaMemset(void *, int, size_t) { return cudaSuccess; }

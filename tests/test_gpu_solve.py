@@ -159,3 +159,31 @@ def test_solves_on_the_bulk_copy_line_kernel(gpu, mode, prec):
     xs = x.cpu().numpy()
     for r in range(b.shape[0]):
         assert _true_resid(L, AP, W, -0.05, xs[r], b[r]) <= 1e-10
+
+
+@pytest.mark.parametrize("mode", [0, 1, 4])
+def test_solves_after_the_operator_changed(gpu, mode):
+    """one context, the same mass: other weights, other links, another storage,
+    each solved to its own true residual"""
+    from paper_1012_3615_gb300.core import WEIGHTS
+
+    L = (4, 4, 4, 6)
+    b = torch.as_tensor(synth.z2_spinor(L, 1, 71), device=gpu)
+    op = Brillouin(L, (1, 1, 1, -1))
+    op.build_hops(torch.as_tensor(synth.random_su3_links(L, 0.3, 72), device=gpu), prec="f32", comp="full")
+
+    def check():
+        x, info = op.solve(b, m0=0.2, tol=1e-10, mode=mode, maxit=500)
+        assert info[0]["status"] == "BRI_OK"
+        assert info[0]["outer_iters"] <= 4  # the inner operator is the outer one's
+        assert (b - op.apply(x, m0=0.2)).norm().item() <= 1.01e-10 * b.norm().item()
+
+    check()
+    op.set_weights(*WEIGHTS["wilson"])
+    check()
+    op.build_hops(torch.as_tensor(synth.random_su3_links(L, 0.4, 73), device=gpu), prec="f32", comp="full")
+    check()
+    op.store_hops("f32", "2row")
+    check()
+    op.set_weights(*WEIGHTS["brillouin"])
+    check()

@@ -74,6 +74,12 @@ def fake(lib):
         def build(self, h, prec=0, comp=0):
             return lib.bri_build_hops(h, 1 << 57, prec, comp, None)
 
+        def solve(self, h, mode, nrhs=1, maxit=8):
+            from paper_1012_3615_gb300 import abi
+
+            info = (abi.bri_solve_info * nrhs)()
+            return lib.bri_solve(h, 1 << 50, 1 << 56, nrhs, 0.1, 1e-10, maxit, mode, info, 1 << 40)
+
         def log(self):
             text = lib.fake_log().decode().split("\n")
             lib.fake_clear_log()
@@ -95,3 +101,35 @@ def test_fp64_apply_on_two_devices(fake, L):
         assert fake.build(h) == 0
         assert fake.apply(h) == 0, fake.lib.bri_last_error(h)
         assert any("k_dslash_fx" in t for t in fake.log())
+
+
+def _weights(lib, h, lam, rho):
+    assert lib.bri_set_weights(h, (ctypes.c_double * 5)(*lam), (ctypes.c_double * 5)(*rho)) == 0
+
+
+def test_solver_graphs_follow_the_operator(fake):
+    """captured iterations hold the weights by value and the fields by address:
+    after either changed they are captured again, and after neither they are not"""
+    h = fake.op()
+    assert fake.build(h, prec=1, comp=0) == 0
+    wilson = [4.0, -0.5, 0, 0, 0], [0, 0.5, 0, 0, 0]
+    for mode in (0, 1):
+        fake.lib.fake_fill(0x3f if mode else 0)  # norms, so that the mixed solve runs
+        for what, want in (("first", True), ("same", False), ("weights", True), ("links", False)):
+            if what == "weights":
+                _weights(fake.lib, h, *wilson)
+            elif what == "links":  # same buffers, new contents
+                assert fake.build(h, prec=1, comp=0) == 0
+            fake.log()
+            fake.solve(h, mode)
+            log = fake.log()
+            assert any(t.startswith("captured") for t in log) == want, (mode, what)
+            assert any(t.startswith("replayed") for t in log), (mode, what)
+            assert not any(t.startswith("STALE") for t in log), (mode, what)
+        _weights(fake.lib, h, [1.9, -0.1, -0.1, -0.1, -0.1], [0, 0.1, 0.1, 0.1, 0.1])
+    # another storage of the fields takes other memory
+    assert fake.lib.bri_store_hops(h, 1, 1, None) == 0
+    fake.log()
+    fake.solve(h, 1)
+    log = fake.log()
+    assert any(t.startswith("captured") for t in log) and not any(t.startswith("STALE") for t in log)
