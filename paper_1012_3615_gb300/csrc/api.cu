@@ -124,6 +124,7 @@ bri_status bri_destroy(bri_ctx *ctx) {
     cudaFree(ctx->hopsfx);
     cudaFree(ctx->fxinfo);
     if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+    bri_captured_free(ctx, true);
     cudaFreeHost(ctx->werr_h);
     for (LinkStore *st : {&ctx->f32, &ctx->f16, &ctx->p32, &ctx->p16}) {
         cudaFree(st->a);

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <map>
+#include <memory>
 #include <string>
 
 #include "brillouin.h"
@@ -16,6 +17,7 @@ struct LinkStore {
     void *b = nullptr;  // tail array (8/4-byte chunk, [40][V]) or null
 };
 
+struct CapturedWork; // work space of captured applies (captured.cu)
 struct SolverWork;   // solver work spaces (solve.cu)
 struct OverlapWork;  // Lanczos / overlap state (overlap.cu)
 struct HostApplyWork;  // staging buffers and streams of bri_apply_host (hostapply.cu)
@@ -31,6 +33,7 @@ struct bri_ctx {
     bool have_fx = false, fx_tried = false;
     unsigned fx_attr = 0;        // its kernels whose shared-memory limit is raised on this device
     cudaMemPool_t pool = nullptr;  // stream-ordered work space of the calls, released by bri_destroy
+    std::shared_ptr<CapturedWork> captured;
     LinkStore f32, f16;
     LinkStore p32, p16;  // site-pair interleaved copies (full / 2-row, even t extent)
     SolverWork *work = nullptr;
@@ -113,13 +116,17 @@ bri_status bri_dslash_tc(bri_ctx *ctx, void *out, const void *in, int nrhs, doub
 bri_status bri_tc_reserve(bri_ctx *ctx, int nrhs, int cap);
 // dslash with an explicit launch shape; skip[r] != 0 skips right-hand side r
 bri_status bri_dslash_raw(bri_ctx *ctx, void *out, const void *in, int nrhs, double m0, int mode, bri_prec prec,
-                          const int *skip, int threads, cudaStream_t s, void *work = nullptr);
+                          const int *skip, int threads, cudaStream_t s);
 // FP64 apply in fixed point (dslash_fx.cu)
 bri_status bri_fx_reserve(bri_ctx *ctx);
 bool bri_fx_ready(const bri_ctx *ctx);
-size_t bri_fx_work_bytes(bri_ctx *ctx, int nrhs);
 bri_status bri_dslash_fx(bri_ctx *ctx, const bri::Geom &g, void *out, const void *in, int nrhs, double m0, int mode,
-                         const int *skip, void *work, int *ndone, cudaStream_t s);
+                         const int *skip, int *ndone, cudaStream_t s);
+// work space of a captured stream (captured.cu): whether s is captured, with the
+// capture's id and graph; work space that the graph holds, or null; its release
+bool bri_capturing(cudaStream_t s, unsigned long long *id, cudaGraph_t *graph);
+void *bri_captured_work(bri_ctx *ctx, cudaStream_t s, unsigned long long id, cudaGraph_t graph, size_t bytes);
+bool bri_captured_free(bri_ctx *ctx, bool all);
 int bri_dslash_threads(bri_ctx *ctx, bri_prec prec, int nrhs);
 std::string bri_tune_key(bri_ctx *ctx, bri_prec prec, int nrhs);
 bri_status bri_export_hops_impl(bri_ctx *ctx, double2 *out, cudaStream_t s);

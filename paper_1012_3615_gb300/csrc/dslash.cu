@@ -57,11 +57,11 @@ int bri_dslash_threads(bri_ctx *ctx, bri_prec prec, int nrhs) {
 }
 
 static bri_status dslash_geom(bri_ctx *ctx, const Geom &g, void *out, const void *in, int nrhs, double m0, int mode,
-                              bri_prec prec, const int *skip, int threads, cudaStream_t s, void *work = nullptr);
+                              bri_prec prec, const int *skip, int threads, cudaStream_t s);
 
 bri_status bri_dslash_raw(bri_ctx *ctx, void *out, const void *in, int nrhs, double m0, int mode, bri_prec prec,
-                          const int *skip, int threads, cudaStream_t s, void *work) {
-    return dslash_geom(ctx, ctx->g, out, in, nrhs, m0, mode, prec, skip, threads, s, work);
+                          const int *skip, int threads, cudaStream_t s) {
+    return dslash_geom(ctx, ctx->g, out, in, nrhs, m0, mode, prec, skip, threads, s);
 }
 
 // only sites [s0, s1) of out are written (the plain kernels; the tiled and
@@ -77,7 +77,7 @@ bri_status bri_dslash_range(bri_ctx *ctx, void *out, const void *in, int nrhs, d
 }
 
 static bri_status dslash_geom(bri_ctx *ctx, const Geom &g, void *out, const void *in, int nrhs, double m0, int mode,
-                              bri_prec prec, const int *skip, int threads, cudaStream_t s, void *work) {
+                              bri_prec prec, const int *skip, int threads, cudaStream_t s) {
     if (ctx->werr_h && *(volatile int *)ctx->werr_h) {
         *(volatile int *)ctx->werr_h = 0;
         return bri_fail(ctx, BRI_ETIMEOUT, "a bounded wait of an earlier apply gave up; its output is invalid");
@@ -87,7 +87,7 @@ static bri_status dslash_geom(bri_ctx *ctx, const Geom &g, void *out, const void
         if (!ctx->have64) return bri_fail(ctx, BRI_ESTATE, "FP64 hopping fields not built");
         if (bri_fx_ready(ctx)) {
             int done = 0;
-            BRI_RETURN_IF(bri_dslash_fx(ctx, g, out, in, nrhs, m0, mode & 3, skip, work, &done, s));
+            BRI_RETURN_IF(bri_dslash_fx(ctx, g, out, in, nrhs, m0, mode & 3, skip, &done, s));
             if (done == nrhs) return BRI_OK;
             const size_t field = (size_t)done * g.V * 12;
             out = (double2 *)out + field;

@@ -605,34 +605,37 @@ bool bri_fx_ready(const bri_ctx *ctx) {
     return mixes;
 }
 
-size_t bri_fx_work_bytes(bri_ctx *ctx, int nrhs) { return fx_bytes(ctx->g, nrhs); }
-
-// FP64 apply of sites [g.s0, g.s1) in fixed point; work: bri_fx_work_bytes, or
-// null to take it from the context's stream-ordered pool.  The right-hand
+// FP64 apply of sites [g.s0, g.s1) in fixed point.  Its work space is stream-ordered
+// from the context's pool, during capture held by the graph.  The right-hand
 // sides done so far are counted in *ndone; fewer than nrhs with BRI_OK: no
 // memory for the limb copies, the caller runs the FP64 kernel on the rest.
 bri_status bri_dslash_fx(bri_ctx *ctx, const Geom &g, void *out, const void *in, int nrhs, double m0, int mode,
-                         const int *skip, void *work, int *ndone, cudaStream_t s) {
+                         const int *skip, int *ndone, cudaStream_t s) {
     const double diag = m0 + g.lamd[0];
     const size_t field = (size_t)g.V * 12;
     // right-hand sides per launch: up to 2 GB of limb copies
     const int rmax = (int)std::max<size_t>(1, std::min<size_t>(32, ((size_t)2 << 30) / fx_bytes(g, 1)));
-    if (nrhs > rmax && !work) {
+    if (nrhs > rmax) {
         for (int r = 0; r < nrhs && *ndone == r; r += rmax)
             BRI_RETURN_IF(bri_dslash_fx(ctx, g, (double2 *)out + r * field, (const double2 *)in + r * field,
-                                        nrhs - r < rmax ? nrhs - r : rmax, m0, mode, skip ? skip + r : nullptr, work,
-                                        ndone, s));
+                                        nrhs - r < rmax ? nrhs - r : rmax, m0, mode, skip ? skip + r : nullptr, ndone,
+                                        s));
         return BRI_OK;
     }
-    void *own = nullptr;
-    if (!work) {
-        const cudaError_t e = cudaMallocFromPoolAsync(&own, fx_bytes(g, nrhs), ctx->pool, s);
+    void *work = nullptr;
+    unsigned long long id = 0;
+    cudaGraph_t graph = nullptr;
+    const bool captured = bri_capturing(s, &id, &graph);
+    if (captured) {
+        work = bri_captured_work(ctx, s, id, graph, fx_bytes(g, nrhs));
+        if (!work) return BRI_OK;
+    } else {
+        const cudaError_t e = cudaMallocFromPoolAsync(&work, fx_bytes(g, nrhs), ctx->pool, s);
         if (e == cudaErrorMemoryAllocation) {
             cudaGetLastError();
             return BRI_OK;
         }
         BRI_TRY_CUDA(ctx, e);
-        work = own;
     }
     int4 *P = (int4 *)work;
     int *ex = (int *)(P + 12 * fx_vp(g) * nrhs);
@@ -656,7 +659,7 @@ bri_status bri_dslash_fx(bri_ctx *ctx, const Geom &g, void *out, const void *in,
                            : (S == 1 ? fx_launch<1, false> : S == 2 ? fx_launch<2, false> : fx_launch<4, false>);
     bri_status st = convert();
     if (st == BRI_OK) st = launch(mode, ctx, g, P, ex, in, out, nrhs, diag, skip, s);
-    if (own) BRI_TRY_CUDA(ctx, cudaFreeAsync(own, s));
+    if (!captured) BRI_TRY_CUDA(ctx, cudaFreeAsync(work, s));
     BRI_RETURN_IF(st);
     *ndone += nrhs;
     return BRI_OK;

@@ -426,7 +426,6 @@ struct SolverWork {
     int nrhs = 0;
     VecSet v64, v32;
     double2 *r64 = nullptr;
-    void *fxw = nullptr;  // work space of the FP64 apply inside captured iterations (one right-hand side)
     BiState *st = nullptr;
     int *flag = nullptr;
     int *done = nullptr;
@@ -463,7 +462,6 @@ void bri_solver_free(bri_ctx *ctx) {
     free_vecs(w->v64);
     free_vecs(w->v32);
     cudaFree(w->r64);
-    cudaFree(w->fxw);
     cudaFree(w->st);
     cudaFree(w->flag);
     cudaFree(w->done);
@@ -494,10 +492,7 @@ static bri_status ensure_work(bri_ctx *ctx, int nrhs, bool need64, bool need32) 
     w->n = n;
     w->nrhs = nrhs > have_nrhs ? nrhs : have_nrhs;
     const size_t R = w->nrhs;
-    if (need64 || had64) {
-        BRI_RETURN_IF(alloc_vecs(ctx, w->v64, sizeof(double2) * n * R));
-        BRI_TRY_CUDA(ctx, cudaMalloc(&w->fxw, bri_fx_work_bytes(ctx, 1)));
-    }
+    if (need64 || had64) BRI_RETURN_IF(alloc_vecs(ctx, w->v64, sizeof(double2) * n * R));
     if (need32 || had32) {
         BRI_RETURN_IF(alloc_vecs(ctx, w->v32, sizeof(float2) * n * R));
         BRI_TRY_CUDA(ctx, cudaMalloc(&w->r64, sizeof(double2) * n * R));
@@ -534,12 +529,12 @@ bri_status enqueue_iters(bri_ctx *ctx, const VecSet &vs, int nrhs, double m0, br
     for (int it = 0; it < iters; it++) {
         k_bi_p<T><<<grid, RT, 0, s>>>(p, r, v, w->st, w->flag, n);
         BRI_LAUNCHED(ctx);
-        BRI_RETURN_IF(bri_dslash_raw(ctx, v, p, nrhs, m0, 0, prec, w->flag, thr, s, w->fxw));
+        BRI_RETURN_IF(bri_dslash_raw(ctx, v, p, nrhs, m0, 0, prec, w->flag, thr, s));
         k_bi_alpha<T><<<grid, RT, 0, s>>>(rh, v, w->st, w->flag, w->part, w->tick, n);
         BRI_LAUNCHED(ctx);
         k_bi_s<T><<<grid, RT, 0, s>>>(sv, r, v, w->st, w->flag, n);
         BRI_LAUNCHED(ctx);
-        BRI_RETURN_IF(bri_dslash_raw(ctx, t, sv, nrhs, m0, 0, prec, w->flag, thr, s, w->fxw));
+        BRI_RETURN_IF(bri_dslash_raw(ctx, t, sv, nrhs, m0, 0, prec, w->flag, thr, s));
         k_bi_omega<T><<<grid, RT, 0, s>>>(t, sv, w->st, w->flag, w->part, w->tick, n);
         BRI_LAUNCHED(ctx);
         k_bi_xr<T><<<grid, RT, 0, s>>>(x, r, p, sv, t, rh, w->st, w->flag, w->part, w->tick, n);

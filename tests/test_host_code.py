@@ -133,3 +133,61 @@ def test_solver_graphs_follow_the_operator(fake):
     fake.solve(h, 1)
     log = fake.log()
     assert any(t.startswith("captured") for t in log) and not any(t.startswith("STALE") for t in log)
+
+
+def _capture(fake, stream, body):
+    s = ctypes.c_void_p(stream)
+    assert fake.lib.cudaStreamBeginCapture(s, 1) == 0
+    body()
+    g = ctypes.c_void_p()
+    assert fake.lib.cudaStreamEndCapture(s, ctypes.byref(g)) == 0
+    return g
+
+
+def _instantiate(fake, g):
+    e = ctypes.c_void_p()
+    assert fake.lib.cudaGraphInstantiate(ctypes.byref(e), g, 0) == 0
+    return e
+
+
+def test_captured_fp64_apply_owns_its_work_space(fake):
+    """no allocation nodes (they forbid a second executable graph); one work space
+    per graph, shared by the applies of one stream, taken again by the next
+    capture once the graph and its executable forms are gone"""
+    h = fake.op((8, 8, 8, 8))
+    assert fake.build(h) == 0 and fake.apply(h) == 0
+    base = fake.lib.fake_used()
+    s = 1 << 41
+
+    def twice():
+        assert fake.apply(h, 2, stream=s) == 0 and fake.apply(h, 1, stream=s) == 0
+
+    g = _capture(fake, s, twice)
+    one = fake.lib.fake_used() - base
+    assert 2 * 4096 * 196 <= one < 3 * 4096 * 196
+    e1, e2 = _instantiate(fake, g), _instantiate(fake, g)
+    fake.lib.cudaGraphDestroy(g)
+    fake.lib.cudaGraphExecDestroy(e1)
+    g2 = _capture(fake, s, twice)  # e2 is alive: its work space is not taken
+    assert fake.lib.fake_used() - base == 2 * one
+    fake.log()
+    fake.lib.cudaGraphLaunch(e2, None)
+    assert [t.split()[0] for t in fake.log()] == ["replayed"] * 4
+    fake.lib.cudaGraphExecDestroy(e2)
+    fake.lib.cudaGraphDestroy(g2)
+    for _ in range(5):
+        g = _capture(fake, s, twice)
+        fake.lib.cudaGraphDestroy(g)
+    assert fake.lib.fake_used() - base == 2 * one
+
+
+def test_captured_fp64_apply_without_memory(fake):
+    """no memory for the work space: the FP64 kernel is captured"""
+    h = fake.op((8, 8, 8, 8))
+    assert fake.build(h) == 0
+    fake.log()
+    fake.lib.fake_refuse(0, 1)
+    g = _capture(fake, 1 << 41, lambda: fake.apply(h, stream=1 << 41))
+    log = fake.log()
+    assert any("k_dslash" in t for t in log) and not any("_fx" in t for t in log)
+    fake.lib.cudaGraphDestroy(g)
