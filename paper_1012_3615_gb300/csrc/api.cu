@@ -142,7 +142,7 @@ bri_status bri_build_hops(bri_ctx *ctx, const double *U, bri_prec prec, bri_comp
         return bri_fail(ctx, BRI_EINVAL, "invalid compression");
     cudaStream_t s = as_stream(stream);
     const size_t bytes = sizeof(double2) * 36 * (size_t)ctx->g.V;
-    if (!ctx->U) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->U, bytes));
+    if (!ctx->U) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ctx->U, bytes));
     BRI_TRY_CUDA(ctx, cudaMemcpyAsync(ctx->U, U, bytes, cudaMemcpyDeviceToDevice, s));
     ctx->gen++;
     BRI_RETURN_IF(bri_hops_build_impl(ctx, s));
@@ -272,7 +272,7 @@ static bri_status inverse_action(bri_ctx *ctx, double *S, double *Xout, double *
                                  double tol, int maxit, bri_solve_info *info, cudaStream_t s) {
     const size_t n = (size_t)ctx->g.V * 12, bytes = n * sizeof(double2);
     DevBuf work;
-    BRI_TRY_CUDA(ctx, cudaMalloc(&work.p, 4 * bytes));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &work.p, 4 * bytes));
     double2 *Z = work.as<double2>(), *X = Z + n, *Y = X + n, *t = Y + n;
     bri_status st = BRI_OK;
     bri_solve_info i1{}, i2{};
@@ -485,8 +485,8 @@ bri_status bri_tune_impl(bri_ctx *ctx, bri_prec prec, int nrhs, cudaStream_t s) 
     const size_t elt = prec == BRI_F64 ? 16 : 8;
     const size_t bytes = elt * 12 * (size_t)ctx->g.V * nrhs;
     DevBuf inb, outb;
-    BRI_TRY_CUDA(ctx, cudaMalloc(&inb.p, bytes));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&outb.p, bytes));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &inb.p, bytes));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &outb.p, bytes));
     void *in = inb.p, *out = outb.p;
     BRI_TRY_CUDA(ctx, cudaMemsetAsync(in, 0, bytes, s));
     cudaEvent_t e0, e1;

@@ -16,7 +16,7 @@ struct CapturedWork {
     struct Item {
         void *p;
         size_t bytes;
-        bool busy;
+        bool busy, own;              // in use; by a graph of the solver
         unsigned long long capture;  // id of the capture that took it
         cudaStream_t stream;
     };
@@ -73,9 +73,10 @@ void *bri_captured_work(bri_ctx *ctx, cudaStream_t s, unsigned long long id, cud
                 return nullptr;
             }
             at = w.items.size();
-            w.items.push_back({p, bytes, false, 0, nullptr});
+            w.items.push_back({p, bytes, false, false, 0, nullptr});
         }
         w.items[at].busy = true;
+        w.items[at].own = ctx->own_capture;
         w.items[at].capture = id;
         w.items[at].stream = s;
     }
@@ -108,4 +109,13 @@ bool bri_captured_free(bri_ctx *ctx, bool all) {
             some = true;
         }
     return some;
+}
+
+// a graph of the program, there or yet to run, refers to the context's fields
+bool bri_in_program_graph(bri_ctx *ctx) {
+    if (!ctx->captured) return false;
+    std::lock_guard<std::mutex> lock(ctx->captured->m);
+    for (const CapturedWork::Item &it : ctx->captured->items)
+        if (it.busy && !it.own) return true;
+    return false;
 }

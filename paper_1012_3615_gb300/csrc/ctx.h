@@ -30,10 +30,11 @@ struct bri_ctx {
     bool have64 = false;
     int4 *hopsfx = nullptr;      // fixed-point copy of hops64 (dslash_fx.cu), [40][9][V]; null without memory for it
     unsigned *fxinfo = nullptr;  // whether the links are not unitary, the copy not usable (device)
-    bool have_fx = false, fx_tried = false;
+    bool have_fx = false;
     unsigned fx_attr = 0;        // its kernels whose shared-memory limit is raised on this device
     cudaMemPool_t pool = nullptr;  // stream-ordered work space of the calls, released by bri_destroy
     std::shared_ptr<CapturedWork> captured;
+    bool own_capture = false;      // the solver captures a graph that it can capture again
     LinkStore f32, f16;
     LinkStore p32, p16;  // site-pair interleaved copies (full / 2-row, even t extent)
     SolverWork *work = nullptr;
@@ -77,6 +78,15 @@ bri_status bri_fail(bri_ctx *ctx, bri_status st, const std::string &msg);
         if (s_ != BRI_OK) return s_;   \
     } while (0)
 
+// Device memory for the context.  Where there is none, the context gives back
+// what it holds for speed only, idle work space first and then the fixed-point
+// copy of the FP64 fields, and tries again.
+cudaError_t bri_malloc_bytes(bri_ctx *ctx, void **p, size_t bytes);
+template <class T> cudaError_t bri_malloc(bri_ctx *ctx, T **p, size_t bytes) {
+    return bri_malloc_bytes(ctx, (void **)p, bytes);
+}
+bool bri_give_back(bri_ctx *ctx, int step);
+
 inline bool bri_aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 // device buffer released when it goes out of scope (cudaFree waits for the
@@ -118,7 +128,7 @@ bri_status bri_tc_reserve(bri_ctx *ctx, int nrhs, int cap);
 bri_status bri_dslash_raw(bri_ctx *ctx, void *out, const void *in, int nrhs, double m0, int mode, bri_prec prec,
                           const int *skip, int threads, cudaStream_t s);
 // FP64 apply in fixed point (dslash_fx.cu)
-bri_status bri_fx_reserve(bri_ctx *ctx);
+bri_status bri_fx_reserve(bri_ctx *ctx, cudaStream_t s);
 bool bri_fx_ready(const bri_ctx *ctx);
 bri_status bri_dslash_fx(bri_ctx *ctx, const bri::Geom &g, void *out, const void *in, int nrhs, double m0, int mode,
                          const int *skip, int *ndone, cudaStream_t s);
@@ -127,6 +137,8 @@ bri_status bri_dslash_fx(bri_ctx *ctx, const bri::Geom &g, void *out, const void
 bool bri_capturing(cudaStream_t s, unsigned long long *id, cudaGraph_t *graph);
 void *bri_captured_work(bri_ctx *ctx, cudaStream_t s, unsigned long long id, cudaGraph_t graph, size_t bytes);
 bool bri_captured_free(bri_ctx *ctx, bool all);
+bool bri_in_program_graph(bri_ctx *ctx);
+void bri_solver_drop_graphs(bri_ctx *ctx);
 int bri_dslash_threads(bri_ctx *ctx, bri_prec prec, int nrhs);
 std::string bri_tune_key(bri_ctx *ctx, bri_prec prec, int nrhs);
 bri_status bri_export_hops_impl(bri_ctx *ctx, double2 *out, cudaStream_t s);

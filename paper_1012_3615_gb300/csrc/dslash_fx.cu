@@ -565,19 +565,55 @@ bri_status fx_launch(int mode, bri_ctx *ctx, const Geom &g, const int4 *P, const
 
 }  // namespace
 
-// memory for the fixed-point copy of the FP64 fields and the work space pool;
-// without memory for the copy (ctx->hopsfx null) the FP64 kernel is used
-bri_status bri_fx_reserve(bri_ctx *ctx) {
+// step 0: work space between calls; step 1: the fixed-point copy, unless a graph of
+// the program reads it (the solver's are captured again).  The next build takes
+// the copy back if there is room.  False: nothing was given back
+bool bri_give_back(bri_ctx *ctx, int step) {
+    if (step == 1 && (!ctx->hopsfx || bri_in_program_graph(ctx))) return false;
+    if (cudaDeviceSynchronize() != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (step == 0) {
+        if (ctx->pool) cudaMemPoolTrimTo(ctx->pool, 0);
+        bri_captured_free(ctx, false);
+    } else {
+        bri_solver_drop_graphs(ctx);
+        cudaFree(ctx->hopsfx);
+        ctx->hopsfx = nullptr;
+        ctx->have_fx = false;
+    }
+    return true;
+}
+
+cudaError_t bri_malloc_bytes(bri_ctx *ctx, void **p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    for (int step = 0; e == cudaErrorMemoryAllocation && step < 2; step++) {
+        cudaGetLastError();
+        if (bri_give_back(ctx, step)) e = cudaMalloc(p, bytes);
+    }
+    if (e != cudaSuccess) cudaGetLastError();  // not for the next launch to report
+    return e;
+}
+
+// memory for the fixed-point copy of the FP64 fields (5,760 bytes a site) and the
+// work space pool; without the copy (ctx->hopsfx null) the FP64 kernel is used.
+// The copy is taken where three times as much stays free, enough for FP32 fields
+// (2,880 bytes), the vectors of an FP64 solve (1,536) and the force (11,520), and
+// given back where that was not enough
+bri_status bri_fx_reserve(bri_ctx *ctx, cudaStream_t s) {
     const Geom &g = ctx->g;
     ctx->have_fx = false;
-    if (!ctx->hopsfx && !ctx->fx_tried) {
-        ctx->fx_tried = true;
-        if (cudaMalloc(&ctx->hopsfx, sizeof(int4) * 9 * NCANON * fx_vp(g)) != cudaSuccess) {
+    if (!ctx->hopsfx && !bri_capturing(s, nullptr, nullptr)) {
+        const size_t bytes = sizeof(int4) * 9 * NCANON * fx_vp(g);
+        size_t room = 0, total = 0;
+        if (cudaMemGetInfo(&room, &total) != cudaSuccess || room / 4 < bytes ||
+            cudaMalloc(&ctx->hopsfx, bytes) != cudaSuccess) {
             cudaGetLastError();
             ctx->hopsfx = nullptr;
         }
     }
-    if (!ctx->fxinfo) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->fxinfo, 2 * sizeof(unsigned)));
+    if (!ctx->fxinfo) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ctx->fxinfo, 2 * sizeof(unsigned)));
     if (!ctx->pool) {
         cudaMemPoolProps pp{};
         pp.allocType = cudaMemAllocationTypePinned;

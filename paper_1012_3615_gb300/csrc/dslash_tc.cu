@@ -356,7 +356,7 @@ using namespace bri;
 // bri_dslash_tc); the apply allocates them on first use, which a stream
 // capture does not allow, so callers that capture reserve them first
 bri_status bri_tc_reserve(bri_ctx *ctx, int nrhs, int cap) {
-    if (!ctx->tc_amax) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->tc_amax, sizeof(unsigned) * 65536));
+    if (!ctx->tc_amax) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ctx->tc_amax, sizeof(unsigned) * 65536));
     int rchunk, nt, Rp;
     tc_chunks(nrhs, cap & 511, rchunk, nt, Rp);
     const size_t fbytes = (size_t)ctx->g.V * Rp * 4 * sizeof(uint4);
@@ -364,7 +364,7 @@ bri_status bri_tc_reserve(bri_ctx *ctx, int nrhs, int cap) {
         cudaFree(ctx->tc_f);
         ctx->tc_f = nullptr;
         ctx->tc_fbytes = 0;
-        BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->tc_f, fbytes));
+        BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ctx->tc_f, fbytes));
         ctx->tc_fbytes = fbytes;
     }
     return BRI_OK;

@@ -339,7 +339,14 @@ bri_status bri_force_impl(bri_ctx *ctx, double2 *dU, const double2 *chi, const d
     const Geom &g = ctx->g;
     const size_t fields = (size_t)9 * NCANON * g.V;
     double2 *A = nullptr;
-    BRI_TRY_CUDA(ctx, cudaMallocFromPoolAsync((void **)&A, sizeof(double2) * 2 * fields, ctx->pool, s));
+    const size_t bytes = sizeof(double2) * 2 * fields;
+    cudaError_t e = cudaMallocFromPoolAsync((void **)&A, bytes, ctx->pool, s);
+    for (int step = 0; e == cudaErrorMemoryAllocation && step < 2; step++) {
+        cudaGetLastError();
+        if (bri_give_back(ctx, step)) e = cudaMallocFromPoolAsync((void **)&A, bytes, ctx->pool, s);
+    }
+    if (e != cudaSuccess) cudaGetLastError();
+    BRI_TRY_CUDA(ctx, e);
     double2 *GA = A + fields;
     auto run = [&]() -> bri_status {
         BRI_RETURN_IF(bri_path_sums(ctx, A, s));

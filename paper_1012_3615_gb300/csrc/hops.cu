@@ -402,8 +402,8 @@ bri_status bri_path_sums(bri_ctx *ctx, double2 *A, cudaStream_t s) {
 
 bri_status bri_hops_build_impl(bri_ctx *ctx, cudaStream_t s) {
     const Geom &g = ctx->g;
-    if (!ctx->hops64) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->hops64, sizeof(double2) * 9 * NCANON * (size_t)g.V));
-    BRI_RETURN_IF(bri_fx_reserve(ctx));
+    if (!ctx->hops64) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ctx->hops64, sizeof(double2) * 9 * NCANON * (size_t)g.V));
+    BRI_RETURN_IF(bri_fx_reserve(ctx, s));
     ctx->have64 = false;
     BRI_TRY_CUDA(ctx, cudaMemsetAsync(ctx->fxinfo, 0, 2 * sizeof(unsigned), s));
     k_link_check<<<(unsigned)(((size_t)g.V * 4 + 127) / 128), 128, 0, s>>>(ctx->U, 4 * g.V, ctx->fxinfo);
@@ -434,9 +434,9 @@ bri_status bri_hops_store_impl(bri_ctx *ctx, bri_prec prec, bri_comp comp, cudaS
     }
     st.valid = false;
     if (!st.a) {
-        BRI_TRY_CUDA(ctx, cudaMalloc(&st.a, store_bytes_a(prec, comp) * NCANON * pad32(V)));
+        BRI_TRY_CUDA(ctx, bri_malloc(ctx, &st.a, store_bytes_a(prec, comp) * NCANON * pad32(V)));
         size_t nb = store_bytes_b(prec, comp);
-        if (nb) BRI_TRY_CUDA(ctx, cudaMalloc(&st.b, nb * NCANON * pad32(V)));
+        if (nb) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &st.b, nb * NCANON * pad32(V)));
     }
     st.comp = comp;
     const int T = 128;
@@ -473,7 +473,7 @@ bri_status bri_pair_store_impl(bri_ctx *ctx, bri_prec prec, cudaStream_t s) {
         cudaFree(ps.a);
         ps.a = nullptr;
     }
-    if (!ps.a) BRI_TRY_CUDA(ctx, cudaMalloc(&ps.a, (prec == BRI_F32 ? 16 : 8) * (size_t)E * NCANON * (V / 2)));
+    if (!ps.a) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ps.a, (prec == BRI_F32 ? 16 : 8) * (size_t)E * NCANON * (V / 2)));
     ps.comp = comp;
     dim3 pg((unsigned)((V / 2 + T - 1) / T), NCANON);
     if (prec == BRI_F32) {

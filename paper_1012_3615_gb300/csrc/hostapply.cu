@@ -62,8 +62,8 @@ static bri_status ensure_host_work(bri_ctx *ctx, size_t bytes) {
         if (w->dout) cudaFree(w->dout);
         w->din = w->dout = nullptr;
         w->cap = 0;
-        BRI_TRY_CUDA(ctx, cudaMalloc(&w->din, bytes));
-        BRI_TRY_CUDA(ctx, cudaMalloc(&w->dout, bytes));
+        BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->din, bytes));
+        BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->dout, bytes));
         w->cap = bytes;
     }
     return BRI_OK;

@@ -421,7 +421,7 @@ bri_status ensure_ov(bri_ctx *ctx) {
     OverlapWork *w = new OverlapWork();
     ctx->ov = w;
     w->n = (size_t)ctx->g.V * 12;
-    BRI_TRY_CUDA(ctx, cudaMalloc(&w->cdef, 2 * MAX_WANT * sizeof(double2)));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->cdef, 2 * MAX_WANT * sizeof(double2)));
     return BRI_OK;
 }
 
@@ -431,13 +431,13 @@ bri_status ensure_red(bri_ctx *ctx, int m) {
     if (w->part_cap < need_part) {
         free_ptr(w->part);
         w->part = nullptr;
-        BRI_TRY_CUDA(ctx, cudaMalloc(&w->part, need_part * sizeof(double2)));
+        BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->part, need_part * sizeof(double2)));
         w->part_cap = need_part;
     }
     if (w->h_cap < need_h) {
         free_ptr(w->h);
         w->h = nullptr;
-        BRI_TRY_CUDA(ctx, cudaMalloc(&w->h, need_h * sizeof(double2)));
+        BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->h, need_h * sizeof(double2)));
         w->h_cap = need_h;
     }
     return BRI_OK;
@@ -506,14 +506,14 @@ bri_status lanczos(bri_ctx *ctx, bri_prec aprec, double m0, int nlow, int mmax, 
     if (nlow + 1 > mmax) return bri_fail(ctx, BRI_EINVAL, "max_krylov must exceed the number of wanted eigenpairs");
     const int nw = nlow + 1;
     DevBuf Vb, wb, tmpb, abb, outb, workb, pwb, Sb;
-    BRI_TRY_CUDA(ctx, cudaMalloc(&Vb.p, sizeof(T) * n * (size_t)(mmax + 1)));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&wb.p, sizeof(T) * n));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&tmpb.p, sizeof(T) * n));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&abb.p, sizeof(double) * 2 * (size_t)(mmax + 2)));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&outb.p, sizeof(double) * 2 * nw));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&workb.p, sizeof(double) * 5 * (size_t)mmax * nw));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&pwb.p, (size_t)mmax * nw));
-    if (nlow > 0 && Y) BRI_TRY_CUDA(ctx, cudaMalloc(&Sb.p, sizeof(double2) * (size_t)mmax * nlow));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &Vb.p, sizeof(T) * n * (size_t)(mmax + 1)));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &wb.p, sizeof(T) * n));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &tmpb.p, sizeof(T) * n));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &abb.p, sizeof(double) * 2 * (size_t)(mmax + 2)));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &outb.p, sizeof(double) * 2 * nw));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &workb.p, sizeof(double) * 5 * (size_t)mmax * nw));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &pwb.p, (size_t)mmax * nw));
+    if (nlow > 0 && Y) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &Sb.p, sizeof(double2) * (size_t)mmax * nlow));
     T *V = Vb.as<T>(), *w = wb.as<T>(), *tmp = tmpb.as<T>();
     double2 *S = Sb.as<double2>();
     double *ab = abb.as<double>(), *tri_out = outb.as<double>(), *tri_work = workb.as<double>();
@@ -595,8 +595,8 @@ bri_status build_poly(bri_ctx *ctx, double lo, double hi, double eps, std::vecto
     const double rate = std::log((std::sqrt(kappa) + 1.0) / (std::sqrt(kappa) - 1.0));
     int N = std::max(8, (int)std::floor(0.9 * std::log(1.0 / eps) / rate));
     DevBuf eb_, cb;
-    BRI_TRY_CUDA(ctx, cudaMalloc(&eb_.p, sizeof(unsigned long long)));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&cb.p, sizeof(double) * MAX_DEGREE));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &eb_.p, sizeof(unsigned long long)));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &cb.p, sizeof(double) * MAX_DEGREE));
     double *c = cb.as<double>();
     unsigned long long *e = eb_.as<unsigned long long>();
     for (;;) {
@@ -667,10 +667,10 @@ bri_status poly_apply(bri_ctx *ctx, T *q, const T *v, T *b1, T *b2, T *Bb, T *tm
 bri_status alloc_vecs(bri_ctx *ctx, bri_prec prec) {
     OverlapWork *o = ctx->ov;
     for (auto &p : o->v64)
-        if (!p) BRI_TRY_CUDA(ctx, cudaMalloc(&p, sizeof(double2) * o->n));
+        if (!p) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &p, sizeof(double2) * o->n));
     if (prec != BRI_F64)
         for (auto &p : o->v32)
-            if (!p) BRI_TRY_CUDA(ctx, cudaMalloc(&p, sizeof(float2) * o->n));
+            if (!p) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &p, sizeof(float2) * o->n));
     return BRI_OK;
 }
 
@@ -736,9 +736,9 @@ bri_status setup_modes(bri_ctx *ctx, bri_prec aprec, double m0, int nlow, int ma
         return BRI_OK;
     }
     DevBuf Yb, HYb, Mb;
-    BRI_TRY_CUDA(ctx, cudaMalloc(&Yb.p, sizeof(T) * n * nlow));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&HYb.p, sizeof(T) * n * nlow));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&Mb.p, sizeof(double2) * nlow * nlow * 4));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &Yb.p, sizeof(T) * n * nlow));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &HYb.p, sizeof(T) * n * nlow));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &Mb.p, sizeof(double2) * nlow * nlow * 4));
     T *Y = Yb.as<T>(), *HY = HYb.as<T>();
     double2 *M = Mb.as<double2>();
     double2 *Q = M + nlow * nlow, *C = Q + nlow * nlow, *YHY = C + nlow * nlow;
@@ -803,7 +803,7 @@ bri_status bri_eigs_impl(bri_ctx *ctx, double *evals, double *lmax, double *evec
     } else {
         // FP32 Lanczos (FP32 or FP16 hopping fields): Ritz vectors converted to FP64
         DevBuf y32;
-        if (evecs) BRI_TRY_CUDA(ctx, cudaMalloc(&y32.p, sizeof(float2) * ctx->ov->n * nev));
+        if (evecs) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &y32.p, sizeof(float2) * ctx->ov->n * nev));
         BRI_RETURN_IF(lanczos<float2>(ctx, prec, m0, nev, max_krylov, tol, nullptr, 0, y32.as<float2>(), 0x1012ull, r,
                                       s));
         if (evecs) {
@@ -848,17 +848,17 @@ bri_status bri_overlap_setup_impl(bri_ctx *ctx, double rho, int nlow, double eps
     BRI_RETURN_IF(ensure_red(ctx, MAX_WANT));
     const double m0 = -rho;
     SetupStats st;
-    if (nlow > 0) BRI_TRY_CUDA(ctx, cudaMalloc(&o->lam, sizeof(double) * nlow));
+    if (nlow > 0) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &o->lam, sizeof(double) * nlow));
     if (prec == BRI_F64) {
-        if (nlow > 0) BRI_TRY_CUDA(ctx, cudaMalloc(&o->Z, sizeof(double2) * n * nlow));
+        if (nlow > 0) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &o->Z, sizeof(double2) * n * nlow));
         BRI_RETURN_IF(setup_modes<double2>(ctx, BRI_F64, m0, nlow, max_krylov, tol, o->Z, st, s));
     } else {
         // FP32 / FP16 polynomial: the Lanczos runs, the Rayleigh-Ritz step and the
         // deflation vectors in FP32 too (their accuracy matches the polynomial's);
         // an FP64 copy of the vectors serves the FP64 deflation of the input
         if (nlow > 0) {
-            BRI_TRY_CUDA(ctx, cudaMalloc(&o->Z32, sizeof(float2) * n * nlow));
-            BRI_TRY_CUDA(ctx, cudaMalloc(&o->Z, sizeof(double2) * n * nlow));
+            BRI_TRY_CUDA(ctx, bri_malloc(ctx, &o->Z32, sizeof(float2) * n * nlow));
+            BRI_TRY_CUDA(ctx, bri_malloc(ctx, &o->Z, sizeof(double2) * n * nlow));
         }
         BRI_RETURN_IF(setup_modes<float2>(ctx, prec, m0, nlow, max_krylov, std::max(tol, 1e-6), o->Z32, st, s));
         if (nlow > 0) {

@@ -191,7 +191,7 @@ bri_status bri_ape_impl(bri_ctx *ctx, double2 *V, const double2 *U, double alpha
         return BRI_OK;
     }
     DevBuf tmpb;
-    if (nsteps > 1) BRI_TRY_CUDA(ctx, cudaMalloc(&tmpb.p, bytes));
+    if (nsteps > 1) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &tmpb.p, bytes));
     double2 *tmp = tmpb.as<double2>();
     const unsigned nb = (unsigned)((ctx->g.V + 127) / 128);
     const double2 *src = U;
@@ -208,8 +208,8 @@ bri_status bri_ape_impl(bri_ctx *ctx, double2 *V, const double2 *U, double alpha
 
 bri_status bri_clover_build_impl(bri_ctx *ctx, cudaStream_t s) {
     if (!ctx->clov64) {
-        BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->clov64, sizeof(double2) * 36 * (size_t)ctx->g.V));
-        BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->clov32, sizeof(float4) * 18 * (size_t)ctx->g.V));
+        BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ctx->clov64, sizeof(double2) * 36 * (size_t)ctx->g.V));
+        BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ctx->clov32, sizeof(float4) * 18 * (size_t)ctx->g.V));
     }
     SigmaBlocks sb;
     if (!sigma_blocks(sb)) return bri_fail(ctx, BRI_ESTATE, "sigma_{mu nu} is not block diagonal in this basis");

@@ -455,6 +455,10 @@ static void free_vecs(VecSet &v) {
     }
 }
 
+void bri_solver_drop_graphs(bri_ctx *ctx) {
+    if (ctx->work) drop_graphs(ctx->work);
+}
+
 void bri_solver_free(bri_ctx *ctx) {
     SolverWork *w = ctx->work;
     if (!w) return;
@@ -475,7 +479,7 @@ void bri_solver_free(bri_ctx *ctx) {
 
 static bri_status alloc_vecs(bri_ctx *ctx, VecSet &v, size_t bytes) {
     void **a[] = {&v.x, &v.r, &v.rhat, &v.p, &v.v, &v.s, &v.t};
-    for (void **p : a) BRI_TRY_CUDA(ctx, cudaMalloc(p, bytes));
+    for (void **p : a) BRI_TRY_CUDA(ctx, bri_malloc(ctx, p, bytes));
     return BRI_OK;
 }
 
@@ -495,15 +499,15 @@ static bri_status ensure_work(bri_ctx *ctx, int nrhs, bool need64, bool need32) 
     if (need64 || had64) BRI_RETURN_IF(alloc_vecs(ctx, w->v64, sizeof(double2) * n * R));
     if (need32 || had32) {
         BRI_RETURN_IF(alloc_vecs(ctx, w->v32, sizeof(float2) * n * R));
-        BRI_TRY_CUDA(ctx, cudaMalloc(&w->r64, sizeof(double2) * n * R));
+        BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->r64, sizeof(double2) * n * R));
     }
-    BRI_TRY_CUDA(ctx, cudaMalloc(&w->st, sizeof(BiState) * R));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&w->flag, sizeof(int) * R));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&w->done, sizeof(int) * R));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&w->part, sizeof(double) * NPART * RBLK * R));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&w->tick, sizeof(unsigned) * R));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->st, sizeof(BiState) * R));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->flag, sizeof(int) * R));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->done, sizeof(int) * R));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->part, sizeof(double) * NPART * RBLK * R));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->tick, sizeof(unsigned) * R));
     BRI_TRY_CUDA(ctx, cudaMemset(w->tick, 0, sizeof(unsigned) * R));
-    BRI_TRY_CUDA(ctx, cudaMalloc(&w->nrm, sizeof(double) * 2 * R));
+    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->nrm, sizeof(double) * 2 * R));
     BRI_TRY_CUDA(ctx, cudaStreamCreateWithFlags(&w->own, cudaStreamNonBlocking));
     return BRI_OK;
 }
@@ -592,9 +596,14 @@ bri_status bicgstab(bri_ctx *ctx, const VecSet &vs, const T *b, bool have_x0, in
         cudaGraph_t graph;
         const long before = ctx->launches;
         BRI_TRY_CUDA(ctx, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+        ctx->own_capture = true;
         bri_status st = enqueue_iters<T>(ctx, vs, nrhs, m0, prec, K, s);
+        ctx->own_capture = false;
         cudaError_t e = cudaStreamEndCapture(s, &graph);
-        if (st != BRI_OK) return st;
+        if (st != BRI_OK) {
+            if (e == cudaSuccess) cudaGraphDestroy(graph);
+            return st;
+        }
         if (e != cudaSuccess) return bri_fail(ctx, BRI_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
         BRI_TRY_CUDA(ctx, cudaGraphInstantiate(&run.exec, graph, 0));
         cudaGraphDestroy(graph);
@@ -758,7 +767,7 @@ bri_status bri_solve_impl(bri_ctx *ctx, double *x, const double *b, int nrhs, do
     const size_t n = (size_t)ctx->g.V * 12;
     if (mode == 0) {
         BRI_RETURN_IF(ensure_work(ctx, 1, true, false));
-        if (!ctx->work->r64) BRI_TRY_CUDA(ctx, cudaMalloc(&ctx->work->r64, sizeof(double2) * n * ctx->work->nrhs));
+        if (!ctx->work->r64) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ctx->work->r64, sizeof(double2) * n * ctx->work->nrhs));
     } else {
         if (mode <= 2 && nrhs > 1) {
             // sequential right-hand sides in modes 1, 2; a right-hand side that

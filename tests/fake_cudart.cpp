@@ -165,6 +165,11 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3 block, void **arg
         log("captured " + l.name);
         return cudaSuccess;
     }
+    if (l.name.find("k_dslash") != std::string::npos && l.name.find("_fx") == std::string::npos) {
+        char io[64];  // (mode, fields, in, out, ...)
+        snprintf(io, sizeof io, " in %llx out %llx", *(unsigned long long *)args[2], *(unsigned long long *)args[3]);
+        l.name += io;
+    }
     log("run " + l.name + " " + std::to_string(grid.x) + "x" + std::to_string(grid.y) + " " + std::to_string(block.x));
     return cudaSuccess;
 }

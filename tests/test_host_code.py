@@ -191,3 +191,102 @@ def test_captured_fp64_apply_without_memory(fake):
     log = fake.log()
     assert any("k_dslash" in t for t in log) and not any("_fx" in t for t in log)
     fake.lib.cudaGraphDestroy(g)
+
+
+F64, F32, FULL, TWO_ROW = 0, 1, 0, 1
+SITE_COPY = 5760  # bytes of the fixed-point copy
+
+
+def _kind(log):
+    """which FP64 apply ran"""
+    return {"fx" if "k_dslash_fx" in t else "fp64" for t in log if t.startswith("run") and "k_dslash" in t}
+
+
+def test_fixed_point_copy_only_with_room(fake):
+    """the copy is taken where three times as much stays free, and tried again by
+    the next build"""
+    h = fake.op((8, 8, 8, 8))
+    need = 4096 * (576 + SITE_COPY)
+    fake.lib.fake_budget(need + 4 * 4096 * SITE_COPY - 4096)
+    assert fake.build(h) == 0 and fake.apply(h) == 0
+    assert _kind(fake.log()) == {"fp64"}
+    fake.lib.fake_budget(1 << 40)
+    assert fake.build(h) == 0 and fake.apply(h) == 0
+    assert _kind(fake.log()) == {"fx"}
+
+
+@pytest.mark.parametrize("what", ["store", "solve", "force"])
+def test_fixed_point_copy_gives_way(fake, what):
+    """a required allocation that fails takes the memory of the copy; the solver's
+    graphs that read it go with it"""
+    lib = fake.lib
+    h = fake.op((8, 8, 8, 8))
+    assert fake.build(h) == 0 and fake.apply(h) == 0 and fake.solve(h, 0) == 0
+    assert "fx" in str(fake.log())
+    lib.fake_budget(lib.fake_used() + 4096 * 200)
+    if what == "store":
+        assert lib.bri_store_hops(h, F32, FULL, None) == 0
+    elif what == "solve":
+        lib.fake_budget(1 << 40)
+        assert lib.bri_store_hops(h, F32, TWO_ROW, None) == 0
+        lib.fake_budget(lib.fake_used() + 4096 * 200)
+        assert fake.solve(h, 4, nrhs=2) == 0
+    else:
+        lib.fake_budget(lib.fake_used() + 4096 * (2 * SITE_COPY - 1000))
+        assert lib.bri_force(h, 1 << 50, 1 << 56, 1 << 57, 0.0, 1, None) == 0
+    fake.log()
+    assert fake.apply(h) == 0 and fake.solve(h, 0) == 0
+    log = fake.log()
+    assert _kind(log) == {"fp64"} and not any("STALE" in t or "replayed" in t and "_fx" in t for t in log)
+    lib.fake_budget(1 << 40)
+    assert fake.build(h) == 0 and fake.apply(h) == 0 and fake.solve(h, 0) == 0
+    log = fake.log()
+    assert _kind(log) == {"fx"} and not any("STALE" in t for t in log)
+
+
+def test_fixed_point_copy_stays_for_a_program_graph(fake):
+    """a captured apply of the program reads the copy for as long as its graph is
+    there: an allocation that fails then is reported, and the next launch is not
+    taken for the failure"""
+    lib = fake.lib
+    h = fake.op((8, 8, 8, 8))
+    assert fake.build(h) == 0
+    g = _capture(fake, 1 << 41, lambda: fake.apply(h, stream=1 << 41))
+    e = _instantiate(fake, g)
+    lib.cudaGraphDestroy(g)
+    lib.fake_budget(lib.fake_used() + 4096 * 200)
+    assert lib.bri_store_hops(h, F32, FULL, None) == -2  # BRI_ENOMEM
+    fake.log()
+    lib.cudaGraphLaunch(e, None)
+    assert not any("STALE" in t for t in fake.log())
+    assert fake.apply(h) == 0
+    lib.cudaGraphExecDestroy(e)
+    assert lib.bri_store_hops(h, F32, FULL, None) == 0
+
+
+def test_pool_memory_gives_way_first(fake):
+    lib = fake.lib
+    h = fake.op((8, 8, 8, 8))
+    assert fake.build(h) == 0
+    before = lib.fake_used()
+    assert fake.apply(h, 30) == 0
+    assert lib.fake_used() - before > 4096 * 196 * 29
+    lib.fake_budget(lib.fake_used())
+    assert lib.bri_store_hops(h, F32, TWO_ROW, None) == 0
+    fake.log()
+    assert fake.apply(h) == 0
+    assert _kind(fake.log()) == {"fx"}
+
+
+def test_work_space_refused_after_the_first_chunk(fake):
+    """32 right-hand sides a launch: the other 8 through the FP64 kernel, at their
+    own addresses"""
+    h = fake.op((8, 8, 8, 8))
+    assert fake.build(h) == 0
+    fake.log()
+    fake.lib.fake_refuse(1, 1)
+    field = 4096 * 12 * 16
+    assert fake.apply(h, 40) == 0
+    log = [t for t in fake.log() if "k_dslash" in t]
+    assert len(log) == 2 and "_fx" in log[0] and "_fx" not in log[1]
+    assert "in %x out %x" % ((1 << 56) + 32 * field, (1 << 50) + 32 * field) in log[1]
