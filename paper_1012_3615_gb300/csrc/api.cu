@@ -373,6 +373,7 @@ bri_status bri_set_clover(bri_ctx *ctx, double csw, void *stream) {
     if (!ctx) return BRI_EINVAL;
     if (!std::isfinite(csw)) return bri_fail(ctx, BRI_EINVAL, "csw must be finite");
     ctx->gen++;
+    const double before = ctx->csw;
     ctx->csw = csw;
     if (csw == 0.0) {
         ctx->g.clov64 = nullptr;
@@ -380,7 +381,9 @@ bri_status bri_set_clover(bri_ctx *ctx, double csw, void *stream) {
         return BRI_OK;
     }
     if (!ctx->U) return bri_fail(ctx, BRI_ESTATE, "no links: call bri_build_hops first");
-    return bri_clover_build_impl(ctx, as_stream(stream));
+    const bri_status st = bri_clover_build_impl(ctx, as_stream(stream));
+    if (st == BRI_ENOMEM) ctx->csw = before;  // the term is as it was
+    return st;
 }
 
 // ---- spectra and the overlap operator ------------------------------------------------

@@ -592,7 +592,10 @@ cudaError_t bri_malloc_bytes(bri_ctx *ctx, void **p, size_t bytes) {
         cudaGetLastError();
         if (bri_give_back(ctx, step)) e = cudaMalloc(p, bytes);
     }
-    if (e != cudaSuccess) cudaGetLastError();  // not for the next launch to report
+    if (e != cudaSuccess) {
+        cudaGetLastError();  // not for the next launch to report
+        *p = nullptr;
+    }
     return e;
 }
 

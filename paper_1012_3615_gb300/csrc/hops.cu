@@ -433,12 +433,10 @@ bri_status bri_hops_store_impl(bri_ctx *ctx, bri_prec prec, bri_comp comp, cudaS
         st.a = st.b = nullptr;
     }
     st.valid = false;
-    if (!st.a) {
-        BRI_TRY_CUDA(ctx, bri_malloc(ctx, &st.a, store_bytes_a(prec, comp) * NCANON * pad32(V)));
-        size_t nb = store_bytes_b(prec, comp);
-        if (nb) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &st.b, nb * NCANON * pad32(V)));
-    }
     st.comp = comp;
+    if (!st.a) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &st.a, store_bytes_a(prec, comp) * NCANON * pad32(V)));
+    const size_t nb = store_bytes_b(prec, comp);
+    if (nb && !st.b) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &st.b, nb * NCANON * pad32(V)));
     const int T = 128;
     dim3 grid((unsigned)((V + T - 1) / T), NCANON);
     if (prec == BRI_F32) {

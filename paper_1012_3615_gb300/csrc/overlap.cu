@@ -417,11 +417,10 @@ void bri_overlap_free(bri_ctx *ctx) {
 namespace {
 
 bri_status ensure_ov(bri_ctx *ctx) {
-    if (ctx->ov) return BRI_OK;
-    OverlapWork *w = new OverlapWork();
-    ctx->ov = w;
+    if (!ctx->ov) ctx->ov = new OverlapWork();
+    OverlapWork *w = ctx->ov;
     w->n = (size_t)ctx->g.V * 12;
-    BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->cdef, 2 * MAX_WANT * sizeof(double2)));
+    if (!w->cdef) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->cdef, 2 * MAX_WANT * sizeof(double2)));
     return BRI_OK;
 }
 
@@ -431,12 +430,14 @@ bri_status ensure_red(bri_ctx *ctx, int m) {
     if (w->part_cap < need_part) {
         free_ptr(w->part);
         w->part = nullptr;
+        w->part_cap = 0;
         BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->part, need_part * sizeof(double2)));
         w->part_cap = need_part;
     }
     if (w->h_cap < need_h) {
         free_ptr(w->h);
         w->h = nullptr;
+        w->h_cap = 0;
         BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->h, need_h * sizeof(double2)));
         w->h_cap = need_h;
     }

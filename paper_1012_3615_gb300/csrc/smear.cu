@@ -207,10 +207,8 @@ bri_status bri_ape_impl(bri_ctx *ctx, double2 *V, const double2 *U, double alpha
 }
 
 bri_status bri_clover_build_impl(bri_ctx *ctx, cudaStream_t s) {
-    if (!ctx->clov64) {
-        BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ctx->clov64, sizeof(double2) * 36 * (size_t)ctx->g.V));
-        BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ctx->clov32, sizeof(float4) * 18 * (size_t)ctx->g.V));
-    }
+    if (!ctx->clov64) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ctx->clov64, sizeof(double2) * 36 * (size_t)ctx->g.V));
+    if (!ctx->clov32) BRI_TRY_CUDA(ctx, bri_malloc(ctx, &ctx->clov32, sizeof(float4) * 18 * (size_t)ctx->g.V));
     SigmaBlocks sb;
     if (!sigma_blocks(sb)) return bri_fail(ctx, BRI_ESTATE, "sigma_{mu nu} is not block diagonal in this basis");
     k_clover_build<<<(ctx->g.V + 127) / 128, 128, 0, s>>>(ctx->U, ctx->g, sb, ctx->csw, ctx->clov64, ctx->clov32);

@@ -483,21 +483,10 @@ static bri_status alloc_vecs(bri_ctx *ctx, VecSet &v, size_t bytes) {
     return BRI_OK;
 }
 
-// work spaces for nrhs right-hand sides; need32 / need64 select the vector sets
-static bri_status ensure_work(bri_ctx *ctx, int nrhs, bool need64, bool need32) {
-    const size_t n = (size_t)ctx->g.V * 12;
-    SolverWork *w = ctx->work;
-    if (w && w->nrhs >= nrhs && (!need64 || w->v64.x) && (!need32 || w->v32.x)) return BRI_OK;
-    const int have_nrhs = w ? w->nrhs : 0;
-    const bool had64 = w && w->v64.x, had32 = w && w->v32.x;
-    bri_solver_free(ctx);
-    w = new SolverWork();
-    ctx->work = w;
-    w->n = n;
-    w->nrhs = nrhs > have_nrhs ? nrhs : have_nrhs;
-    const size_t R = w->nrhs;
-    if (need64 || had64) BRI_RETURN_IF(alloc_vecs(ctx, w->v64, sizeof(double2) * n * R));
-    if (need32 || had32) {
+static bri_status alloc_work(bri_ctx *ctx, SolverWork *w, bool with64, bool with32) {
+    const size_t n = w->n, R = w->nrhs;
+    if (with64) BRI_RETURN_IF(alloc_vecs(ctx, w->v64, sizeof(double2) * n * R));
+    if (with32) {
         BRI_RETURN_IF(alloc_vecs(ctx, w->v32, sizeof(float2) * n * R));
         BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->r64, sizeof(double2) * n * R));
     }
@@ -510,6 +499,21 @@ static bri_status ensure_work(bri_ctx *ctx, int nrhs, bool need64, bool need32) 
     BRI_TRY_CUDA(ctx, bri_malloc(ctx, &w->nrm, sizeof(double) * 2 * R));
     BRI_TRY_CUDA(ctx, cudaStreamCreateWithFlags(&w->own, cudaStreamNonBlocking));
     return BRI_OK;
+}
+
+// work spaces for nrhs right-hand sides; need32 / need64 select the vector sets
+static bri_status ensure_work(bri_ctx *ctx, int nrhs, bool need64, bool need32) {
+    SolverWork *w = ctx->work;
+    if (w && w->nrhs >= nrhs && (!need64 || w->v64.x) && (!need32 || w->v32.x)) return BRI_OK;
+    const int have_nrhs = w ? w->nrhs : 0;
+    const bool had64 = w && w->v64.x, had32 = w && w->v32.x;
+    bri_solver_free(ctx);
+    w = ctx->work = new SolverWork();
+    w->n = (size_t)ctx->g.V * 12;
+    w->nrhs = nrhs > have_nrhs ? nrhs : have_nrhs;
+    const bri_status st = alloc_work(ctx, w, need64 || had64, need32 || had32);
+    if (st != BRI_OK) bri_solver_free(ctx);  // all of it or nothing
+    return st;
 }
 
 namespace {

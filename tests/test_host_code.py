@@ -290,3 +290,45 @@ def test_work_space_refused_after_the_first_chunk(fake):
     log = [t for t in fake.log() if "k_dslash" in t]
     assert len(log) == 2 and "_fx" in log[0] and "_fx" not in log[1]
     assert "in %x out %x" % ((1 << 56) + 32 * field, (1 << 50) + 32 * field) in log[1]
+
+
+def test_calls_that_run_out_of_memory_can_be_repeated(fake):
+    """every allocation of a call refused in turn (with what would give way): the
+    call succeeds or says so, and its repetition leaves the context with the same
+    memory as one that never failed"""
+    lib = fake.lib
+
+    def run(refuse):
+        """memory of a context whose calls were all repeated, and whether one failed"""
+        lib.fake_reset()
+        at = lib.fake_used()
+        h = fake.op((8, 8, 8, 8))
+        failed = False
+        calls = [lambda: fake.build(h, prec=F32, comp=FULL), lambda: fake.apply(h), lambda: fake.solve(h, 1),
+                 lambda: lib.bri_store_hops(h, F32, TWO_ROW, None), lambda: lib.bri_store_hops(h, F32, FULL, None),
+                 lambda: lib.bri_set_clover(h, ctypes.c_double(1.0), None), lambda: fake.solve(h, 4, nrhs=2),
+                 lambda: fake.solve(h, 0), lambda: lib.bri_set_clover(h, ctypes.c_double(0.0), None)]
+        for i, call in enumerate(calls):
+            lib.fake_refuse(*(refuse[1:] if refuse and refuse[0] == i else (-1, 0)))
+            st = call()
+            assert st in (0, -2), (refuse, i, st)
+            failed = failed or st != 0
+            lib.fake_refuse(-1, 0)
+            if st:
+                assert call() == 0, (refuse, i)
+        # what may have given way comes back (the copy; a new set of solver vectors
+        # without graphs, then one graph), and idle work space goes
+        assert fake.build(h, prec=F32, comp=FULL) == 0 and fake.solve(h, 4, nrhs=3) == 0 and fake.solve(h, 0) == 0
+        lib.fake_refuse(0, 1)
+        assert lib.bri_store_hops(h, F32, TWO_ROW, None) == 0
+        return lib.fake_used() - at, failed
+
+    want, failed = run(None)
+    assert not failed
+    hits = 0
+    for i in (0, 2, 3, 4, 5, 6, 7):
+        for k in range(30):
+            used, failed = run((i, k, 9))
+            hits += failed
+            assert used == want, (i, k, used, want)
+    assert hits > 20
