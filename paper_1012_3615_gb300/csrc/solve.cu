@@ -18,6 +18,7 @@
 #include <chrono>
 #include <cmath>
 #include <map>
+#include <type_traits>
 #include <vector>
 
 #include "ctx.h"
@@ -96,9 +97,19 @@ template <int NV> BRI_D void gather_partials(const double *part, double out[NV])
 
 // per-thread accumulator of the BiCGstab reductions: FP32 vectors sum their few
 // elements per thread in FP32 (FP64 is 1/64 of the FP32 rate on this GPU),
-// FP64 vectors in FP64; partials across threads and blocks are always FP64
+// FP64 vectors in FP64; partials across threads and blocks are always FP64.
+// A thread has four elements or more.  Up to EXACT_N elements, 19,456 sites, it
+// keeps the rounding errors of their sum (SumF32) and is as exact as one to three
+// elements a thread; the sums that end in FP64 by the block would cost more than
+// that with fewer per thread (8^4, 12 right-hand sides, cold: alpha, omega, x/r
+// 10.6, 11.2, 15.9 us in plain FP32, 11.6, 13.0, 17.7 with the errors, 15.5, 16.7,
+// 22.9 with two elements a thread)
 template <typename T> struct AccT { using A = double; };
 template <> struct AccT<float2> { using A = float; };
+template <typename A> BRI_D double value(A a) {
+    if constexpr (std::is_same_v<A, SumF32>) return a.get();
+    else return a;
+}
 
 BRI_D double2 dcdiv(double2 a, double2 b) {
     double d = b.x * b.x + b.y * b.y;
@@ -147,11 +158,17 @@ template <typename T> BRI_D T cfms(T a, T b, T z) {
 }
 // (re, im) += conj(a) b;  s += |a|^2
 template <typename T, typename A> BRI_D void dot_add(T a, T b, A &re, A &im) {
-    re = fma((A)a.x, (A)b.x, fma((A)a.y, (A)b.y, re));
-    im = fma((A)a.x, (A)b.y, fma(-(A)a.y, (A)b.x, im));
+    if constexpr (std::is_same_v<A, SumF32>) {
+        re.add(fmaf(a.x, b.x, a.y * b.y));
+        im.add(fmaf(a.x, b.y, -(a.y * b.x)));
+    } else {
+        re = fma((A)a.x, (A)b.x, fma((A)a.y, (A)b.y, re));
+        im = fma((A)a.x, (A)b.y, fma(-(A)a.y, (A)b.x, im));
+    }
 }
 template <typename T, typename A> BRI_D void norm_add(T a, A &s) {
-    s = fma((A)a.x, (A)a.x, fma((A)a.y, (A)a.y, s));
+    if constexpr (std::is_same_v<A, SumF32>) s.add(fmaf(a.x, a.x, a.y * a.y));
+    else s = fma((A)a.x, (A)a.x, fma((A)a.y, (A)a.y, s));
 }
 
 template <typename T>
@@ -171,14 +188,13 @@ __global__ void __launch_bounds__(RT) k_bi_p(T *p, const T *__restrict__ r, cons
         });
 }
 
-template <typename T>
+template <typename T, typename A>
 __global__ void __launch_bounds__(RT) k_bi_alpha(const T *__restrict__ rhat, const T *__restrict__ v, BiState *st,
                                                  int *flag, double *part, unsigned *tick, size_t n) {
     const int rh = blockIdx.y;
     if (flag[rh]) return;
     rhat += rh * n; v += rh * n;
-    using A = typename AccT<T>::A;
-    A ac[2] = {0, 0};
+    A ac[2] = {};
     struct In { Pack<T> h, v; };
     for_packs<T>(
         n, [&](size_t i) { return In{pk(rhat, i), pk(v, i)}; },
@@ -186,7 +202,7 @@ __global__ void __launch_bounds__(RT) k_bi_alpha(const T *__restrict__ rhat, con
 #pragma unroll
             for (int k = 0; k < PK<T>; k++) dot_add(z.h.e[k], z.v.e[k], ac[0], ac[1]);
         });
-    double acc[2] = {ac[0], ac[1]};
+    double acc[2] = {value(ac[0]), value(ac[1])};
     if (partial_and_ticket<2>(acc, part + (size_t)rh * RBLK * NPART, tick + rh)) {
         double s[2];
         gather_partials<2>(part + (size_t)rh * RBLK * NPART, s);
@@ -216,14 +232,13 @@ __global__ void __launch_bounds__(RT) k_bi_s(T *__restrict__ s, const T *__restr
         });
 }
 
-template <typename T>
+template <typename T, typename A>
 __global__ void __launch_bounds__(RT) k_bi_omega(const T *__restrict__ t, const T *__restrict__ s, BiState *st,
                                                  int *flag, double *part, unsigned *tick, size_t n) {
     const int rh = blockIdx.y;
     if (flag[rh]) return;
     t += rh * n; s += rh * n;
-    using A = typename AccT<T>::A;
-    A ac[3] = {0, 0, 0};
+    A ac[3] = {};
     struct In { Pack<T> t, s; };
     for_packs<T>(
         n, [&](size_t i) { return In{pk(t, i), pk(s, i)}; },
@@ -234,7 +249,7 @@ __global__ void __launch_bounds__(RT) k_bi_omega(const T *__restrict__ t, const 
                 norm_add(z.t.e[k], ac[2]);
             }
         });
-    double acc[3] = {ac[0], ac[1], ac[2]};
+    double acc[3] = {value(ac[0]), value(ac[1]), value(ac[2])};
     if (partial_and_ticket<3>(acc, part + (size_t)rh * RBLK * NPART, tick + rh)) {
         double q[3];
         gather_partials<3>(part + (size_t)rh * RBLK * NPART, q);
@@ -246,7 +261,7 @@ __global__ void __launch_bounds__(RT) k_bi_omega(const T *__restrict__ t, const 
     }
 }
 
-template <typename T>
+template <typename T, typename A>
 __global__ void __launch_bounds__(RT) k_bi_xr(T *x, T *__restrict__ r, const T *__restrict__ p, const T *__restrict__ s,
                                               const T *__restrict__ t, const T *__restrict__ rhat, BiState *st,
                                               int *flag, double *part, unsigned *tick, size_t n) {
@@ -255,8 +270,7 @@ __global__ void __launch_bounds__(RT) k_bi_xr(T *x, T *__restrict__ r, const T *
     const T a = tc<T>(st[rh].alpha), om = tc<T>(st[rh].omega);
     const size_t o = rh * n;
     x += o; r += o; p += o; s += o; t += o; rhat += o;
-    using A = typename AccT<T>::A;
-    A ac[3] = {0, 0, 0};
+    A ac[3] = {};
     struct In { Pack<T> x, p, s, t, h; };
     for_packs<T>(
         n, [&](size_t i) { return In{pk(x, i), pk(p, i), pk(s, i), pk(t, i), pk(rhat, i)}; },
@@ -272,7 +286,7 @@ __global__ void __launch_bounds__(RT) k_bi_xr(T *x, T *__restrict__ r, const T *
             put(x, i, z.x);
             put(r, i, z.s);
         });
-    double acc[3] = {ac[0], ac[1], ac[2]};
+    double acc[3] = {value(ac[0]), value(ac[1]), value(ac[2])};
     if (partial_and_ticket<3>(acc, part + (size_t)rh * RBLK * NPART, tick + rh)) {
         double q[3];
         gather_partials<3>(part + (size_t)rh * RBLK * NPART, q);
@@ -298,7 +312,7 @@ __global__ void k_bi_init(T *r, T *rhat, T *p, T *v, const T *b, int have_ax, Bi
     const int rh = blockIdx.y;
     const size_t o = rh * n;
     using A = typename AccT<T>::A;
-    A ac[2] = {0, 0};
+    A ac[2] = {};
     for (size_t i = (size_t)blockIdx.x * RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT) {
         T bi = b[o + i];
         T ri = have_ax ? csub(bi, r[o + i]) : bi;
@@ -524,29 +538,41 @@ template <typename T> dim3 vec_grid(size_t n, int nrhs) {
     return dim3((unsigned)(b < 1 ? 1 : b < RBLK ? b : RBLK), (unsigned)nrhs);
 }
 
+// FP32 vectors of which 304 blocks would have up to three elements per thread
+constexpr size_t EXACT_N = (size_t)304 * RT * 3;
+
 // enqueue `iters` BiCGstab iterations on vectors vs (element T) for nrhs right-hand sides
 template <typename T>
 bri_status enqueue_iters(bri_ctx *ctx, const VecSet &vs, int nrhs, double m0, bri_prec prec, int iters,
                          cudaStream_t s) {
     SolverWork *w = ctx->work;
     const size_t n = w->n;
+    const bool exact = sizeof(T) == 8 && n <= EXACT_N;
     const dim3 grid = vec_grid<T>(n, nrhs);
     T *x = (T *)vs.x, *r = (T *)vs.r, *rh = (T *)vs.rhat, *p = (T *)vs.p, *v = (T *)vs.v, *sv = (T *)vs.s,
       *t = (T *)vs.t;
     const int thr = bri_dslash_threads(ctx, prec, nrhs);
-    for (int it = 0; it < iters; it++) {
+    auto step = [&](auto acc) -> bri_status {
+        using A = decltype(acc);
         k_bi_p<T><<<grid, RT, 0, s>>>(p, r, v, w->st, w->flag, n);
         BRI_LAUNCHED(ctx);
         BRI_RETURN_IF(bri_dslash_raw(ctx, v, p, nrhs, m0, 0, prec, w->flag, thr, s));
-        k_bi_alpha<T><<<grid, RT, 0, s>>>(rh, v, w->st, w->flag, w->part, w->tick, n);
+        k_bi_alpha<T, A><<<grid, RT, 0, s>>>(rh, v, w->st, w->flag, w->part, w->tick, n);
         BRI_LAUNCHED(ctx);
         k_bi_s<T><<<grid, RT, 0, s>>>(sv, r, v, w->st, w->flag, n);
         BRI_LAUNCHED(ctx);
         BRI_RETURN_IF(bri_dslash_raw(ctx, t, sv, nrhs, m0, 0, prec, w->flag, thr, s));
-        k_bi_omega<T><<<grid, RT, 0, s>>>(t, sv, w->st, w->flag, w->part, w->tick, n);
+        k_bi_omega<T, A><<<grid, RT, 0, s>>>(t, sv, w->st, w->flag, w->part, w->tick, n);
         BRI_LAUNCHED(ctx);
-        k_bi_xr<T><<<grid, RT, 0, s>>>(x, r, p, sv, t, rh, w->st, w->flag, w->part, w->tick, n);
+        k_bi_xr<T, A><<<grid, RT, 0, s>>>(x, r, p, sv, t, rh, w->st, w->flag, w->part, w->tick, n);
         BRI_LAUNCHED(ctx);
+        return BRI_OK;
+    };
+    for (int it = 0; it < iters; it++) {
+        bri_status st;
+        if constexpr (sizeof(T) == 8) st = exact ? step(SumF32()) : step(float());
+        else st = step(double());
+        BRI_RETURN_IF(st);
     }
     return BRI_OK;
 }

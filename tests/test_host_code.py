@@ -332,3 +332,38 @@ def test_calls_that_run_out_of_memory_can_be_repeated(fake):
             hits += failed
             assert used == want, (i, k, used, want)
     assert hits > 20
+
+
+def test_fp32_sums_without_loss(tmp_path):
+    """the accumulator of the FP32 solver's dot products: sums of FP32 numbers of
+    any sign and size as exact as FP64 gives them, to 2^-44 of the sum of their
+    magnitudes (one element a thread went to FP64 by itself)"""
+    from paper_1012_3615_gb300 import build
+
+    src = tmp_path / "sum.cu"
+    src.write_text(r"""
+#include <cmath>
+#include <cstdio>
+#include <cstdlib>
+#include "common.cuh"
+int main() {
+    srand(5);
+    double worst = 0;
+    for (int t = 0; t < 20000; t++) {
+        bri::SumF32 s;
+        double ref = 0, size = 0;
+        const int n = 1 + t % 12;
+        for (int i = 0; i < n; i++) {
+            const float v = (float)(std::ldexp(rand() / (double)RAND_MAX - 0.5, rand() % 30 - 15));
+            s.add(v);
+            ref += v;
+            size += std::fabs(v);
+        }
+        worst = std::fmax(worst, std::fabs(s.get() - ref) / size);
+    }
+    printf("%.3e", worst);
+}
+""")
+    exe = str(tmp_path / "sum")
+    subprocess.run([build_nvcc()] + build.FLAGS + ["-o", exe, str(src)], check=True, capture_output=True, text=True)
+    assert float(subprocess.run([exe], check=True, capture_output=True, text=True).stdout) <= 2.0**-44
