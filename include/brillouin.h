@@ -386,7 +386,9 @@ bri_status bri_apply_overlap(bri_ctx *ctx, double *out, const double *in, int nr
 /* Tune the launch shape of the apply kernels for (prec, nrhs) on this
  * lattice (timed with CUDA events, result cached in the context and, when the
  * environment variable BRI_TUNE_CACHE names a file, in that file).
- * Requires the fields of that precision.  Synchronises the stream. */
+ * Requires the fields of that precision.  Synchronises the stream.  BRI_F64:
+ * the fixed-point apply has one shape, so nothing is timed or stored where it
+ * can be used. */
 bri_status bri_tune(bri_ctx *ctx, bri_prec prec, int nrhs, void *stream);
 
 /* Set / read the launch shape of the apply kernels for (prec, nrhs) (what
@@ -421,8 +423,13 @@ bri_status bri_tune(bri_ctx *ctx, bri_prec prec, int nrhs, void *stream);
  * the tuner considers it for BRI_F16 fields and nrhs >= 2 only, the accuracy
  * class it shares).  For 16384 the low bits give the right-hand sides one
  * warp takes per pass (an even number 2..12; 0 or anything else: 12).
+ * The shape for BRI_F64 is that of the FP64 kernel, which runs where the
+ * fixed-point apply cannot (bri_apply; also without memory for its copy of the
+ * fields).  On lattices of up to 4,096 sites 10240, 12288 and 18432, and FP32
+ * and FP16 fields with the clover term, run the pair loop of the field format
+ * with the hop list of a site in four parts, whatever the block size.
  * bri_get_threads returns the current choice or a negative bri_status;
- * untuned: the unrolled kernel at 128 threads (BRI_F64); on an x extent of
+ * untuned: 128 threads (BRI_F64); on an x extent of
  * 32, 22528 + 64 (FP32 and FP16 fields); otherwise 128 threads with variant 10240 (FP32 full fields), 18432
  * (FP32 2-row, FP16 full and 2-row fields) or 12288 (8-parameter fields).  bri_set_threads returns BRI_EINVAL for nrhs < 1, a
  * negative value, 1..31 or more than 1024 threads (other than with 16384), or

@@ -485,6 +485,7 @@ const char *bri_last_error(bri_ctx *ctx) { return ctx ? ctx->err.c_str() : g_cre
 
 // ---- launch-shape tuner ---------------------------------------------------------
 bri_status bri_tune_impl(bri_ctx *ctx, bri_prec prec, int nrhs, cudaStream_t s) {
+    if (prec == BRI_F64 && bri_fx_ready(ctx)) return BRI_OK;  // one shape: every candidate would run the same kernel
     const size_t elt = prec == BRI_F64 ? 16 : 8;
     const size_t bytes = elt * 12 * (size_t)ctx->g.V * nrhs;
     DevBuf inb, outb;

@@ -367,3 +367,20 @@ int main() {
     exe = str(tmp_path / "sum")
     subprocess.run([build_nvcc()] + build.FLAGS + ["-o", exe, str(src)], check=True, capture_output=True, text=True)
     assert float(subprocess.run([exe], check=True, capture_output=True, text=True).stdout) <= 2.0**-44
+
+
+def test_tuning_the_fp64_apply(fake, tmp_path, monkeypatch):
+    """one shape in fixed point: nothing is timed, kept or written; the FP64 kernel,
+    where that one runs, is tuned"""
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("BRI_TUNE_CACHE", str(cache))
+    lib = fake.lib
+    h = fake.op((8, 8, 8, 8))
+    assert lib.bri_tune(h, F64, 1, None) == -8  # BRI_ESTATE: no fields
+    assert fake.build(h) == 0
+    fake.log()
+    assert lib.bri_tune(h, F64, 1, None) == 0
+    assert fake.log() == [] and lib.bri_get_threads(h, F64, 1) == 128 and not cache.exists()
+    _weights(lib, h, [1e-300] * 5, [1e-300] * 5)
+    assert lib.bri_tune(h, F64, 1, None) == 0
+    assert _kind(fake.log()) == {"fp64"} and cache.exists()
