@@ -79,18 +79,6 @@ template <typename T> BRI_HD T cmulc(T a, T b) {
 template <typename T, typename S> BRI_HD T cscale(T a, S s) { T r; r.x = a.x * s; r.y = a.y * s; return r; }
 template <typename T> BRI_HD double cnorm2(T a) { return (double)a.x * a.x + (double)a.y * a.y; }
 
-// sum of FP32 numbers with its rounding errors (Knuth's two-sum), exact to about
-// 2^-47 of the terms for any few of them
-struct SumF32 {
-    float s = 0.f, e = 0.f;
-    BRI_HD void add(float v) {
-        const float t = s + v, z = t - s;
-        e += (s - (t - z)) + (v - z);
-        s = t;
-    }
-    BRI_HD double get() const { return (double)s + (double)e; }
-};
-
 // 3x3 complex matrix, row-major
 template <typename T> struct M3 {
     T e[9];

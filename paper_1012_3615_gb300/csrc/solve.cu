@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "ctx.h"
+#include "sum.cuh"
 
 using namespace bri;
 

@@ -345,7 +345,7 @@ def test_fp32_sums_without_loss(tmp_path):
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
-#include "common.cuh"
+#include "sum.cuh"
 int main() {
     srand(5);
     double worst = 0;
