@@ -61,3 +61,22 @@ def test_flop_count_of_one_apply():
     colour = 80 * 4 * 9 * 8                                  # complex MACs, 8 flops each
     spin = sum(k * 2 * (2 * 24 + 24 + 24 * n) for n, k in pairs.items())  # sum/difference, lambda, gamma
     assert colour + spin + 2 * 24 == bench.IMPL_FLOPS_PER_SITE == 34032
+
+
+def test_counters_of_the_fp64_apply_go_with_its_own_sources(tmp_path, monkeypatch):
+    for f in bench.FP64_SOURCES:
+        dst = tmp_path / f
+        dst.parent.mkdir(parents=True, exist_ok=True)
+        shutil.copy(os.path.join(bench.ROOT, f), dst)
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    (tmp_path / "profiles").mkdir()
+    caps = [{"mode": m, "nrhs": 1, "launch_shape": 128, "lattice": [16, 16, 16, 32], "dram_bytes_per_launch": 1000.0}
+            for m in ("f64-full", "f32-full")]
+    doc = {"kernel_hash": bench.kernel_hash(), "kernel_hash_f64": bench.kernel_hash("f64-full"), "captures": caps}
+    (tmp_path / "profiles" / "dslash_traffic.json").write_text(json.dumps(doc))
+    for m in ("f64-full", "f32-full"):
+        assert bench.measured_traffic(m, 1, 128, [16, 16, 16, 32]) == 1000.0
+    src = tmp_path / "paper_1012_3615_gb300/csrc/dslash_fx.cu"
+    src.write_text(src.read_text() + "\nint changed;\n")
+    assert bench.measured_traffic("f64-full", 1, 128, [16, 16, 16, 32]) is None
+    assert bench.measured_traffic("f32-full", 1, 128, [16, 16, 16, 32]) == 1000.0
