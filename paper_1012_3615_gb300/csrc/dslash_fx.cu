@@ -631,17 +631,18 @@ bri_status bri_fx_reserve(bri_ctx *ctx, cudaStream_t s) {
 
 // the fixed-point apply can be used: its fields are there, and the class weights
 // lie within 2^+-60 or are zero, so that their products with the class scales
-// (2^+-958) stay normal numbers with all their digits.  rho all zero leaves the
-// chiralities apart, which share an exponent (FX_WIDE)
+// (2^+-958) stay normal numbers with all their digits.  A class whose gamma terms
+// are much smaller than its others leaves the chiralities apart, which share an
+// exponent (FX_WIDE)
 bool bri_fx_ready(const bri_ctx *ctx) {
     if (!ctx->have_fx) return false;
-    bool mixes = false;
     for (int n = 1; n <= 4; n++) {
-        for (double w : {std::fabs(ctx->g.lamd[n]), std::fabs(ctx->g.rhod[n])})
+        const double lam = std::fabs(ctx->g.lamd[n]), rho = std::fabs(ctx->g.rhod[n]);
+        for (double w : {lam, rho})
             if (w != 0.0 && !(w >= 0x1p-60 && w <= 0x1p60)) return false;
-        mixes = mixes || ctx->g.rhod[n] != 0.0;
+        if (rho * (double)(1 << FX_WIDE) < lam) return false;
     }
-    return mixes;
+    return true;
 }
 
 // FP64 apply of sites [g.s0, g.s1) in fixed point.  Its work space is stream-ordered

@@ -293,3 +293,26 @@ def test_components_of_different_size(gpu, oracle_weights, what):
         far = np.abs(ref).max(axis=(1, 2)) < 1e-10
         assert far.any()
         assert (np.abs(out - ref)[far] <= 4e-15 * np.abs(ref[far]).max(axis=(1, 2), keepdims=True)).all()
+
+
+@pytest.mark.parametrize("rho2", [0.0, 1e-12])
+def test_class_without_gamma_terms(gpu, oracle_weights, rho2):
+    """the chiralities of a site that is seen through a class without (or with tiny)
+    gamma terms do not mix: what the small one gives keeps its digits"""
+    L = (4, 4, 3, 5)
+    U = synth.random_su3_links(L, 0.3, 30)
+    psi = 1e-14 * synth.gaussian_spinor(L, 1, 31)
+    psi[0, 100, :2] *= 1e14
+    op, W = _op(L, U, gpu)
+    lam, rho = [0, -0.1, -0.05, -0.02, -0.01], [0, 0.1, rho2, 0.02, 0.01]
+    op.set_weights(lam, rho)
+    oracle_weights(lam, rho)
+    out = op.apply(torch.as_tensor(psi, device=gpu), m0=0.0).cpu().numpy()[0]
+    ref = oracle.apply(L, AP, W, 0.0, psi[0])
+    x = synth.coordinates(L)
+    d = np.abs(x - x[100])
+    d = np.minimum(d, np.array(L) - d)
+    seen = (d.max(1) == 1) & (d.sum(1) == 2)  # by a two-hop offset only
+    size = np.abs(ref[:, 2:]).max(axis=(1, 2), keepdims=True)
+    assert seen.sum() == 24 and size[seen].max() < 1e-11
+    assert (np.abs(out - ref)[:, 2:] <= 4e-15 * size)[seen].all()
