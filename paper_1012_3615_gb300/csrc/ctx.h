@@ -85,7 +85,7 @@ cudaError_t bri_malloc_bytes(bri_ctx *ctx, void **p, size_t bytes);
 template <class T> cudaError_t bri_malloc(bri_ctx *ctx, T **p, size_t bytes) {
     return bri_malloc_bytes(ctx, (void **)p, bytes);
 }
-bool bri_give_back(bri_ctx *ctx, int step);
+bool bri_give_back(bri_ctx *ctx, int step, size_t need);
 
 inline bool bri_aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 

@@ -28,7 +28,7 @@
 // 1.02e-16 (1.6e-16) for a field that falls by e^-2 a step in every direction.
 //
 // Measured: 16^3x32 0.736 ms (FP64 kernel 4.12; cross products as integers 0.887),
-// 8^4 47 us (629; 62), 32^4 5.5 ms (31.2; 6.7).  Per pair and warp 144 wide
+// 8^4 45 us (629; 62), 32^4 5.5 ms (31.2; 6.7).  Per pair and warp 144 wide
 // multiply-adds (4 clocks each), 144 packed FMAs (2) and 770 other
 // instructions; latency at 12 warps per SM bounds it (issue 42%, long
 // scoreboard and fixed-latency waits the top stalls).
@@ -565,11 +565,19 @@ bri_status fx_launch(int mode, bri_ctx *ctx, const Geom &g, const int4 *P, const
 
 }  // namespace
 
-// step 0: work space between calls; step 1: the fixed-point copy, unless a graph of
-// the program reads it (the solver's are captured again).  The next build takes
-// the copy back if there is room.  False: nothing was given back
-bool bri_give_back(bri_ctx *ctx, int step) {
-    if (step == 1 && (!ctx->hopsfx || bri_in_program_graph(ctx))) return false;
+// for an allocation of `need` bytes, step 0: work space between calls; step 1: the
+// fixed-point copy, if that is enough and unless a graph of the program reads it
+// (the solver's are captured again).  The next build takes the copy back if there
+// is room.  False: nothing was given back
+bool bri_give_back(bri_ctx *ctx, int step, size_t need) {
+    if (step == 1) {
+        size_t room = 0, total = 0;
+        if (!ctx->hopsfx || bri_in_program_graph(ctx) || cudaMemGetInfo(&room, &total) != cudaSuccess ||
+            room + sizeof(int4) * 9 * NCANON * fx_vp(ctx->g) < need) {
+            cudaGetLastError();
+            return false;
+        }
+    }
     if (cudaDeviceSynchronize() != cudaSuccess) {
         cudaGetLastError();
         return false;
@@ -590,7 +598,7 @@ cudaError_t bri_malloc_bytes(bri_ctx *ctx, void **p, size_t bytes) {
     cudaError_t e = cudaMalloc(p, bytes);
     for (int step = 0; e == cudaErrorMemoryAllocation && step < 2; step++) {
         cudaGetLastError();
-        if (bri_give_back(ctx, step)) e = cudaMalloc(p, bytes);
+        if (bri_give_back(ctx, step, bytes)) e = cudaMalloc(p, bytes);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();  // not for the next launch to report

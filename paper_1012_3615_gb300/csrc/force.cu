@@ -343,7 +343,7 @@ bri_status bri_force_impl(bri_ctx *ctx, double2 *dU, const double2 *chi, const d
     cudaError_t e = cudaMallocFromPoolAsync((void **)&A, bytes, ctx->pool, s);
     for (int step = 0; e == cudaErrorMemoryAllocation && step < 2; step++) {
         cudaGetLastError();
-        if (bri_give_back(ctx, step)) e = cudaMallocFromPoolAsync((void **)&A, bytes, ctx->pool, s);
+        if (bri_give_back(ctx, step, bytes)) e = cudaMallocFromPoolAsync((void **)&A, bytes, ctx->pool, s);
     }
     if (e != cudaSuccess) cudaGetLastError();
     BRI_TRY_CUDA(ctx, e);

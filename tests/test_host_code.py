@@ -264,6 +264,19 @@ def test_fixed_point_copy_stays_for_a_program_graph(fake):
     assert lib.bri_store_hops(h, F32, FULL, None) == 0
 
 
+def test_fixed_point_copy_stays_when_it_would_not_do(fake):
+    lib = fake.lib
+    h = fake.op((8, 8, 8, 8))
+    assert fake.build(h) == 0
+    lib.fake_budget(lib.fake_used() + 4096 * 2000)
+    ev = (ctypes.c_double * 4)()
+    st = lib.bri_eigs_ddag_d(h, ev, None, None, 4, ctypes.c_double(0.1), 2000, ctypes.c_double(1e-8), F64, None, None)
+    assert st == -2  # 2,001 vectors of 192 bytes a site
+    fake.log()
+    assert fake.apply(h) == 0
+    assert _kind(fake.log()) == {"fx"}
+
+
 def test_pool_memory_gives_way_first(fake):
     lib = fake.lib
     h = fake.op((8, 8, 8, 8))
