@@ -43,6 +43,8 @@
  *    hopping fields, its work spaces and its tuning cache, all released by
  *    bri_destroy.  Nothing is retained from caller buffers beyond the call,
  *    except that bri_build_hops keeps a device copy of U (used by the force).
+ *    A captured apply adds kernel nodes only; its work space is held by the
+ *    graph and its copies, the fields that it reads are the context's.
  *  - Streams: `stream` is a cudaStream_t (NULL = legacy default stream).  All
  *    work is enqueued on it; calls return once the work is enqueued, except
  *    where stated (solvers synchronise the stream to read convergence data).

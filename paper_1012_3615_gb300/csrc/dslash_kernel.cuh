@@ -925,12 +925,19 @@ __global__ void __maxnreg__(128) k_dslash_split_r128(int mode, LL ll, const floa
     dslash_split_body<LL, 5, false, S>(mode, ll, in, out, g, diag, skip);
 }
 // Lattices that are summed in parts, and the warps per group for a launch of so
-// many groups.  Measured (us; FP32 full, FP32 2-row, FP16 2-row): 8^4, one
-// right-hand side: one thread a site 31, 35, 34, four warps 12.9; three: 31, 35,
-// 35 -> 18.7; twelve: 55, 56, 58 -> 56, 56, 57.  Above 128 groups the parts cost
-// twelve right-hand sides 3-11% (12^4: 224 -> 249) for a quarter of one's time,
-// so the line lies there; up to 1,600 groups of a launch four warps a site are
-// the faster form of the two, above it one (8^4, 24: 109 against 100 in one part).
+// many groups.  Measured (us in one part -> in parts; FP32 full, FP32 2-row, FP16
+// 2-row):
+//   sites    one right-hand side              three                          twelve
+//   4,096    31, 35, 34 -> 12.7, 12.6, 12.6   31, 35, 35 -> 18.6, 18.5, 18.7   54, 55, 57 -> 55, 55, 56
+//   5,120    31, 35, 35 -> 14.6, 14.6, 14.6   32, 35, 35 -> 25.3, 24.7, 24.6   72, 72, 76 -> 80, 76, 78
+//   8,192    31, 35, 35 -> 14.6, 14.4, 15.0   41, 39, 43 -> 32.8, 32.8, 32.8  100, 101, 106 -> 109, 105, 109
+//  13,824    33, 35, 35 -> 20.5, 19.5, 20.3   55, 57, 57 -> 49, 49, 49        155, 152, 156 -> 171, 160, 162
+//  20,736    41, 40, 44 -> 30.8, 28.8, 29.0   77, 76, 78 -> 86, 80, 80        223, 218, 222 -> 247, 231, 231
+// Up to 128 groups of 32 sites no count loses.  Above, few right-hand sides
+// gain and twelve lose 3-13%, and the form cannot go by the count (equal bits
+// alone and in a batch), so the line lies there.  Up to 1,600 groups of a launch
+// four warps a site are the faster of the two forms in parts, above it one (8^4, 24:
+// 109 against 100 in one part).  An x extent of 32 keeps the line kernel.
 inline bool dslash_in_parts(int V) { return V <= 128 * 32; }
 inline int dslash_splits(long long groups) { return groups <= 1600 ? 4 : 1; }
 

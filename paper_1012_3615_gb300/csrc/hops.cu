@@ -35,8 +35,8 @@ namespace {
 // cross products stay below 2 sqrt(6) 2^60 < 2^63 and those of its high
 // products, over the n terms of a level, below n sqrt(6) 2^58.  A level's sum
 // is scaled by 2^-1, 2^-2, 2^-2 (n = 2, 3, 4) instead of 1/n.  Known to 2^-57.
-// 16^3x32: 0.90 ms (FP64 products: 2.7), the whole build 5.1 ms (7.7), of which
-// the projection takes 3.7.
+// 16^3x32: 0.90 ms (FP64 products: 2.7), the whole build 4.45 ms, of which the
+// projection takes 3.1 (project_fx.cuh).
 // Links that are not unitary to 2^-16 (only their user knows what they are)
 // take the FP64 form; every kernel takes the same branch.  Norms alone would not
 // do: products of matrices with rows and columns of norm 1 grow to 1.73^n.

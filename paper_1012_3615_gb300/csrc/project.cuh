@@ -295,8 +295,8 @@ static __device__ __noinline__ void project_su3_general(const M3<double2> &A, M3
 // FP64 and L inverted in the FP32 basis (L as in the derivative, force.cu): an
 // error falls by the FP32 accuracy of L per step, 1e-6, 1e-12, 1e-18.  About
 // 400 FP64 operations, which still bound it: 262,144 averages of six links
-// exp(i 0.5 H) in 209 us instead of 3,080, the hopping fields of 16^3x32 in
-// 10.1 ms instead of 52.4; the stationarity R comes out at 2e-17 |A| on
+// exp(i 0.5 H) in 209 us instead of 3,080, the hopping fields of 16^3x32
+// (path sums in FP64 then, see project_fx.cuh) in 10.1 ms instead of 52.4; the stationarity R comes out at 2e-17 |A| on
 // average instead of 1e-16.  What FP32 does not settle (an exponent far from 1,
 // branch B or near it, a small h, slow or no convergence, infinities and NaN)
 // takes the general form.
